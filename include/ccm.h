@@ -246,15 +246,16 @@ int ccm_apply(ccm_handle* h, const double* u, const double* g, double* out, int 
  * device.  The handle is set up beforehand, and its device must be the current device
  * (CCM_EINVAL otherwise, before any work is queued).  Unlike ccm_apply, this call does not use
  * the handle's work arrays.  It uses a fixed file-scope device array (the library keeps
- * CCM_NOALLOC_SCRATCH_BYTES = 16 MiB on every device that loads it, until the process exits).
+ * CCM_NOALLOC_SCRATCH_BYTES = 16 MiB on every device that loads it, until the process exits),
+ * and touches it only where out overlaps u or g (else u and out are all it reads and writes).
  * That array holds two padded FP64 grids of at most CCM_NOALLOC_MAX_PADDED cells each, where
  * the padded size is ((nx + 4) rounded up to a multiple of 32) * (ny + 4); larger grids are
  * rejected with CCM_ETOOLARGE before any work is queued.  It calls no cudaMalloc, cudaFree or
  * allocating library routine.  The first call on a device looks up the array's device address
- * (once per device), so make that first call before any stream capture.  Every call shares
- * the array, so calls that overlap on the GPU (other streams, other handles) race; the call
- * clears the part of the array it uses before filling it.  The paper has no counterpart of
- * this entry point: it exists for the memory model of its callers. */
+ * (once per device), so make that first call before any stream capture.  Every call whose out
+ * overlaps u or g shares the array, so such calls race where they overlap on the GPU (other
+ * streams, other handles).  The paper has no counterpart of this entry point: it exists for
+ * the memory model of its callers. */
 #define CCM_NOALLOC_MAX_PADDED (1L << 20)
 #define CCM_NOALLOC_SCRATCH_BYTES (2L * CCM_NOALLOC_MAX_PADDED * 8L)
 int ccm_apply_noalloc(const ccm_handle* h, const double* u, const double* g, double* out, void* stream);

@@ -1,0 +1,147 @@
+// The operator and its transpose on whole arrays (ccm_apply, ccm_apply_T, ccm_level_apply).
+//
+// One launch covers the box's 64 x 32 tiles and, in CTAs ahead of them, the fitted rows (or the
+// boundary part of the transpose), for all vectors (grid y).  The arrays are read and written
+// in the caller's layout, with the empty cells masked by their class (their values are never
+// used), so that nothing is packed into the padded layout and back: what is left is one read of
+// the vector's active cells and one write of the whole result.  The regular stencil runs in
+// integer form (fixed.cuh).
+#pragma once
+
+#include "smooth.cuh"
+
+namespace ccm {
+namespace dev {
+
+// a cell array: value (i, j) of vector z at p[z batch + j stride + i]
+template <typename P>
+struct Grid {
+  P p;
+  long stride, batch;
+};
+
+struct ApplyArgs {
+  Grid<const double*> u;
+  Grid<double*> out;
+  const uint8_t* cls;        // padded
+  int nx, ny, pitch, tx;     // tx: tiles per row of the box
+  int nrow;                  // CTAs [0, nrow): 256 fitted rows each
+  int n2, W;
+  const int32_t* cell;       // padded
+  const int32_t* col;        // padded
+  const double* val;
+  const double* nb;
+  const int32_t* seg;
+  const double* g;           // forward: boundary data, or null
+  double* og;                // transpose: N^T v, or null
+  long nseg;
+  double scale;              // 1 / h^2
+  bool vec;                  // out rows start on 16 bytes
+  Stencil<double> S;
+  QStencil Q;
+};
+
+// the offset of padded cell p in a cell array
+__device__ __forceinline__ long cell_at(int p, int pitch, long stride) {
+  const int j = (int)((unsigned)p / (unsigned)pitch), i = p - j * pitch;
+  return (j - 2) * stride + (i - 2);
+}
+
+// out = L u + N g (TRANS: the regular cells' part of L^T v on every non-empty cell, and N^T v).
+// Bound by memory at large sizes: star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134
+// MB written.
+template <bool CROSS, bool TRANS>
+__global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
+  __shared__ __align__(16) double tile[HY * HX];
+  __shared__ __align__(16) unsigned wmax[8];
+  const int z = blockIdx.y;
+  pdl_enter();
+  const double* __restrict__ u = A.u.p + z * A.u.batch;
+  double* __restrict__ out = TRANS && !A.out.p ? nullptr : A.out.p + z * A.out.batch;
+  if ((int)blockIdx.x < A.nrow) {
+    const int row = blockIdx.x * 256 + threadIdx.x;
+    if (row >= A.n2) return;
+    const int c = A.cell[row];
+    if (TRANS) {
+      const int sg = A.seg[row];
+      if (sg >= 0) A.og[z * A.nseg + sg] = A.scale * A.nb[row] * u[cell_at(c, A.pitch, A.u.stride)];
+      return;
+    }
+    double acc = 0.0;
+#pragma unroll 15
+    for (int k = 0; k < A.W; ++k)
+      acc += A.val[(long)k * A.n2 + row] * u[cell_at(A.col[(long)k * A.n2 + row], A.pitch, A.u.stride)];
+    if (A.g != nullptr && A.seg[row] >= 0) acc += A.nb[row] * A.g[z * A.nseg + A.seg[row]];
+    out[cell_at(c, A.pitch, A.out.stride)] = A.scale * acc;
+    return;
+  }
+  const int t = blockIdx.x - A.nrow;
+  const int cx0 = (t % A.tx) * JX, cy0 = (t / A.tx) * JY;
+  // classes of the staged slots (threadIdx.x + 256 k of the 68 x 36 tile with its halo)
+  constexpr int N = (HY * HX + 255) / 256;
+  bool on[N];
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const int idx = threadIdx.x + 256 * k, y = idx / HX, x = idx - y * HX;
+    const int i = cx0 + x - 2, j = cy0 + y - 2;
+    const bool in = idx < HY * HX && (unsigned)i < (unsigned)A.nx && (unsigned)j < (unsigned)A.ny;
+    const uint8_t c = in ? A.cls[(long)(j + 2) * A.pitch + i + 2] : (uint8_t)0;
+    on[k] = TRANS ? c == 1 : c != 0;
+    any |= c != 0;
+  }
+  const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
+  const int i0 = cx0 + x0;
+  auto put = [&](int kk, double s0, double s1, uint32_t c2) {
+    const int j = cy0 + y0 + kk;
+    if (j >= A.ny || i0 >= A.nx) return;
+    // forward: the fitted rows' cells are written by their own CTAs
+    const bool g0 = TRANS || (c2 & 0xffu) != 2u, g1 = (TRANS || (c2 >> 8) != 2u) && i0 + 1 < A.nx;
+    const double v0 = (c2 & 0xffu) ? A.scale * s0 : 0.0, v1 = (c2 >> 8) ? A.scale * s1 : 0.0;
+    double* o = out + (long)j * A.out.stride + i0;
+    if (A.vec && g0 && g1) {
+      *reinterpret_cast<double2*>(o) = make_double2(v0, v1);
+    } else {
+      if (g0) o[0] = v0;
+      if (g1) o[1] = v1;
+    }
+  };
+  if (!__syncthreads_or(any)) {
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) put(kk, 0.0, 0.0, 0u);
+    return;
+  }
+  uint32_t c2[4];
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk) {
+    const int j = cy0 + y0 + kk;
+    c2[kk] = (i0 < A.nx && j < A.ny) ? *reinterpret_cast<const uint16_t*>(A.cls + (long)(j + 2) * A.pitch + i0 + 2) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const int idx = threadIdx.x + 256 * k, y = idx / HX, x = idx - y * HX;
+    if (idx < HY * HX) tile[idx] = on[k] ? u[(cy0 + y - 2) * A.u.stride + (cx0 + x - 2)] : 0.0;
+  }
+  // each thread reads back its own slots first (tile_stencil64's maximum), so no barrier here
+  tile_stencil64<CROSS>(tile, wmax, x0, y0, true, A.S, A.Q, [&](int kk, double s0, double s1) {
+    put(kk, s0, s1, kk == 0 ? c2[0] : kk == 1 ? c2[1] : kk == 2 ? c2[2] : c2[3]);
+  });
+}
+
+// out += the fitted rows' part of L^T v, by the transposed CSR (one thread per column cell; the
+// entry's row is given by its cell)
+__global__ void k_rows_T(int ncol, const int32_t* __restrict__ ptr, const int32_t* __restrict__ ccell,
+                         const int32_t* __restrict__ rcell, const double* __restrict__ val, Grid<const double*> v,
+                         Grid<double*> out, int pitch, double scale) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int e0 = k < ncol ? ptr[k] : 0, e1 = k < ncol ? ptr[k + 1] : 0;
+  pdl_enter();
+  if (k >= ncol) return;
+  const double* vz = v.p + blockIdx.y * v.batch;
+  double acc = 0;
+  for (int e = e0; e < e1; ++e) acc += val[e] * vz[cell_at(rcell[e], pitch, v.stride)];
+  out.p[blockIdx.y * out.batch + cell_at(ccell[k], pitch, out.stride)] += scale * acc;
+}
+
+}  // namespace dev
+}  // namespace ccm

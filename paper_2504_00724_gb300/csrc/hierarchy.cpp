@@ -352,7 +352,7 @@ int build_smo2_blocks(HostLevel& L, int block, int overlap, int nthreads, std::s
     L.blk[4 * bk + 2] = es;
     L.blk[4 * bk + 3] = ee;
     L.blk_off[bk] = off;
-    off += (long)(ee - es) * (ce - cs);
+    off += ((long)(ee - es) * (ce - cs) + 3) & ~3L;   // every block on 16 bytes in FP32 too (bulk copies)
   }
   L.blk_inv.assign(off, 0.0);
   // the padded cell of every row, to look up the L22 entries

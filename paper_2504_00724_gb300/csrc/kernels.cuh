@@ -11,6 +11,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "fixed.cuh"
+
 namespace ccm {
 namespace dev {
 
@@ -293,6 +295,7 @@ struct SweepArgs {
   const T* u_old;
   T* u_new;
   Stencil<T> S;
+  QStencil Q;                // the stencil in integer form (FP64 tiles of the persistent sweep)
   const int32_t* blk;
   const int64_t* blk_off;
   const T* inv;
@@ -1057,46 +1060,6 @@ __global__ void k_to_float(long n, const double* __restrict__ a, float* __restri
   pdl_enter();
   for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < n; p += (long)gridDim.x * blockDim.x)
     b[p] = (float)a[p];
-}
-
-// transposed operator, scatter-free: out[c] = sum_d w_d v[c + d] [c + d regular]
-// (the regular stencil is point-symmetric) for every non-empty c ...
-template <bool CROSS>
-__global__ void k_regular_T(const int32_t* __restrict__ tiles, const uint8_t* __restrict__ cls, int nx, int ny,
-                            int pitch, const double* __restrict__ v, double* __restrict__ out, Stencil<double> S) {
-  int i, j;
-  long p;
-  if (!tile_cell(tiles, nx, ny, pitch, i, j, p)) return;
-  if (cls[p] == 0) return;
-  double acc = 0;
-#pragma unroll
-  for (int dj = -2; dj <= 2; ++dj)
-#pragma unroll
-    for (int di = -2; di <= 2; ++di) {
-      double w = S.w[(dj + 2) * 5 + di + 2];
-      if (!CROSS && dj != 0 && di != 0) continue;
-      long q = p + (long)dj * pitch + di;
-      if (cls[q] == 1) acc += w * v[q];
-    }
-  out[p] = acc;
-}
-// ... plus the fitted rows through the transposed CSR (one thread per column cell)
-__global__ void k_rows_T(int ncol, const int32_t* __restrict__ ptr, const int32_t* __restrict__ ccell,
-                         const int32_t* __restrict__ row, const double* __restrict__ val,
-                         const int32_t* __restrict__ rcell, const double* __restrict__ v, double* __restrict__ out) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= ncol) return;
-  double acc = 0;
-  for (int e = ptr[k]; e < ptr[k + 1]; ++e) acc += val[e] * v[rcell[row[e]]];
-  out[ccell[k]] += acc;
-}
-// N^T v: one entry per segment (each segment belongs to exactly one fitted row)
-__global__ void k_bnd_T(int n2, const int32_t* __restrict__ cell, const double* __restrict__ nb,
-                        const int32_t* __restrict__ seg, const double* __restrict__ v, double* __restrict__ og,
-                        double scale) {
-  int row = blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= n2 || seg[row] < 0) return;
-  og[seg[row]] = scale * nb[row] * v[cell[row]];
 }
 
 }  // namespace dev

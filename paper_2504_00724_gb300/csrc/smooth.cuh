@@ -9,8 +9,9 @@
 //   tile item:  the 68 x 36 halo tile of u, the 68 x 32 box of r over the tile's rows and the
 //               80 x 36 class bytes (one 2-D TMA box each; x origin 64a, 16-byte aligned),
 //               and with PRO the 36 x 18 box of the coarse iterate under the tile;
-//   block item: the block's rows of inv(L22[ext, ext]) by one bulk copy (cp.async.bulk); the
-//               residuals of its extended rows are gathered from global memory meanwhile.
+//   block item: the block's rows of inv(L22[ext, ext]) by one bulk copy (cp.async.bulk; in FP64
+//               two copies of half the rows each, in consecutive stages); the residuals of its
+//               extended rows are gathered from global memory meanwhile.
 // With PRO the sweep is the first post-smoothing sweep of Alg. 2 and reads u + P uc, the
 // coarse correction added to regular cells only (Sec. 4.1).  A level's first sweep may start
 // from a zero iterate (zero_u: no iterate copied or gathered), and the last level-0 sweep of
@@ -26,6 +27,14 @@
 
 namespace ccm {
 namespace dev {
+
+// stages that one block item takes: its inverse rows whole in FP32; half of them at a time in
+// FP64, where the whole (57 KB at 64 core and 112 extended rows) would make a stage so large
+// that one CTA per SM is resident instead of two
+template <typename T>
+constexpr int BLOCK_PARTS = sizeof(T) == 8 ? 2 : 1;
+// extended rows of the first part (even: the second part's copy starts on 16 bytes)
+__host__ __device__ constexpr int block_split(int ne) { return (ne / 2 + 1) & ~1; }
 
 template <typename T>
 struct SmoothArgs {
@@ -78,13 +87,14 @@ __device__ __forceinline__ bool wait_parity(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// The copy of an item into stage st, completing on bar.  part 0: all of it; part 1: what
+// The copy of an item (of the given half of a block's rows where BLOCK_PARTS is 2) into stage
+// st, completing on bar.  part 0: all of it; part 1: what
 // does not depend on the previous launch (a block's inverse rows; a tile's class bytes, with
 // the byte count of the whole tile), issued before the grid dependency wait; part 2: the rest
 // of a tile (iterate, right-hand side, coarse iterate), after it.
 template <typename T, bool PRO>
 __device__ __forceinline__ void smooth_issue(const SmoothArgs<T>& A, const CUtensorMap* tin, const CUtensorMap* tr,
-                                             const CUtensorMap* tcls, const CUtensorMap* tuc, int item,
+                                             const CUtensorMap* tcls, const CUtensorMap* tuc, int item, int half,
                                              unsigned char* st, uint64_t* bar, int part = 0) {
   const int z = blockIdx.y;      // right-hand side of the batch
   const SweepArgs<T>& a = A.a;
@@ -92,14 +102,16 @@ __device__ __forceinline__ void smooth_issue(const SmoothArgs<T>& A, const CUten
     if (part == 2) return;
     const int b = item;
     const int nc = a.blk[4 * b + 1] - a.blk[4 * b], ne = a.blk[4 * b + 3] - a.blk[4 * b + 2];
-    const uint32_t abytes = (uint32_t)(((long)ne * nc * sizeof(T) + 15) & ~15L);
+    const int e0 = BLOCK_PARTS<T> == 2 && half ? block_split(ne) : 0;
+    const int e1 = BLOCK_PARTS<T> == 2 && !half ? block_split(ne) : ne;
+    const uint32_t abytes = (uint32_t)(((long)(e1 - e0) * nc * sizeof(T) + 15) & ~15L);
     mbar_expect_tx(bar, abytes);
-    bulk_load(st, a.inv + a.blk_off[b], abytes, bar);
+    if (abytes) bulk_load(st, a.inv + a.blk_off[b] + (long)e0 * nc, abytes, bar);   // (a block of 1 or 2 rows: an empty half)
   } else {
     using S = TileStage<T>;
     const int t = item - A.nbi;
     const int cx0 = a.tiles[2 * t] * JX, cy0 = a.tiles[2 * t + 1] * JY;
-    const bool no_u = !PRO && sizeof(T) == 4 && a.zero_u;     // the old iterate is 0
+    const bool no_u = !PRO && a.zero_u;     // the old iterate is 0
     if (part != 2) {
       mbar_expect_tx(bar, (no_u ? 0u : S::u_bytes) + S::r_bytes + S::c_bytes + (PRO ? S::uc_bytes : 0));
       tma_load_2d(st + S::c_off, tcls, bar, cx0, cy0);
@@ -128,7 +140,7 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
   for (int e = threadIdx.x; e < ne; e += blockDim.x) {
     const int row = es + e;
     const int q = a.cell[row];
-    if (!PRO && sizeof(T) == 4 && a.zero_u) {   // the old iterate is 0: the residual is r
+    if (!PRO && a.zero_u) {   // the old iterate is 0: the residual is r
       sres[e] = rhs[q];
       sold[e] = (T)0;
       scell[e] = q;
@@ -179,12 +191,87 @@ __device__ __forceinline__ void block_apply(const T* As, const T* sres, const T*
   }
 }
 
+// FP64: the product of one part of the block's inverse rows with the residuals, one core
+// column per thread and 256 / (64 or 128) groups of extended rows, added to acc; after the last
+// part the groups' sums and the core cells' update as in block_apply.  FP64 issue bounds it (112
+// x 64 FMA at two a clock are 1.7 us), so the columns spread over as many warps as there are
+// for the final sums too.
+__device__ __forceinline__ void block_apply_part(const double* As, const double* sres, const double* sold,
+                                                 const int* scell, int c0, int nc, int e0, int e1, bool last, double& acc,
+                                                 double* __restrict__ u_new, double* part) {
+  const int ncp = nc > 64 ? 128 : 64, ng = 256 / ncp;
+  const int c = threadIdx.x & (ncp - 1), g = threadIdx.x / ncp;
+  if (c < nc)
+    for (int e = e0 + g; e < e1; e += ng) acc += As[(e - e0) * nc + c] * sres[e];
+  if (!last) return;
+  part[threadIdx.x] = acc;
+  acc = 0;
+  __syncthreads();
+  if (g == 0 && c < nc) {
+    double tot = part[c];
+    for (int w = 1; w < ng; ++w) tot += part[w * ncp + c];
+    u_new[scell[c0 + c]] = sold[c0 + c] + tot;
+  }
+}
+
+// FP64 sum of the stencil on a staged tile in factored form (the x-derivative of each entering
+// row and 13 FMA per cell): the tiles that the integer form does not take
+template <bool CROSS, class Emit>
+__device__ __forceinline__ void fp64_rows(const double* __restrict__ tile, int x0, int y0, const Stencil<double>& S,
+                                          Emit emit) {
+#pragma unroll 1
+  for (int k = 0; k < 4; ++k) {
+    double s[2];
+#pragma unroll 1
+    for (int j = 0; j < 2; ++j) {
+      const double* c = tile + (y0 + k + 2) * HX + x0 + j + 2;
+      double acc = S.cc * c[0];
+      acc = fma(S.lx[0], c[-2], acc);
+      acc = fma(S.lx[1], c[-1], acc);
+      acc = fma(S.lx[3], c[1], acc);
+      acc = fma(S.lx[4], c[2], acc);
+      acc = fma(S.ly[0], c[-2 * HX], acc);
+      acc = fma(S.ly[1], c[-HX], acc);
+      acc = fma(S.ly[3], c[HX], acc);
+      acc = fma(S.ly[4], c[2 * HX], acc);
+      if (CROSS)
+        for (int dj = 0; dj < 5; ++dj) {
+          const double* r = c + (dj - 2) * HX;
+          if (dj != 2) acc = fma(S.gy[dj], S.gx[0] * r[-2] + S.gx[1] * r[-1] + S.gx[3] * r[1] + S.gx[4] * r[2], acc);
+        }
+      s[j] = acc;
+    }
+    emit(k, s[0], s[1]);
+  }
+}
+
+// h^2 L u at the cells (x0, y0 + k) and (x0 + 1, y0 + k), k = 0 .. 3, of a staged tile of doubles
+// for all 256 threads of a CTA (x0, y0: two columns and four rows a thread): in integer form,
+// the tile's values replaced by their integers in place, or as an FP64 sum where that does not
+// apply (see fixed.cuh).  emit(k, Lu0, Lu1) only where on.  Barriers inside; a thread that needs
+// the tile's own values reads them before the call.
+template <bool CROSS, class Emit>
+__device__ __forceinline__ void tile_stencil64(double* tile, unsigned* wmax, int x0, int y0, bool on,
+                                               const Stencil<double>& S, const QStencil& Q, Emit emit) {
+  QSlots<(HY * HX + 255) / 256> v;
+  const int E = q_scale(q_cta_max(v.load(tile, HY * HX), wmax), Q);
+  if (E < 0) {
+    if (on) fp64_rows<CROSS>(tile, x0, y0, S, emit);
+    return;
+  }
+  long long* q = reinterpret_cast<long long*>(tile);
+  v.store(q, HY * HX, E);
+  __syncthreads();
+  const int e = E - 1022 + Q.cexp;
+  if (on) q_rows<CROSS, HX>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
+}
+
 // SMO-1 on the regular cells of a staged 64 x 32 tile (halo box of u, box of r and class bytes
 // at the TileStage offsets of st; with PRO the coarse box too, whose parent values are first
 // added to the staged regular cells: the sweep then reads u + P uc)
 template <typename T, bool CROSS, bool PRO>
 __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char* st, int cx0, int cy0,
-                                           T* __restrict__ u_new, double* __restrict__ uhat) {
+                                           T* __restrict__ u_new, double* __restrict__ uhat, unsigned* wmax) {
   using S = TileStage<T>;
   T* tile = reinterpret_cast<T*>(st);
   const T* rt = reinterpret_cast<const T*>(st + S::r_off);
@@ -211,60 +298,39 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
     __syncthreads();
   }
   if constexpr (sizeof(T) == 8) {
-    // FP64: one cell column of eight rows per thread (the paired form below spills).  FP64
-    // issue bounds this loop, so with the mixed term the stencil is taken in factored form: the
-    // x-derivative of each entering row (4 FMA) and 13 FMA per cell, against 25
-    const int x = threadIdx.x & 63, y0 = (threadIdx.x >> 6) * 8;
-    const int i = cx0 + x;
-    if (i < a.nx) {
-      T w[5][5], D[5];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int b = 0; b < 5; ++b) w[q][b] = tile[(y0 + q) * HX + x + b];
-        if (CROSS) D[q] = a.S.gx[0] * w[q][0] + a.S.gx[1] * w[q][1] + a.S.gx[3] * w[q][3] + a.S.gx[4] * w[q][4];
+    // FP64: the same two columns and four rows per thread as below; the stencil in integer form
+    // (FP64 issue would bound it: 19 operations a cell, 9.4 us a tile)
+    using V2 = double2;
+    const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
+    const int i0 = cx0 + x0;
+    auto put = [&](int kk, double v0, double v1) {
+      const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y0 + kk + 2) * CLX + x0 + 2);
+      const bool g0 = (c2 & 0xffu) == 1u, g1 = (c2 >> 8) == 1u && i0 + 1 < a.nx;
+      const long p = (long)(cy0 + y0 + kk + 2) * a.pitch + (i0 + 2);
+      if (g0 && g1) {
+        *reinterpret_cast<V2*>(u_new + p) = make_double2(v0, v1);
+      } else {
+        if (g0) u_new[p] = v0;
+        if (g1) u_new[p + 1] = v1;
       }
+    };
+    if (!PRO && a.zero_u) {
+      if (i0 < a.nx)
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-        for (int b = 0; b < 5; ++b) w[4][b] = tile[(y0 + kk + 4) * HX + x + b];
-        if (CROSS) D[4] = a.S.gx[0] * w[4][0] + a.S.gx[1] * w[4][1] + a.S.gx[3] * w[4][3] + a.S.gx[4] * w[4][4];
-        if (ct[(y0 + kk + 2) * CLX + x + 2] == 1) {
-          T acc = 0;
-          if (CROSS) {
-            acc = a.S.cc * w[2][2];
-            acc = fma(a.S.lx[0], w[2][0], acc);
-            acc = fma(a.S.lx[1], w[2][1], acc);
-            acc = fma(a.S.lx[3], w[2][3], acc);
-            acc = fma(a.S.lx[4], w[2][4], acc);
-            acc = fma(a.S.ly[0], w[0][2], acc);
-            acc = fma(a.S.ly[1], w[1][2], acc);
-            acc = fma(a.S.ly[3], w[3][2], acc);
-            acc = fma(a.S.ly[4], w[4][2], acc);
-            acc = fma(a.S.gy[0], D[0], acc);
-            acc = fma(a.S.gy[1], D[1], acc);
-            acc = fma(a.S.gy[3], D[3], acc);
-            acc = fma(a.S.gy[4], D[4], acc);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 5; ++q)
-#pragma unroll
-              for (int b = 0; b < 5; ++b) {
-                if (q != 2 && b != 2) continue;
-                acc += a.S.w[q * 5 + b] * w[q][b];
-              }
-          }
-          const long p = (long)(cy0 + y0 + kk + 2) * a.pitch + (i + 2);
-          u_new[p] = w[2][2] + a.S.omega_d * (rt[(y0 + kk) * HX + x + 2] - acc);
+        for (int kk = 0; kk < 4; ++kk) {
+          const V2 r2 = *reinterpret_cast<const V2*>(rt + (y0 + kk) * HX + x0 + 2);
+          put(kk, a.S.omega_d * r2.x, a.S.omega_d * r2.y);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-          for (int b = 0; b < 5; ++b) w[q][b] = w[q + 1][b];
-          if (CROSS) D[q] = D[q + 1];
-        }
-      }
+      return;
     }
+    V2 c[4];
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) c[kk] = *reinterpret_cast<const V2*>(tile + (y0 + kk + 2) * HX + x0 + 2);
+    tile_stencil64<CROSS>(tile, wmax, x0, y0, i0 < a.nx, a.S, a.Q, [&](int kk, double s0, double s1) {
+      const V2 r2 = *reinterpret_cast<const V2*>(rt + (y0 + kk) * HX + x0 + 2);
+      const V2 u = kk == 0 ? c[0] : kk == 1 ? c[1] : kk == 2 ? c[2] : c[3];
+      put(kk, u.x + a.S.omega_d * (r2.x - s0), u.y + a.S.omega_d * (r2.y - s1));
+    });
   } else {
     // FP32: two adjacent cells (x0, x0 + 1) in four rows per thread: each staged row is read
     // as three aligned pairs (x0 - 2 .. x0 + 3) and serves both cells' stencils, and the
@@ -331,13 +397,14 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
 }
 
 template <typename T, bool CROSS, bool PRO>
-__global__ void __launch_bounds__(256, 3) k_smooth(const __grid_constant__ CUtensorMap tin,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __grid_constant__ CUtensorMap tin,
                                                 const __grid_constant__ CUtensorMap tr,
                                                 const __grid_constant__ CUtensorMap tcls,
                                                 const __grid_constant__ CUtensorMap tuc, SmoothArgs<T> A) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ T part[8][32];
+  __shared__ __align__(16) unsigned wmax[8];
   const SweepArgs<T>& a = A.a;
   // While the previous launch drains: pull the static fitted-row data (columns, coefficients,
   // cells, parents) of this CTA's SMO-2 block items into L1, so that each block's residual
@@ -358,13 +425,19 @@ __global__ void __launch_bounds__(256, 3) k_smooth(const __grid_constant__ CUten
   }
   const int G = gridDim.x;
   const int K = (A.nitems - (int)blockIdx.x + G - 1) / G;   // items of this CTA (>= 1)
+  // its block items come first and take BLOCK_PARTS steps of the ring each: NB block steps in
+  // all, K steps with the tiles'
+  constexpr int BP = BLOCK_PARTS<T>;
+  const int kb = (int)blockIdx.x < A.nbi ? (A.nbi - 1 - (int)blockIdx.x) / G + 1 : 0;
+  const int NB = BP * kb, KS = K + (BP - 1) * kb;
+  auto item_of = [&](int k) { return (int)blockIdx.x + (k < NB ? k / BP : k - NB + kb) * G; };
   // also before the wait: the copy barriers, and the parts of the first two items' copies
   // that no earlier launch writes (the rest follows the wait)
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
-    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, blockIdx.x, smem_raw, &bar[0], 1);
-    if (K > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, blockIdx.x + G, smem_raw + A.stage, &bar[1], 1);
+    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(0), 0, smem_raw, &bar[0], 1);
+    if (KS > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(1), 1, smem_raw + A.stage, &bar[1], 1);
   }
   __syncthreads();
   pdl_enter();
@@ -381,16 +454,18 @@ __global__ void __launch_bounds__(256, 3) k_smooth(const __grid_constant__ CUten
   T* sold = reinterpret_cast<T*>(smem_raw + 2 * A.stage + slot);
   int* scell = reinterpret_cast<int*>(smem_raw + 2 * A.stage + 2 * slot);
   if (threadIdx.x == 0) {
-    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, blockIdx.x, smem_raw, &bar[0], 2);
-    if (K > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, blockIdx.x + G, smem_raw + A.stage, &bar[1], 2);
+    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(0), 0, smem_raw, &bar[0], 2);
+    if (KS > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(1), 1, smem_raw + A.stage, &bar[1], 2);
   }
-  for (int k = 0; k < K; ++k) {
-    const int item = blockIdx.x + k * G;
+  T acc = 0;                     // BP == 2: a block's product, carried from its first half to its second
+  int cs = 0, nc = 0, ne = 0, es = 0;
+  for (int k = 0; k < KS; ++k) {
+    const int item = item_of(k), half = k % BP;      // half: of a block item
     const int sb = k & 1;
     const uint32_t parity = (k >> 1) & 1;
-    int cs = 0, nc = 0, ne = 0, es = 0, cx0 = 0, cy0 = 0;
+    int cx0 = 0, cy0 = 0;
     if (item < A.nbi) {
-      block_residuals<T, PRO, false>(a, item, u_old, rhs, ucs, sres, sold, scell, cs, nc, ne, es);
+      if (half == 0) block_residuals<T, PRO, false>(a, item, u_old, rhs, ucs, sres, sold, scell, cs, nc, ne, es);
     } else {
       const int t = item - A.nbi;       // the tile's origin, read before the wait
       cx0 = a.tiles[2 * t] * JX;
@@ -400,20 +475,25 @@ __global__ void __launch_bounds__(256, 3) k_smooth(const __grid_constant__ CUten
     if (!ok) {
       // this copy and the other stage's (if one was issued) must land before the CTA leaves
       wait_parity(&bar[sb], parity);
-      if (k + 1 < K) wait_parity(&bar[sb ^ 1], ((k + 1) >> 1) & 1);
+      if (k + 1 < KS) wait_parity(&bar[sb ^ 1], ((k + 1) >> 1) & 1);
       if (threadIdx.x == 0) atomicExch(a.err, 1);
       return;
     }
     if (item < A.nbi) {
-      block_apply<T>(reinterpret_cast<const T*>(smem_raw + sb * A.stage), sres, sold, scell, cs - es, nc, ne, u_new,
-                     uhat, part);
+      const T* As = reinterpret_cast<const T*>(smem_raw + sb * A.stage);
+      if constexpr (BP == 2) {
+        const int e0 = half ? block_split(ne) : 0, e1 = half ? ne : block_split(ne);
+        block_apply_part(As, sres, sold, scell, cs - es, nc, e0, e1, half == 1, acc, u_new, &part[0][0]);
+      } else {
+        block_apply<T>(As, sres, sold, scell, cs - es, nc, ne, u_new, uhat, part);
+      }
     } else {
-      tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, u_new, uhat);
+      tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, u_new, uhat, wmax);
     }
     __syncthreads();      // stage sb is free
-    if (threadIdx.x == 0 && k + 2 < K) {
+    if (threadIdx.x == 0 && k + 2 < KS) {
       fence_proxy_async();
-      smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item + 2 * G, (smem_raw + sb * A.stage), &bar[sb]);
+      smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(k + 2), k % BP, smem_raw + sb * A.stage, &bar[sb]);
     }
   }
 }
@@ -426,9 +506,11 @@ namespace dev {
 
 // ---- residual + restriction of a level (Alg. 2: the coarse right-hand side and a zero coarse
 // iterate) as one persistent launch over the fine 64 x 32 tiles that restriction visits.
-// A tile item's halo tile of u, its boxes of r and of the cell volumes (68 x 32 over the
+// A tile item's halo tile of u, its boxes of r and (FP32) of the cell volumes (68 x 32 over the
 // tile's rows) and its class bytes (80 x 36) arrive by TMA in one of two stages while the
-// previous item computes.  The fitted rows of the tile's irregular cells (listed per tile:
+// previous item computes.  In FP64 each thread loads the volumes of its coarse cells' children
+// into registers before the wait instead: without their box two CTAs per SM are resident, not
+// one.  The fitted rows of the tile's irregular cells (listed per tile:
 // row and position) are gathered from global memory before the wait, and so are the class
 // bytes of the coarse cells the thread restricts to; regular cells take the stencil from the
 // staged tile; then the 32 x 16 coarse cells get the volume-weighted 2 x 2 sums.
@@ -448,7 +530,9 @@ struct RestrictArgs {
   const uint8_t* clsc;
   T* rc;
   T* uc;
+  const T* vol;        // fine cell volumes
   Stencil<T> S;
+  QStencil Q;
   int* err;
   uint32_t stage;
   long bs, bsc;        // batch strides (elements) of the fine and the coarse level arrays
@@ -466,9 +550,10 @@ struct RestrictStage {
   static constexpr uint32_t c_bytes = HY * CLX;
   static constexpr uint32_t r_off = al(u_bytes);
   static constexpr uint32_t c_off = r_off + al(r_bytes);
+  static constexpr bool vbox = sizeof(T) == 4;     // the volumes arrive by TMA too
   static constexpr uint32_t v_off = c_off + al(c_bytes);
-  static constexpr uint32_t bytes = al(v_off + r_bytes);
-  static constexpr uint32_t tx = u_bytes + 2 * r_bytes + c_bytes;
+  static constexpr uint32_t bytes = al(v_off + (vbox ? r_bytes : 0));
+  static constexpr uint32_t tx = u_bytes + (vbox ? 2 : 1) * r_bytes + c_bytes;
 };
 
 // the static data of restriction tile t's irregular rows (cell and position pairs, columns
@@ -486,14 +571,15 @@ __device__ __forceinline__ void prefetch_tile_rows(const RestrictArgs<T>& A, int
 }
 
 template <typename T, bool CROSS>
-__global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ CUtensorMap tin,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(const __grid_constant__ CUtensorMap tin,
                                                        const __grid_constant__ CUtensorMap tr,
                                                        const __grid_constant__ CUtensorMap tcls,
                                                        const __grid_constant__ CUtensorMap tvol, RestrictArgs<T> A) {
   using S = RestrictStage<T>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ T res[JY][JX];      // residual of every fine cell of the tile (0 on empty cells)
+  __shared__ __align__(16) T res[JY][JX];      // residual of every fine cell of the tile (0 on empty cells)
   __shared__ __align__(8) uint64_t bar[2];
+  __shared__ __align__(16) unsigned wmax[8];
   const int G = gridDim.x;
   const int K = (A.ntiles - (int)blockIdx.x + G - 1) / G;
   // the first tile's row range and rows while the previous launch drains
@@ -510,7 +596,7 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
     if (part != 2) {
       mbar_expect_tx(&bar[sb], S::tx);
       tma_load_2d(st + S::c_off, &tcls, &bar[sb], cx0, cy0);
-      tma_load_2d(st + S::v_off, &tvol, &bar[sb], cx0, cy0 + 2);
+      if (S::vbox) tma_load_2d(st + S::v_off, &tvol, &bar[sb], cx0, cy0 + 2);
     }
     if (part != 1) {
       tma_load_3d(st, &tin, &bar[sb], cx0, cy0, z);
@@ -534,7 +620,6 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
     issue(blockIdx.x, 0, 2);
     if (K > 1) issue(blockIdx.x + G, 1, 2);
   }
-  const int x = threadIdx.x & 63, y0 = (threadIdx.x >> 6) * 8;
   for (int k = 0; k < K; ++k) {
     const int t = blockIdx.x + k * G;
     const int sb = k & 1;
@@ -553,13 +638,24 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
       for (int m = 0; m < A.W; ++m) acc += A.rq_val[(long)m * A.nrr + q] * uf[A.rq_col[(long)m * A.nrr + q]];
       res[loc >> 6][loc & 63] = rf[cell] - acc;
     }
-    // class bytes of this thread's two coarse cells (0 outside the coarse level)
+    // class bytes of this thread's two coarse cells (0 outside the coarse level), and in FP64
+    // their children's volumes
     uint8_t cc[2];
+    T vv[2][4];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c = threadIdx.x + h * 256;
       const int I = cx0 / 2 + c % (JX / 2), J = cy0 / 2 + c / (JX / 2);
       cc[h] = (I < A.nxc && J < A.nyc) ? A.clsc[(long)(J + 2) * A.pitchc + (I + 2)] : (uint8_t)0;
+      if constexpr (!S::vbox)
+        if (I < A.nxc && J < A.nyc) {
+          const T* v = A.vol + (long)(2 * J + 2) * A.pitchf + (2 * I + 2);
+          const double2 va = *reinterpret_cast<const double2*>(v), vb = *reinterpret_cast<const double2*>(v + A.pitchf);
+          vv[h][0] = va.x;
+          vv[h][1] = va.y;
+          vv[h][2] = vb.x;
+          vv[h][3] = vb.y;
+        }
     }
     const bool ok = __syncthreads_and(wait_parity(&bar[sb], parity));
     if (!ok) {
@@ -568,8 +664,8 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
       if (threadIdx.x == 0) atomicExch(A.err, 1);
       return;
     }
-    const unsigned char* st = smem_raw + sb * A.stage;
-    const T* tile = reinterpret_cast<const T*>(st);
+    unsigned char* st = smem_raw + sb * A.stage;
+    T* tile = reinterpret_cast<T*>(st);
     const T* rt = reinterpret_cast<const T*>(st + S::r_off);
     const uint8_t* ct = st + S::c_off;
     const T* vt = reinterpret_cast<const T*>(st + S::v_off);
@@ -604,56 +700,17 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
           for (int b = 0; b < 6; ++b) w[q][b] = w[q + 1][b];
       }
     } else {
-      // FP64 (one column per thread), with the mixed term in factored form as in tile_sweep
-      T w[5][5], D[5];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int b = 0; b < 5; ++b) w[q][b] = tile[(y0 + q) * HX + x + b];
-        if (CROSS) D[q] = A.S.gx[0] * w[q][0] + A.S.gx[1] * w[q][1] + A.S.gx[3] * w[q][3] + A.S.gx[4] * w[q][4];
-      }
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-#pragma unroll
-        for (int b = 0; b < 5; ++b) w[4][b] = tile[(y0 + kk + 4) * HX + x + b];
-        if (CROSS) D[4] = A.S.gx[0] * w[4][0] + A.S.gx[1] * w[4][1] + A.S.gx[3] * w[4][3] + A.S.gx[4] * w[4][4];
-        const uint8_t cv = ct[(y0 + kk + 2) * CLX + x + 2];
-        if (cv == 1) {
-          T acc = 0;
-          if (CROSS) {
-            acc = A.S.cc * w[2][2];
-            acc = fma(A.S.lx[0], w[2][0], acc);
-            acc = fma(A.S.lx[1], w[2][1], acc);
-            acc = fma(A.S.lx[3], w[2][3], acc);
-            acc = fma(A.S.lx[4], w[2][4], acc);
-            acc = fma(A.S.ly[0], w[0][2], acc);
-            acc = fma(A.S.ly[1], w[1][2], acc);
-            acc = fma(A.S.ly[3], w[3][2], acc);
-            acc = fma(A.S.ly[4], w[4][2], acc);
-            acc = fma(A.S.gy[0], D[0], acc);
-            acc = fma(A.S.gy[1], D[1], acc);
-            acc = fma(A.S.gy[3], D[3], acc);
-            acc = fma(A.S.gy[4], D[4], acc);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 5; ++q)
-#pragma unroll
-              for (int b = 0; b < 5; ++b) {
-                if (q != 2 && b != 2) continue;
-                acc += A.S.w[q * 5 + b] * w[q][b];
-              }
-          }
-          res[y0 + kk][x] = rt[(y0 + kk) * HX + x + 2] - acc;
-        } else if (cv == 0) {
-          res[y0 + kk][x] = (T)0;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-          for (int b = 0; b < 5; ++b) w[q][b] = w[q + 1][b];
-          if (CROSS) D[q] = D[q + 1];
-        }
-      }
+      // FP64: the stencil in integer form, two columns and four rows per thread (as in k_smooth)
+      const int x0 = 2 * (threadIdx.x & 31), y1 = (threadIdx.x >> 5) * 4;
+      tile_stencil64<CROSS>(tile, wmax, x0, y1, true, A.S, A.Q, [&](int kk, double s0, double s1) {
+        const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y1 + kk + 2) * CLX + x0 + 2);
+        const double2 r2 = *reinterpret_cast<const double2*>(rt + (y1 + kk) * HX + x0 + 2);
+        const uint32_t cv0 = c2 & 0xffu, cv1 = c2 >> 8;
+        if (cv0 == 1u) res[y1 + kk][x0] = r2.x - s0;
+        else if (cv0 == 0u) res[y1 + kk][x0] = 0.0;
+        if (cv1 == 1u) res[y1 + kk][x0 + 1] = r2.y - s1;
+        else if (cv1 == 0u) res[y1 + kk][x0 + 1] = 0.0;
+      });
     }
     if (k + 1 < K) prefetch_tile_rows(A, n0, n1);
     __syncthreads();
@@ -665,7 +722,8 @@ __global__ void __launch_bounds__(256, 3) k_restrict_p(const __grid_constant__ C
       const int ci = c % (JX / 2), cj = c / (JX / 2);
       const long pc = (long)(cy0 / 2 + cj + 2) * A.pitchc + (cx0 / 2 + ci + 2);
       const T* v = vt + (2 * cj) * HX + 2 * ci + 2;
-      const T v0 = v[0], v1 = v[1], v2 = v[HX], v3 = v[HX + 1];
+      const T v0 = S::vbox ? v[0] : vv[h][0], v1 = S::vbox ? v[1] : vv[h][1], v2 = S::vbox ? v[HX] : vv[h][2],
+              v3 = S::vbox ? v[HX + 1] : vv[h][3];
       const T s = v0 * res[2 * cj][2 * ci] + v1 * res[2 * cj][2 * ci + 1] + v2 * res[2 * cj + 1][2 * ci] +
                   v3 * res[2 * cj + 1][2 * ci + 1];
       const T sv = v0 + v1 + v2 + v3;

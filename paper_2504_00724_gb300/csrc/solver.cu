@@ -22,6 +22,7 @@
 #include "coarse.cuh"
 #include "smooth.cuh"
 #include "outer.cuh"
+#include "apply.cuh"
 #include "group.cuh"
 #include "krylov.cuh"
 
@@ -79,7 +80,7 @@ struct DevLevel {
   int32_t* bot_cell = nullptr;
   double* bot64 = nullptr;
   float* bot32 = nullptr;
-  int32_t *tr_ptr = nullptr, *tr_cell = nullptr, *tr_row = nullptr;
+  int32_t *tr_ptr = nullptr, *tr_cell = nullptr, *tr_rcell = nullptr;
   double* tr_val = nullptr;
   // work arrays (padded), FP64 and FP32 sets
   double *u64[2] = {nullptr, nullptr}, *r64 = nullptr, *t64 = nullptr, *res64 = nullptr;
@@ -181,13 +182,12 @@ struct ccm_handle {
   int* herr = nullptr;         // pinned copy
   double* rhat = nullptr;      // level-0 padded FP64 right-hand side (h^2-scaled)
   double* uhat = nullptr;      // level-0 padded FP64 solution
-  bool fused_outer = false;    // mixed form: TMA-tiled FP64 residual writing r32 and the norm
+  bool fused_outer = false;    // TMA-tiled FP64 residual that folds in the norm (and writes r32 in the mixed form)
   int B = 1;                   // right-hand sides the FP32 work arrays and level-0 FP64 arrays hold
   int bmax = 1;                // right-hand sides one graph replay advances (B where batching applies)
   int nb = 1;                  // right-hand sides of the launches being issued (<= bmax)
   CUtensorMap tm_uhat, tm_rhat;  // 68 x 36 box over uhat, 68 x 32 box over rhat
-  dev::SepStencil sep{};       // the regular stencil in factored form
-  dev::FFStencil ffs{};        // its three coefficients as FP32 pairs (float-float residual)
+  dev::QStencil Q{};           // the regular stencil in integer form (FP64 passes)
   unsigned long long* dnorm = nullptr;
   unsigned long long* hnorm = nullptr;   // pinned
   ccm_info info{};
@@ -216,7 +216,7 @@ struct ccm_handle {
   cudaStream_t side = nullptr;          // second stream: SMO-2 blocks beside the regular sweep
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool capturing = false;
-  // one-launch requests to the next persistent FP32 sweep (set while a V-cycle is issued,
+  // one-launch requests to the next persistent sweep (set while a V-cycle is issued,
   // cleared when used): zero_u_next, its old iterate is 0 (not read; a level's first sweep);
   // fold_next (level 0), it also adds its new values to u_hat (the outer iteration's update).
   // fold_last marks the last inner cycle; folded reports that a sweep took the update.
@@ -383,6 +383,7 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   a.u_old = U<T>(L);
   a.u_new = Uother<T>(L);
   a.S = stencil<T>(H);
+  a.Q = H->Q;
   a.blk = L.blk;
   a.blk_off = L.blk_off;
   a.inv = Inv<T>(L);
@@ -397,7 +398,7 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   A.stage = L.smooth_stage[k];
   A.max_ext = std::max(1, L.max_ext);
   const bool l0f = &L == &H->L[0] && sizeof(T) == 4;
-  a.zero_u = sizeof(T) == 4 && !C && H->zero_u_next ? 1 : 0;
+  a.zero_u = !C && H->zero_u_next ? 1 : 0;
   a.uhat = l0f && H->fold_next ? H->uhat : nullptr;
   if (a.uhat) H->folded = true;
   H->zero_u_next = H->fold_next = false;
@@ -582,7 +583,9 @@ void restrict_to(ccm_handle* H, DevLevel& F, DevLevel& C, cudaStream_t s) {
     A.clsc = C.cls;
     A.rc = R<T>(C);
     A.uc = U<T>(C);
+    A.vol = Vol<T>(F);
     A.S = stencil<T>(H);
+    A.Q = H->Q;
     A.err = H->derr;
     A.stage = F.restrict_stage[kk];
     A.bs = F.npad;
@@ -752,12 +755,13 @@ void vcycle(ccm_handle* H, int m, cudaStream_t s, bool prolong_first = false) {
   }
   // prolong_first: the initial guess is u + P u^(m+1) (the FMG ascent); the first
   // pre-smoothing sweep reads it on the fly.  Otherwise a coarse level's iterate is 0 on entry
-  // (the restriction cleared it), so its first persistent FP32 sweep does not read it; level
-  // 0's first sweep gets the same request from the outer iteration
+  // (the restriction cleared it), so its first persistent sweep does not read it; level
+  // 0's first sweep gets the same request from the mixed outer iteration
   if (prolong_first && H->par.nu1 == 0) prolong_from<T>(H, F, C, s);
-  const bool persistent = F.smooth_ok[1] && H->persistent && H->par.smoother == 1 && H->par.ras_passes <= 1;
+  const bool persistent =
+      F.smooth_ok[sizeof(T) == 8 ? 0 : 1] && H->persistent && H->par.smoother == 1 && H->par.ras_passes <= 1;
   for (int k = 0; k < H->par.nu1; ++k) {
-    if (k == 0 && m > 0 && !prolong_first && sizeof(T) == 4 && persistent) H->zero_u_next = true;
+    if (k == 0 && m > 0 && !prolong_first && persistent) H->zero_u_next = true;
     if (k > 0 || prolong_first) H->zero_u_next = false;
     if (k == 0 && prolong_first) smooth_step<T>(H, F, s, U<T>(C), C.pitch);
     else smooth_step<T>(H, F, s);
@@ -794,37 +798,86 @@ void fmg(ccm_handle* H, cudaStream_t s) {
   for (int m = M - 1; m >= 0; --m) vcycle<T>(H, m, s, true);
 }
 
-// the regular cells' part of the outer residual runs in float-float arithmetic (about 48
-// bits: good for relative residuals down to about 1e-11) when the tolerance allows, else in
-// FP64
-inline bool resid_float_float(const ccm_handle* H) { return H->par.rtol >= 1e-11; }
-
-// mixed form: t = rhat - L uhat on level 0 into the FP32 right-hand side, max |t| into dnorm
-void outer_residual32(ccm_handle* H, cudaStream_t s) {
+// t = rhat - L u on level 0 (u FP64, tu its tensor map): max |t| into dnorm and, with r32, the
+// FP32 image of t
+void outer_residual(ccm_handle* H, const double* u, const CUtensorMap& tu, float* r32, cudaStream_t s) {
   DevLevel& L = H->L[0];
-  const int nb = H->nb;
-  cudaMemsetAsync(H->dnorm, 0, nb * sizeof(unsigned long long), s);
-  {
-    ProfScope ps(H, CCM_PROF_RESID_FP64, s);
-    const dim3 g(L.ntiles64, nb);
-    if (resid_float_float(H)) {
-      if (H->cross)
-        KL(launch_k(dev::k_resid_ff<true>, g, 256, dev::Resid64Smem::bytes(true), s, H->tm_uhat, H->tm_rhat, L.tmcls,
-                    L.tiles64, L.nx, L.pitch, L.r32, H->dnorm, H->ffs, H->derr, L.npad));
-      else
-        KL(launch_k(dev::k_resid_ff<false>, g, 256, dev::Resid64Smem::bytes(false), s, H->tm_uhat, H->tm_rhat, L.tmcls,
-                    L.tiles64, L.nx, L.pitch, L.r32, H->dnorm, H->ffs, H->derr, L.npad));
-    } else if (H->cross) {
-      KL(launch_k(dev::k_resid64<true>, g, 256, dev::Resid64Smem::bytes(true), s, H->tm_uhat, H->tm_rhat,
-                  L.tmcls, L.tiles64, L.nx, L.pitch, L.r32, H->dnorm, H->sep, H->derr, L.npad));
-    } else {
-      KL(launch_k(dev::k_resid64<false>, g, 256, dev::Resid64Smem::bytes(false), s, H->tm_uhat, H->tm_rhat,
-                  L.tmcls, L.tiles64, L.nx, L.pitch, L.r32, H->dnorm, H->sep, H->derr, L.npad));
-    }
+  cudaMemsetAsync(H->dnorm, 0, H->nb * sizeof(unsigned long long), s);
+  dev::ResidArgs A{};
+  A.tiles = L.tiles64;
+  A.nrow = ceil_div(L.n2, 256);
+  A.nx = L.nx;
+  A.pitch = L.pitch;
+  A.n2 = L.n2;
+  A.W = L.W;
+  A.cell = L.irr_cell;
+  A.col = L.ell_col;
+  A.val = L.ell64;
+  A.u = u;
+  A.r = H->rhat;
+  A.r32 = r32;
+  A.norm = H->dnorm;
+  A.S = H->S64;
+  A.Q = H->Q;
+  A.err = H->derr;
+  A.bs = L.npad;
+  ProfScope ps(H, CCM_PROF_RESID_FP64, s);
+  const dim3 g(A.nrow + L.ntiles64, H->nb);
+  const size_t sm = dev::ResidSmem::bytes;
+  if (H->cross) KL(launch_k(dev::k_resid<true>, g, 256, sm, s, tu, H->tm_rhat, L.tmcls, A));
+  else KL(launch_k(dev::k_resid<false>, g, 256, sm, s, tu, H->tm_rhat, L.tmcls, A));
+}
+
+// the tensor map over u, one of level 0's FP64 iterates
+const CUtensorMap& map_of(const ccm_handle* H, const double* u) {
+  const DevLevel& L = H->L[0];
+  return u == L.u64[0] ? L.tm64[0] : L.tm64[1];
+}
+
+// out = L u + N g over a level (TRANS: the regular part of L^T v, and N^T v into og where wanted)
+// for nrhs vectors in one launch
+template <bool TRANS>
+void launch_apply(ccm_handle* H, DevLevel& L, dev::Grid<const double*> u, dev::Grid<double*> out, const double* g,
+                  double* og, int nrhs, double scale, cudaStream_t s) {
+  dev::ApplyArgs A{};
+  A.u = u;
+  A.out = out;
+  A.cls = L.cls;
+  A.nx = L.nx;
+  A.ny = L.ny;
+  A.pitch = L.pitch;
+  A.tx = ceil_div(L.nx, dev::JX);
+  A.nrow = !TRANS || og ? ceil_div(L.n2, 256) : 0;
+  A.n2 = L.n2;
+  A.W = L.W;
+  A.cell = L.irr_cell;
+  A.col = L.ell_col;
+  A.val = L.ell64;
+  A.nb = L.nb;
+  A.seg = L.seg;
+  A.g = g;
+  A.og = og;
+  A.nseg = H->info.n_segments;
+  A.scale = scale;
+  A.vec = ((uintptr_t)out.p % 16) == 0 && out.stride % 2 == 0 && (out.batch % 2 == 0 || nrhs == 1);
+  A.S = H->S64;
+  A.Q = H->Q;
+  const int tiles = out.p ? A.tx * ceil_div(L.ny, dev::JY) : 0;
+  // the grid's y extent is limited to 65535 vectors a launch
+  for (int k = 0; k < nrhs && A.nrow + tiles > 0; k += 65535) {
+    const dim3 grid(A.nrow + tiles, std::min(nrhs - k, 65535));
+    if (H->cross) KL(launch_k(dev::k_apply<true, TRANS>, grid, 256, 0, s, A));
+    else KL(launch_k(dev::k_apply<false, TRANS>, grid, 256, 0, s, A));
+    A.u.p += 65535 * A.u.batch;
+    if (A.out.p) A.out.p += 65535 * A.out.batch;
+    if (A.g) A.g += 65535 * A.nseg;
+    if (A.og) A.og += 65535 * A.nseg;
   }
-  if (L.n2)
-    KL(launch_k(dev::k_rows_r32, dim3(ceil_div(L.n2, 128), nb), 128, 0, s, L.n2, L.W, L.irr_cell, L.ell_col, L.ell64,
-                (const double*)H->uhat, (const double*)H->rhat, L.r32, H->dnorm, L.npad));
+}
+
+// [p, p + n) and [q, q + m) share a value (null: nothing)
+inline bool overlap(const double* p, long n, const double* q, long m) {
+  return p && q && (uintptr_t)p < (uintptr_t)(q + m) && (uintptr_t)q < (uintptr_t)(p + n);
 }
 
 int check_level(ccm_handle* h, int level) {
@@ -915,7 +968,10 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   for (int k = 0; k < 2 && d.tma && one_chunk && nitems > 0; ++k) {
     const size_t es = k == 0 ? sizeof(double) : sizeof(float);
     const size_t tile = k == 0 ? dev::TileStage<double>::bytes(true) : dev::TileStage<float>::bytes(true);
-    const size_t blk = ((size_t)d.max_ext * d.max_core * es + 15) & ~(size_t)15;
+    // the rows of a block item that one stage takes (all in FP32, half in FP64)
+    const int ext = k == 0 ? std::max(2, dev::block_split(d.max_ext)) : d.max_ext;
+    if (k == 0 && d.max_core > 128) continue;
+    const size_t blk = ((size_t)ext * d.max_core * es + 15) & ~(size_t)15;
     const size_t stage = (std::max(tile, blk) + 127) & ~(size_t)127;
     // two stages, then per extended row of a block: its residual, old value and cell
     const size_t smem = 2 * stage + 3 * (((size_t)std::max(1, d.max_ext) * es + 15) & ~(size_t)15);
@@ -952,6 +1008,7 @@ int upload_hierarchy(ccm_handle* h) {
     h->S64.w[k] = w[k / 5][k % 5];
     h->S32.w[k] = (float)w[k / 5][k % 5];
   }
+  h->Q = dev::q_stencil(h->a, h->b, h->c);
   h->S64.omega_d = h->par.omega / w[2][2];
   h->S32.omega_d = (float)(h->par.omega / w[2][2]);
   {
@@ -1026,7 +1083,9 @@ int upload_hierarchy(ccm_handle* h) {
       d.ncolT = (int)hl.tr_cell.size();
       d.tr_ptr = A.upload(hl.tr_ptr);
       d.tr_cell = A.upload(hl.tr_cell);
-      d.tr_row = A.upload(hl.tr_row);
+      std::vector<int32_t> rc(hl.tr_row.size());
+      for (size_t k = 0; k < rc.size(); ++k) rc[k] = hl.irr_cell[hl.tr_row[k]];
+      d.tr_rcell = A.upload(rc);
       d.tr_val = A.upload(hl.tr_val);
     }
     d.ntiles64 = (int)hl.tiles64.size() / 2;
@@ -1162,6 +1221,9 @@ int upload_hierarchy(ccm_handle* h) {
         if (occ < 1 || nsm < 1) continue;
         d.restrict_ok[k] = true;
         d.restrict_stage[k] = stage;
+        // FP64: one CTA per SM until there are two tiles for each, so that every CTA's first copy
+        // has its SM's bandwidth to itself
+        if (k == 0 && d.ntiles64r < 2 * nsm) occ = 1;
         d.restrict_grid[k] = std::min(d.ntiles64r, nsm * occ);
         d.restrict_cap[k] = nsm * occ;
       }
@@ -1192,27 +1254,9 @@ int upload_hierarchy(ccm_handle* h) {
   h->rhat = A.alloc<double>(h->B * h->L[0].npad);
   h->uhat = A.alloc<double>(h->B * h->L[0].npad);
   {
-    static const double lap[5] = {-1.0, 16.0, -30.0, 16.0, -1.0};
-    static const double grad[5] = {1.0, -8.0, 0.0, 8.0, -1.0};
-    for (int k = 0; k < 5; ++k) {
-      h->sep.lx[k] = h->a * lap[k] / 12.0;
-      h->sep.ly[k] = h->c * lap[k] / 12.0;
-      h->sep.gx[k] = grad[k] / 12.0;
-      h->sep.gy[k] = h->b * grad[k] / 12.0;
-    }
-    h->sep.cc = h->sep.lx[2] + h->sep.ly[2];
-    auto split = [](double v, float& hi, float& lo) {
-      hi = (float)v;
-      lo = (float)(v - (double)hi);
-    };
-    split(h->a / 12.0, h->ffs.ah, h->ffs.al);
-    split(h->c / 12.0, h->ffs.ch, h->ffs.cl);
-    split(h->b / 144.0, h->ffs.bh, h->ffs.bl);
     const DevLevel& d0 = h->L[0];
-    cudaFuncSetAttribute(dev::k_resid64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::Resid64Smem::bytes(true));
-    cudaFuncSetAttribute(dev::k_resid64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::Resid64Smem::bytes(false));
-    cudaFuncSetAttribute(dev::k_resid_ff<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::Resid64Smem::bytes(true));
-    cudaFuncSetAttribute(dev::k_resid_ff<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::Resid64Smem::bytes(false));
+    cudaFuncSetAttribute(dev::k_resid<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::ResidSmem::bytes);
+    cudaFuncSetAttribute(dev::k_resid<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dev::ResidSmem::bytes);
     h->fused_outer = A.err == cudaSuccess && d0.tma && d0.ntiles64 > 0 &&
                      make_tmap(&h->tm_uhat, h->uhat, d0.pitch, d0.rows, true, h->B) &&
                      make_tmap(&h->tm_rhat, h->rhat, d0.pitch, d0.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY,
@@ -1457,30 +1501,10 @@ int ccm_boundary_averages(const ccm_handle* h, ccm_grad_fn g, void* ctx, double*
   return CCM_OK;
 }
 
-int ccm_apply(ccm_handle* h, const double* u, const double* g, double* out, int nrhs, void* stream) {
-  if (!h || !u || !out || nrhs < 1) return CCM_EINVAL;
-  cudaStream_t s = (cudaStream_t)stream;
-  DevLevel& L = h->L[0];
-  const long nu = (long)L.nx * L.ny;
-  dim3 pg(ceil_div(L.nx, 128), L.ny);
-  for (int k = 0; k < nrhs; ++k) {
-    KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, u + k * nu, L.t64, 1.0));
-    launch_regular<double>(h, L, L.t64, nullptr, L.u64[1 - L.cur64], false, s);
-    if (L.n2)
-      KL(launch_k(dev::k_rows<double, double, false, true>, ceil_div(L.n2, 128), 128, 0, s, 
-          L.n2, L.W, L.irr_cell, L.ell_col, L.ell64, L.t64, nullptr, L.u64[1 - L.cur64], L.nb, L.seg,
-          g ? g + (long)k * h->info.n_segments : nullptr));
-    KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, L.u64[1 - L.cur64], out + k * nu,
-                                             1.0 / (L.h * L.h)));
-  }
-  CCM_CUDA(cudaGetLastError());
-  return CCM_OK;
-}
-
 }  // extern "C"
 
-// Scratch of ccm_apply_noalloc: two padded FP64 grids, held by every device that loads the
-// library.  Host code only ever uses the device address looked up below.
+// Scratch of ccm_apply_noalloc: two FP64 grids, held by every device that loads the library.
+// Host code only ever uses the device address looked up below.
 static __device__ __align__(256) double g_noalloc_scratch[2 * CCM_NOALLOC_MAX_PADDED];
 
 namespace {
@@ -1504,10 +1528,33 @@ int noalloc_scratch(double** out) {
 
 extern "C" {
 
+int ccm_apply(ccm_handle* h, const double* u, const double* g, double* out, int nrhs, void* stream) {
+  if (!h || !u || !out || nrhs < 1) return CCM_EINVAL;
+  cudaStream_t s = (cudaStream_t)stream;
+  DevLevel& L = h->L[0];
+  const long nu = (long)L.nx * L.ny, ns = h->info.n_segments;
+  const double sc = 1.0 / (L.h * L.h);
+  if (!overlap(out, nrhs * nu, u, nrhs * nu) && !overlap(out, nrhs * nu, g, nrhs * ns)) {
+    launch_apply<false>(h, L, {u, L.nx, nu}, {out, L.nx, nu}, g, nullptr, nrhs, sc, s);
+  } else {
+    // the result lies over an input: one vector at a time through the padded work arrays
+    const long o = 2L * L.pitch + 2;
+    dim3 pg(ceil_div(L.nx, 128), L.ny);
+    double* w = L.u64[1 - L.cur64];
+    for (int k = 0; k < nrhs; ++k) {
+      KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, u + k * nu, L.t64, 1.0));
+      launch_apply<false>(h, L, {L.t64 + o, L.pitch, 0}, {w + o, L.pitch, 0}, g ? g + k * ns : nullptr, nullptr, 1, 1.0, s);
+      KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, w, out + k * nu, sc));
+    }
+  }
+  CCM_CUDA(cudaGetLastError());
+  return CCM_OK;
+}
+
 int ccm_apply_noalloc(const ccm_handle* hc, const double* u, const double* g, double* out, void* stream) {
   if (!hc || !u || !out) return CCM_EINVAL;
   ccm_handle* h = const_cast<ccm_handle*>(hc);
-  const DevLevel& L = h->L[0];
+  DevLevel& L = h->L[0];
   if (L.npad > CCM_NOALLOC_MAX_PADDED) return CCM_ETOOLARGE;
   // the scratch address below is the current device's; the handle's arrays live on h->device
   int cur = -1;
@@ -1517,23 +1564,17 @@ int ccm_apply_noalloc(const ccm_handle* hc, const double* u, const double* g, do
   int rc = noalloc_scratch(&scratch);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  double* up = scratch;                              // padded u
-  double* op = scratch + CCM_NOALLOC_MAX_PADDED;     // padded L u + N g
-  CCM_CUDA(cudaMemsetAsync(up, 0, L.npad * sizeof(double), s));
-  CCM_CUDA(cudaMemsetAsync(op, 0, L.npad * sizeof(double), s));
-  dim3 pg(ceil_div(L.nx, 128), L.ny);
-  KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, u, up, 1.0));
-  if (L.ntiles) {
-    dim3 blk(dev::TX, dev::TY);
-    if (h->cross)
-      KL(launch_k(dev::k_regular<double, true, false>, L.ntiles, blk, 0, s, L.tiles, L.cls, L.nx, L.ny, L.pitch, up, nullptr, op, h->S64));
-    else
-      KL(launch_k(dev::k_regular<double, false, false>, L.ntiles, blk, 0, s, L.tiles, L.cls, L.nx, L.ny, L.pitch, up, nullptr, op, h->S64));
+  const long nu = (long)L.nx * L.ny;
+  const double sc = 1.0 / (L.h * L.h);
+  if (!overlap(out, nu, u, nu) && !overlap(out, nu, g, h->info.n_segments)) {
+    launch_apply<false>(h, L, {u, L.nx, nu}, {out, L.nx, nu}, g, nullptr, 1, sc, s);
+  } else {
+    // the result lies over an input: through the scratch, which only such calls use
+    CCM_CUDA(cudaMemcpyAsync(scratch, u, nu * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    double* w = scratch + CCM_NOALLOC_MAX_PADDED;
+    launch_apply<false>(h, L, {scratch, L.nx, nu}, {w, L.nx, nu}, g, nullptr, 1, sc, s);
+    CCM_CUDA(cudaMemcpyAsync(out, w, nu * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
-  if (L.n2)
-    KL(launch_k(dev::k_rows<double, double, false, true>, ceil_div(L.n2, 128), 128, 0, s, 
-        L.n2, L.W, L.irr_cell, L.ell_col, L.ell64, up, nullptr, op, L.nb, L.seg, g));
-  KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, op, out, 1.0 / (L.h * L.h)));
   CCM_CUDA(cudaGetLastError());
   return CCM_OK;
 }
@@ -1542,26 +1583,34 @@ int ccm_apply_T(ccm_handle* h, const double* v, double* out_u, double* out_g, in
   if (!h || !v || nrhs < 1 || (!out_u && !out_g)) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   DevLevel& L = h->L[0];
-  const long nu = (long)L.nx * L.ny;
-  dim3 pg(ceil_div(L.nx, 128), L.ny);
+  const long nu = (long)L.nx * L.ny, ns = h->info.n_segments;
   const double sc = 1.0 / (L.h * L.h);
-  for (int k = 0; k < nrhs; ++k) {
-    KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, v + k * nu, L.t64, 1.0));
-    if (out_u) {
-      double* o = L.u64[1 - L.cur64];
-      dim3 blk(dev::TX, dev::TY);
-      if (L.ntiles) {
-        if (h->cross) KL(dev::k_regular_T<true><<<L.ntiles, blk, 0, s>>>(L.tiles, L.cls, L.nx, L.ny, L.pitch, L.t64, o, h->S64));
-        else KL(dev::k_regular_T<false><<<L.ntiles, blk, 0, s>>>(L.tiles, L.cls, L.nx, L.ny, L.pitch, L.t64, o, h->S64));
-      }
-      if (L.ncolT)
-        KL(dev::k_rows_T<<<ceil_div(L.ncolT, 128), 128, 0, s>>>(L.ncolT, L.tr_ptr, L.tr_cell, L.tr_row, L.tr_val,
-                                                            L.irr_cell, L.t64, o));
-      KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, o, out_u + k * nu, sc));
+  auto rows_T = [&](dev::Grid<const double*> vv, dev::Grid<double*> o, int n, double scale) {
+    for (int k = 0; k < n && L.ncolT; k += 65535) {
+      KL(launch_k(dev::k_rows_T, dim3(ceil_div(L.ncolT, 128), std::min(n - k, 65535)), 128, 0, s, L.ncolT,
+                  (const int32_t*)L.tr_ptr, (const int32_t*)L.tr_cell, (const int32_t*)L.tr_rcell, (const double*)L.tr_val,
+                  vv, o, L.pitch, scale));
+      vv.p += 65535 * vv.batch;
+      o.p += 65535 * o.batch;
     }
-    if (out_g && L.n2)
-      KL(dev::k_bnd_T<<<ceil_div(L.n2, 128), 128, 0, s>>>(L.n2, L.irr_cell, L.nb, L.seg, L.t64,
-                                                      out_g + (long)k * h->info.n_segments, sc));
+  };
+  if (!overlap(out_u, nrhs * nu, v, nrhs * nu) && !overlap(out_g, nrhs * ns, v, nrhs * nu)) {
+    launch_apply<true>(h, L, {v, L.nx, nu}, {out_u, L.nx, nu}, nullptr, out_g, nrhs, sc, s);
+    if (out_u) rows_T({v, L.nx, nu}, {out_u, L.nx, nu}, nrhs, sc);
+  } else {
+    // a result lies over the input: one vector at a time through the padded work arrays
+    const long o = 2L * L.pitch + 2;
+    dim3 pg(ceil_div(L.nx, 128), L.ny);
+    double* w = L.u64[1 - L.cur64];
+    for (int k = 0; k < nrhs; ++k) {
+      KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, v + k * nu, L.t64, 1.0));
+      if (out_u) {
+        launch_apply<true>(h, L, {L.t64 + o, L.pitch, 0}, {w + o, L.pitch, 0}, nullptr, nullptr, 1, 1.0, s);
+        rows_T({L.t64 + o, L.pitch, 0}, {w + o, L.pitch, 0}, 1, 1.0);
+        KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, w, out_u + k * nu, sc));
+      }
+      if (out_g) launch_apply<true>(h, L, {L.t64 + o, L.pitch, 0}, {nullptr, 0, 0}, nullptr, out_g + k * ns, 1, sc, s);
+    }
   }
   CCM_CUDA(cudaGetLastError());
   return CCM_OK;
@@ -1645,7 +1694,7 @@ static void iteration_body(ccm_handle* h, bool fp64, cudaStream_t s, bool to_hos
   } else if (h->fused_outer && h->kry_m > 0) {
     // r32 holds the FP32 image of the residual; e by GMRES(m) preconditioned by the cycles
     krylov_correction(h, s);
-    outer_residual32(h, s);
+    outer_residual(h, h->uhat, h->tm_uhat, L.r32, s);
     if (!to_host) return;
     cudaMemcpyAsync(h->hnorm, h->dnorm, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -1674,7 +1723,7 @@ static void iteration_body(ccm_handle* h, bool fp64, cudaStream_t s, bool to_hos
                   (const float*)L.u32[L.cur32], h->uhat, L.npad));
     }
     h->folded = false;
-    outer_residual32(h, s);
+    outer_residual(h, h->uhat, h->tm_uhat, L.r32, s);
     if (!to_host) return;
     cudaMemcpyAsync(h->hnorm, h->dnorm, h->nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -1690,15 +1739,19 @@ static void iteration_body(ccm_handle* h, bool fp64, cudaStream_t s, bool to_hos
     KL(launch_k(dev::k_axpy<float>, std::min(ceil_div(np, 256), 4096), 256, 0, s, np, L.cls, L.u32[L.cur32], h->uhat));
     ucur = h->uhat;
   }
-  {
-    ProfScope ps(h, CCM_PROF_RESID_FP64, s);
-    launch_regular<double>(h, L, ucur, h->rhat, L.t64, true, s);
+  if (fp64 && h->fused_outer) {
+    outer_residual(h, ucur, map_of(h, ucur), nullptr, s);
+  } else {
+    {
+      ProfScope ps(h, CCM_PROF_RESID_FP64, s);
+      launch_regular<double>(h, L, ucur, h->rhat, L.t64, true, s);
+    }
+    if (L.n2)
+      KL(launch_k(dev::k_rows<double, double, true, true>, ceil_div(L.n2, 128), 128, 0, s,
+          L.n2, L.W, L.irr_cell, L.ell_col, L.ell64, ucur, h->rhat, L.t64, nullptr, nullptr, nullptr));
+    cudaMemsetAsync(h->dnorm, 0, sizeof(unsigned long long), s);
+    KL(launch_k(dev::k_absmax<double>, std::min(ceil_div(np, 256), 1216), 256, 0, s, np, L.cls, L.t64, h->dnorm, 0L));
   }
-  if (L.n2)
-    KL(launch_k(dev::k_rows<double, double, true, true>, ceil_div(L.n2, 128), 128, 0, s, 
-        L.n2, L.W, L.irr_cell, L.ell_col, L.ell64, ucur, h->rhat, L.t64, nullptr, nullptr, nullptr));
-  cudaMemsetAsync(h->dnorm, 0, sizeof(unsigned long long), s);
-  KL(launch_k(dev::k_absmax<double>, std::min(ceil_div(np, 256), 1216), 256, 0, s, np, L.cls, L.t64, h->dnorm, 0L));
   if (!to_host) return;
   cudaMemcpyAsync(h->hnorm, h->dnorm, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -1880,8 +1933,9 @@ static int load_rhs(ccm_handle* h, const double* f, const double* g, const doubl
 // max |r_hat - L U0| of one right-hand side into dnorm[0] (no host synchronisation)
 static void initial_residual(ccm_handle* h, const double* U0, cudaStream_t s) {
   DevLevel& L = h->L[0];
-  if (h->par.precision != CCM_FP64 && h->fused_outer) {
-    outer_residual32(h, s);
+  if (h->fused_outer) {
+    if (h->par.precision == CCM_FP64) outer_residual(h, U0, map_of(h, U0), nullptr, s);
+    else outer_residual(h, h->uhat, h->tm_uhat, L.r32, s);
     return;
   }
   launch_regular<double>(h, L, U0, h->rhat, L.t64, true, s);
@@ -2385,13 +2439,16 @@ int ccm_level_apply(ccm_handle* h, int level, const double* u, double* out, void
   if (check_level(h, level) || !u || !out) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   DevLevel& L = h->L[level];
-  dim3 pg(ceil_div(L.nx, 128), L.ny);
-  KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, u, L.t64, 1.0));
-  launch_regular<double>(h, L, L.t64, nullptr, L.r64, false, s);
-  if (L.n2)
-    KL(launch_k(dev::k_rows<double, double, false, true>, ceil_div(L.n2, 128), 128, 0, s, 
-        L.n2, L.W, L.irr_cell, L.ell_col, L.ell64, L.t64, nullptr, L.r64, L.nb, L.seg, nullptr));
-  KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, L.r64, out, 1.0 / (L.h * L.h)));
+  const long nu = (long)L.nx * L.ny;
+  const double sc = 1.0 / (L.h * L.h);
+  if (!overlap(out, nu, u, nu)) {
+    launch_apply<false>(h, L, {u, L.nx, nu}, {out, L.nx, nu}, nullptr, nullptr, 1, sc, s);
+  } else {
+    const long o = 2L * L.pitch + 2;
+    dim3 pg(ceil_div(L.nx, 128), L.ny);
+    KL(dev::k_pack<double, double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, u, L.t64, 1.0));
+    launch_apply<false>(h, L, {L.t64 + o, L.pitch, 0}, {out, L.nx, nu}, nullptr, nullptr, 1, sc, s);
+  }
   CCM_CUDA(cudaGetLastError());
   return CCM_OK;
 }
