@@ -41,7 +41,8 @@ struct CoarseLevel {
   const int64_t* blk_off;
   const T* inv;            // per block: inverse rows [ext][core]
   const int32_t* bot_cell;
-  const T* bot;            // bottom inverse, [col][row]
+  const T* bot;            // bottom inverse, [col][bot_ld]
+  int bot_ld;
 };
 
 template <typename T>
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(COARSE_THREADS, 1) k_coarse_cluster(CoarsePara
       const int k = g * 32 + lane;
       T acc = 0;
       if (k < B.nbc)
-        for (int c = warp; c < B.nbc; c += nw) acc += B.bot[(long)c * B.nbc + k] * sres[c];
+        for (int c = warp; c < B.nbc; c += nw) acc += B.bot[(long)c * B.bot_ld + k] * sres[c];
       part[warp][lane] = acc;
       __syncthreads();
       if (warp == 0 && k < B.nbc) {

@@ -34,6 +34,11 @@ __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
+// 16 bytes of T
+template <typename T> struct Quad;
+template <> struct Quad<float> { using type = float4; };
+template <> struct Quad<double> { using type = double2; };
+
 template <typename T>
 struct Stencil {
   T w[25];        // [dj + 2][di + 2]
@@ -857,11 +862,11 @@ __global__ void k_prolong(const int32_t* __restrict__ tiles, const uint8_t* __re
 }
 
 // bottom solve: u[cell_k] = sum_c inv[c][k] r[cell_c]
-// The bottom solve u = inv(L_bottom) r split over a thread-block cluster of BOTTOM_SPLIT
-// CTAs: CTA q of the cluster takes columns [q n / S, (q + 1) n / S) of the 32 rows of its row
-// block, warps split those columns, and the cluster's rank 0 adds the S partial sums through
-// distributed shared memory in rank order (the same order every run).  Both cluster barriers
-// are passed by every thread of every CTA.
+// The dense product u = M r (the bottom inverse, or the small levels' part of a V-cycle) split
+// over thread-block clusters of BOTTOM_SPLIT CTAs: CTA q of a cluster takes columns [q n / S,
+// (q + 1) n / S) of the RB rows of its row block, its warps split those columns, and the ranks
+// add each other's partial sums through distributed shared memory in rank order (the same order
+// every run).  Both cluster barriers are passed by every thread of every CTA.
 constexpr int BOTTOM_SPLIT = 8;
 
 __device__ __forceinline__ unsigned bottom_rank() {
@@ -874,57 +879,108 @@ __device__ __forceinline__ void bottom_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
+__device__ __forceinline__ float bottom_ld(uint32_t a, float) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ double bottom_ld(uint32_t a, double) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+
+// the sum of one shared value over the cluster's CTAs in rank order
 template <typename T>
-__global__ void __launch_bounds__(256) k_bottom_split(int n, const int32_t* __restrict__ cell, const T* __restrict__ inv,
-                                                      const T* __restrict__ r, T* __restrict__ u, long bs) {
-  __shared__ T part[8][32];
-  __shared__ T tot[32];
+__device__ __forceinline__ T bottom_sum(const T* mine) {
+  const uint32_t local = (uint32_t)__cvta_generic_to_shared(mine);
+  T s = 0;
+#pragma unroll
+  for (unsigned p = 0; p < BOTTOM_SPLIT; ++p) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(p));
+    s += bottom_ld(remote, (T)0);
+  }
+  return s;
+}
+
+// M is stored [column][ld], ld >= n a multiple of 16 bytes, zero beyond row n.  A lane loads 16
+// bytes of a column; RB = 32 rows a block where the matrix is small (so that every SM has part
+// of it), 128 (FP64: 64) where it is large.  The first BOTTOM_AHEAD loads of every thread are
+// issued before the grid dependency wait (all of them at 1.2k unknowns), so that after it only
+// the right-hand side is on the way.
+constexpr int BOTTOM_AHEAD = 8;
+
+template <typename T, int RB>
+__global__ void __launch_bounds__(256) k_bottom_split(int n, int ld, const int32_t* __restrict__ cell,
+                                                      const T* __restrict__ M, const T* __restrict__ r,
+                                                      T* __restrict__ u, long bs) {
+  constexpr int VEC = 16 / sizeof(T), LPC = RB / VEC, CPW = 32 / LPC;   // lanes a column, columns a warp
+  using V = typename Quad<T>::type;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* rs = reinterpret_cast<T*>(smem_raw);               // the right-hand side at this CTA's columns
+  __shared__ __align__(16) T part[8][RB];
+  __shared__ T tot[RB];
   const unsigned q = bottom_rank();
   const int rowblk = blockIdx.x / BOTTOM_SPLIT;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int k = rowblk * 32 + lane;
+  const int k = rowblk * RB + (lane % LPC) * VEC;
   const int c0 = (int)((long)n * q / BOTTOM_SPLIT), c1 = (int)((long)n * (q + 1) / BOTTOM_SPLIT);
-  // this CTA's part of the inverse and the cells of its columns, while the previous launch
-  // drains (a warp's 32 rows of one column are one line)
-  if (k < n)
-    for (int c = c0 + warp; c < c1; c += 8) prefetch_l1(inv + (long)c * n + k);
-  for (int c = c0 + (int)threadIdx.x * 32; c < c1; c += (int)blockDim.x * 32) prefetch_l1(cell + c);
+  const int first = c0 + warp * CPW + lane / LPC;
+  const T* col = M + k;
+  V a[BOTTOM_AHEAD];
+  auto load = [&](int c) { return c < c1 && k < ld ? *reinterpret_cast<const V*>(col + (long)c * ld) : V{}; };
+#pragma unroll
+  for (int j = 0; j < BOTTOM_AHEAD; ++j) a[j] = load(first + j * 8 * CPW);
+  const int i0 = c0 + (int)threadIdx.x;
+  const int cell0 = i0 < c1 ? cell[i0] : 0, cell1 = i0 + 256 < c1 ? cell[i0 + 256] : 0;
   pdl_enter();
   r += blockIdx.y * bs;       // right-hand side blockIdx.y of the batch
   u += blockIdx.y * bs;
-  T acc = 0;
-  if (k < n)
-    for (int c = c0 + warp; c < c1; c += 8) acc += inv[(long)c * n + k] * r[cell[c]];
-  part[warp][lane] = acc;
+  if (i0 < c1) rs[threadIdx.x] = r[cell0];
+  if (i0 + 256 < c1) rs[threadIdx.x + 256] = r[cell1];
+  for (int i = i0 + 512; i < c1; i += 256) rs[i - c0] = r[cell[i]];
   __syncthreads();
-  if (warp == 0) {
+  T acc[VEC] = {};
+  for (int c = first;; ) {
+#pragma unroll
+    for (int j = 0; j < BOTTOM_AHEAD; ++j) {
+      const int cj = c + j * 8 * CPW;
+      const T x = cj < c1 ? rs[cj - c0] : (T)0;
+      const T* v = reinterpret_cast<const T*>(&a[j]);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) acc[e] += v[e] * x;
+    }
+    c += BOTTOM_AHEAD * 8 * CPW;
+    if (c - lane / LPC >= c1) break;                    // the same for a warp's lanes
+#pragma unroll
+    for (int j = 0; j < BOTTOM_AHEAD; ++j) a[j] = load(c + j * 8 * CPW);
+  }
+#pragma unroll
+  for (int e = 0; e < VEC; ++e)
+#pragma unroll
+    for (int o = LPC; o < 32; o <<= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+  if (lane < LPC)
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) part[warp][lane * VEC + e] = acc[e];
+  __syncthreads();
+  if (threadIdx.x < RB) {
     T s = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) s += part[w][lane];
-    tot[lane] = s;
+    for (int w = 0; w < 8; ++w) s += part[w][threadIdx.x];
+    tot[threadIdx.x] = s;
   }
   bottom_cluster_sync();          // every CTA's tot is written
-  if (q == 0 && warp == 0) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(&tot[lane]);
-    T s = 0;
-    for (unsigned p = 0; p < BOTTOM_SPLIT; ++p) {
-      uint32_t remote;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(p));
-      T v;
-      if constexpr (sizeof(T) == 8) {
-        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote) : "memory");
-      } else {
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-      }
-      s += v;
-    }
-    if (k < n) u[cell[k]] = s;
+  if (threadIdx.x < RB / BOTTOM_SPLIT) {                // rank q finishes its share of the rows
+    const int l = (int)q * (RB / BOTTOM_SPLIT) + (int)threadIdx.x, row = rowblk * RB + l;
+    const T s = bottom_sum(&tot[l]);
+    if (row < n) u[cell[row]] = s;
   }
-  bottom_cluster_sync();          // the other CTAs keep their shared memory until rank 0 has read it
+  bottom_cluster_sync();          // the other CTAs keep their shared memory until it has been read
 }
 
 template <typename T>
-__global__ void k_bottom(int n, const int32_t* __restrict__ cell, const T* __restrict__ inv,
+__global__ void k_bottom(int n, int ld, const int32_t* __restrict__ cell, const T* __restrict__ inv,
                          const T* __restrict__ r, T* __restrict__ u, long bs) {
   pdl_enter();
   r += blockIdx.y * bs;       // right-hand side blockIdx.y of the batch
@@ -939,7 +995,7 @@ __global__ void k_bottom(int n, const int32_t* __restrict__ cell, const T* __res
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   T acc = 0;
   if (k < n)
-    for (int c = warp; c < n; c += nw) acc += inv[(long)c * n + k] * s[c];
+    for (int c = warp; c < n; c += nw) acc += inv[(long)c * ld + k] * s[c];
   __syncthreads();
   T* part = s;   // reuse: [nw][32]
   part[warp * 32 + (threadIdx.x & 31)] = acc;

@@ -23,6 +23,7 @@
 #include "smooth.cuh"
 #include "outer.cuh"
 #include "apply.cuh"
+#include "dense.cuh"
 #include "group.cuh"
 #include "krylov.cuh"
 
@@ -31,7 +32,7 @@ using namespace ccm;
 namespace {
 
 struct DevLevel {
-  int nx = 0, ny = 0, pitch = 0, rows = 0, ntiles = 0, n2 = 0, W = 15, nblk = 0, nbc = 0, ncolT = 0;
+  int nx = 0, ny = 0, pitch = 0, rows = 0, ntiles = 0, n2 = 0, W = 15, nblk = 0, nbc = 0, bot_ld = 0, ncolT = 0;
   long npad = 0;
   double h = 0;
   int max_ext = 0, max_core = 0;
@@ -203,6 +204,14 @@ struct ccm_handle {
   int coarse_ctas = 0;         // CTAs of that cluster (16, else 8)
   size_t coarse_smem = 0;      // its dynamic shared memory (SMO-2 extended-row residuals)
   bool persistent = true;      // block-Jacobi sweeps of TMA levels as one persistent launch
+  // from level dense.m down a V-cycle from a zero iterate is one dense matrix (dense.cuh), in the
+  // arithmetic of the handle's cycles; m < 0: none
+  struct Dense {
+    int m = -1, n = 0, ld = 0;
+    int32_t* cell = nullptr;
+    double* m64 = nullptr;
+    float* m32 = nullptr;
+  } dense;
   int launch_cap = 0;          // > 0: at most this many CTAs per right-hand side in the persistent kernels
   // GMRES(kry_m) correction of the mixed outer iteration (0: plain iterative refinement)
   int kry_m = 0;
@@ -645,10 +654,17 @@ void prolong_from(ccm_handle* H, DevLevel& F, DevLevel& C, cudaStream_t s) {
               U<T>(F), F.npad, C.npad));
 }
 
+// u = M r on level B, M dense over the n cells listed, stored [column][ld] (the bottom inverse, or
+// the small levels' part of a V-cycle)
 template <typename T>
-void bottom(ccm_handle* H, DevLevel& B, cudaStream_t s) {
-  if (B.nbc >= 256) {
+void dense_product(ccm_handle* H, DevLevel& B, int n, int ld, const int32_t* cell, const T* M, cudaStream_t s) {
+  if (n >= 256) {
     // column chunks over a cluster of CTAs (latency of the dense matrix-vector product)
+    constexpr int NR = 64 / sizeof(T);    // right-hand sides that share a read of the matrix
+    constexpr int WIDE = 512 / sizeof(T); // rows of a block where the matrix is large
+    const int chunk = ceil_div(n, dev::BOTTOM_SPLIT);
+    const bool multi = H->nb > 2 && (size_t)chunk * NR * sizeof(T) <= 64 * 1024;
+    const bool wide = n >= 2048;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -657,21 +673,32 @@ void bottom(ccm_handle* H, DevLevel& B, cudaStream_t s) {
     at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(ceil_div(B.nbc, 32) * dev::BOTTOM_SPLIT, H->nb);
+    cfg.gridDim = dim3(ceil_div(n, !multi && wide ? WIDE : 32) * dev::BOTTOM_SPLIT, multi ? ceil_div(H->nb, NR) : H->nb);
     cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = (size_t)chunk * (multi ? NR : 1) * sizeof(T);
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = t_pdl ? 2 : 1;
-    KL(cudaLaunchKernelEx(&cfg, dev::k_bottom_split<T>, B.nbc, (const int32_t*)B.bot_cell, (const T*)Bot<T>(B),
-                          (const T*)R<T>(B), U<T>(B), B.npad));
+    const T* r = R<T>(B);
+    T* u = U<T>(B);
+    if (multi) KL(cudaLaunchKernelEx(&cfg, dev::k_bottom_multi<T, NR>, n, ld, H->nb, cell, M, r, u, B.npad));
+    else if (wide) KL(cudaLaunchKernelEx(&cfg, dev::k_bottom_split<T, WIDE>, n, ld, cell, M, r, u, B.npad));
+    else KL(cudaLaunchKernelEx(&cfg, dev::k_bottom_split<T, 32>, n, ld, cell, M, r, u, B.npad));
     return;
   }
   int nw = 8;
-  size_t sm = std::max<size_t>(B.nbc, nw * 32) * sizeof(T);
-  KL(launch_k(dev::k_bottom<T>, dim3(ceil_div(B.nbc, 32), H->nb), nw * 32, sm, s, B.nbc, B.bot_cell, Bot<T>(B), R<T>(B),
-              U<T>(B), B.npad));
+  size_t sm = std::max<size_t>(n, nw * 32) * sizeof(T);
+  KL(launch_k(dev::k_bottom<T>, dim3(ceil_div(n, 32), H->nb), nw * 32, sm, s, n, ld, cell, M, R<T>(B), U<T>(B), B.npad));
 }
+
+template <typename T>
+void bottom(ccm_handle* H, DevLevel& B, cudaStream_t s) {
+  dense_product<T>(H, B, B.nbc, B.bot_ld, B.bot_cell, Bot<T>(B), s);
+}
+
+template <typename T> const T* DenseM(const ccm_handle* H);
+template <> const double* DenseM<double>(const ccm_handle* H) { return H->dense.m64; }
+template <> const float* DenseM<float>(const ccm_handle* H) { return H->dense.m32; }
 
 // the levels from m down to the bottom run as one launch of one thread-block cluster
 template <typename T>
@@ -690,7 +717,7 @@ void coarse_cluster(ccm_handle* H, int m, cudaStream_t s) {
     C.u[0] = sizeof(T) == 8 ? (T*)L.u64[0] : (T*)L.u32[0];
     C.u[1] = sizeof(T) == 8 ? (T*)L.u64[1] : (T*)L.u32[1];
     C.irr_cell = L.irr_cell; C.rowmap = L.rowmap; C.colf = L.ell_colf; C.par = L.ell_par; C.val = Ell<T>(L);
-    C.blk = L.blk; C.blk_off = L.blk_off; C.inv = Inv<T>(L); C.bot_cell = L.bot_cell; C.bot = Bot<T>(L);
+    C.blk = L.blk; C.blk_off = L.blk_off; C.inv = Inv<T>(L); C.bot_cell = L.bot_cell; C.bot = Bot<T>(L); C.bot_ld = L.bot_ld;
     P.cur[k] = sizeof(T) == 8 ? L.cur64 : L.cur32;
   }
   cudaLaunchConfig_t cfg{};
@@ -745,6 +772,11 @@ void vcycle(ccm_handle* H, int m, cudaStream_t s, bool prolong_first = false) {
   DevLevel& F = H->L[m];
   if (m == M) {
     bottom<T>(H, F, s);
+    return;
+  }
+  // (prolong_first starts from another iterate than 0)
+  if (m == H->dense.m && !prolong_first && DenseM<T>(H)) {
+    dense_product<T>(H, F, H->dense.n, H->dense.ld, H->dense.cell, DenseM<T>(H), s);
     return;
   }
   DevLevel& C = H->L[m + 1];
@@ -1000,6 +1032,99 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   cudaGetLastError();
 }
 
+// unknowns up to which the small levels' part of a V-cycle is applied as a dense matrix.  FP32
+// V-cycle of the star 256^2 (1.2k unknowns at 64^2): 108 -> 54 us.  At 3.7k unknowns (55 MB) a
+// single solve still gains (three ellipses 1024^2: 148 -> 137 us a V-cycle), but twelve problems
+// advanced together lose (17.9 -> 19.9 ms): their matrices no longer fit L2 side by side.
+constexpr int DENSE_MAX = 2048;
+
+// (Re)build the dense matrix of the V-cycle from the first level below the finest with at most
+// DENSE_MAX unknowns, for the handle's cycle parameters and SMO-2 blocks.  Block-Jacobi smoother
+// only, and not where the caller asked for the cluster cycle.  A rebuilt matrix keeps its place
+// (the level does not depend on either).  Synchronises the device.
+int build_dense(ccm_handle* h) {
+  ccm_handle::Dense& D = h->dense;
+  Arena& A = h->arena;
+  const int nl = (int)h->H.levels.size();
+  if (h->par.smoother != 1 || h->par.ras_passes > 1 || h->par.coarse_n > 0) return CCM_OK;
+  int m = -1;
+  std::vector<int32_t> cell;
+  for (int l = 1; l + 1 < nl && m < 0; ++l) {
+    const HostLevel& L = h->H.levels[l];
+    if (nl - 1 - l > dev::DENSE_MAXL || (long)L.nx * L.ny > 16L * DENSE_MAX) continue;
+    cell.clear();
+    for (int j = 0; j < L.ny; ++j)
+      for (int i = 0; i < L.nx; ++i)
+        if (L.cls[L.pad(i, j)] != 0) cell.push_back((int32_t)L.pad(i, j));
+    if (!cell.empty() && (int)cell.size() <= DENSE_MAX) m = l;
+  }
+  if (m < 0) return CCM_OK;
+  const int n = (int)cell.size();
+  dev::DenseArgs a{};
+  a.nlev = nl - 1 - m;
+  a.nu1 = h->par.nu1;
+  a.nu2 = h->par.nu2;
+  long off = 0;
+  for (int l = m; l < nl; ++l) {
+    DevLevel& d = h->L[l];
+    dev::DenseLevel& L = a.L[l - m];
+    L.nx = d.nx;
+    L.ny = d.ny;
+    L.pitch = d.pitch;
+    L.n2 = l + 1 < nl ? d.n2 : 0;
+    L.W = d.W;
+    L.core = h->H.levels[l].blk.size() >= 4 ? std::max(1, h->H.levels[l].blk[1] - h->H.levels[l].blk[0]) : 1;
+    L.cls = d.cls;
+    L.vol = d.vol64;
+    L.cell = d.irr_cell;
+    L.col = d.ell_col;
+    L.val = d.ell64;
+    L.blk = d.blk;
+    L.blk_off = d.blk_off;
+    L.inv = d.inv64;
+    for (long* o : {&L.u[0], &L.u[1], &L.r}) {
+      *o = off;
+      off += d.npad;
+    }
+    L.res = off;
+    off += d.n2;
+  }
+  DevLevel& B = h->L[nl - 1];
+  a.nbot = B.nbc;
+  a.bot_cell = B.bot_cell;
+  a.bot = B.bot64;
+  a.bot_ld = B.bot_ld;
+  a.n = n;
+  a.S = h->S64;
+  a.stride = (off + 15) & ~15L;
+  if (D.m < 0) {
+    D.cell = A.upload(cell);
+    D.ld = (n + 3) & ~3;
+    if (h->par.precision == CCM_FP64) D.m64 = A.alloc<double>((long)n * D.ld);
+    else D.m32 = A.alloc<float>((long)n * D.ld);
+  }
+  a.ld = D.ld;
+  a.cell = D.cell;
+  a.out64 = D.m64;
+  a.out32 = D.m32;
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
+  const int ctas = std::min(n, std::max(1, 2 * nsm));
+  if (A.err == cudaSuccess) A.err = cudaMalloc(&a.scratch, (size_t)ctas * a.stride * sizeof(double));
+  if (A.err != cudaSuccess) return A.err == cudaErrorMemoryAllocation ? CCM_ENOMEM : CCM_ECUDA;
+  cudaError_t e = cudaMemset(a.scratch, 0, (size_t)ctas * a.stride * sizeof(double));
+  if (e == cudaSuccess) {
+    if (h->cross) KL(dev::k_dense_columns<true><<<ctas, dev::DENSE_THREADS>>>(a));
+    else KL(dev::k_dense_columns<false><<<ctas, dev::DENSE_THREADS>>>(a));
+    e = cudaDeviceSynchronize();
+  }
+  cudaFree(a.scratch);
+  if (e != cudaSuccess) return CCM_ECUDA;
+  D.m = m;
+  D.n = n;
+  return CCM_OK;
+}
+
 // Device copies of a host hierarchy (every level's arrays, work space, tensor maps, streams)
 int upload_hierarchy(ccm_handle* h) {
   double w[5][5];
@@ -1075,8 +1200,13 @@ int upload_hierarchy(ccm_handle* h) {
     d.nbc = hl.nb_cells;
     if (d.nbc) {
       d.bot_cell = A.upload(hl.bot_cell);
-      d.bot64 = A.upload(hl.bot_inv);
-      std::vector<float> f(hl.bot_inv.begin(), hl.bot_inv.end());
+      // columns padded to 16 bytes (the dense product's loads)
+      d.bot_ld = (d.nbc + 3) & ~3;
+      std::vector<double> g((size_t)d.nbc * d.bot_ld, 0.0);
+      for (int c = 0; c < d.nbc; ++c)
+        std::copy_n(&hl.bot_inv[(size_t)c * d.nbc], d.nbc, &g[(size_t)c * d.bot_ld]);
+      d.bot64 = A.upload(g);
+      std::vector<float> f(g.begin(), g.end());
       d.bot32 = A.upload(f);
     }
     if (!hl.tr_ptr.empty()) {
@@ -1279,11 +1409,12 @@ int upload_hierarchy(ccm_handle* h) {
     A.release();
     return CCM_ECUDA;
   }
-  if (cudaDeviceSynchronize() != cudaSuccess) {
-    A.release();
-    return CCM_ECUDA;
-  }
-  return CCM_OK;
+  cudaFuncSetAttribute(dev::k_bottom_multi<float, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  cudaFuncSetAttribute(dev::k_bottom_multi<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  int rc = build_dense(h);
+  if (!rc && cudaDeviceSynchronize() != cudaSuccess) rc = CCM_ECUDA;
+  if (rc) A.release();
+  return rc;
 }
 
 }  // namespace
@@ -1827,6 +1958,7 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap) {
     }
     t->par.ras_block = block;
     t->par.ras_overlap = overlap;
+    if (int rc = build_dense(t)) return rc;
     t->info.device_bytes = t->arena.bytes;
   }
   return cudaDeviceSynchronize() == cudaSuccess ? CCM_OK : CCM_ECUDA;
@@ -1887,6 +2019,8 @@ int ccm_set_cycle_params(ccm_handle* h, double omega, int nu1, int nu2, int inne
       t->S64.omega_d = omega / w22;
       t->S32.omega_d = (float)(omega / w22);
     }
+    if (int rc = build_dense(t)) return rc;
+    t->info.device_bytes = t->arena.bytes;
   }
   return CCM_OK;
 }
