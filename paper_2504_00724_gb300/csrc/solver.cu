@@ -1747,6 +1747,13 @@ int ccm_apply_T(ccm_handle* h, const double* v, double* out_u, double* out_g, in
   return CCM_OK;
 }
 
+// the first level-0 FP32 sweep of a correction starts from zero without reading it, so nothing
+// clears the iterate
+static bool zero_start(const ccm_handle* h) {
+  return h->L[0].smooth_ok[1] && h->persistent && h->par.smoother == 1 && h->par.ras_passes <= 1 && h->par.nu1 >= 1 &&
+         h->par.cycle == 0;
+}
+
 // The correction of one mixed outer iteration by GMRES(m) on L e = r32 with the inner FP32
 // V-cycles as right preconditioner (see krylov.cuh); u_hat += e.  Level-0 FP32 vectors only,
 // scalars in device memory, no host synchronisation.
@@ -1758,48 +1765,46 @@ static void krylov_correction(ccm_handle* h, cudaStream_t s) {
   for (int i = 0; i <= m; ++i) V.v[i] = h->kv[i];
   for (int i = 0; i < m; ++i) Z.v[i] = h->kz[i];
   R.v[0] = L.r32;
-  const int KT = dev::KRY_THREADS, KG = dev::KRY_GRID;
+  const int KT = dev::KRY_THREADS, KG = std::max(1, std::min(dev::KRY_GRID, ceil_div(nt, dev::KRY_TILES)));
+  const int KGV = std::max(1, std::min(dev::KRY_GRID_V, ceil_div(nt, dev::KRY_TILES)));
+  const int nrow = ceil_div(L.n2, KT);
   const int32_t* tl = L.tiles;
   const uint8_t* cl = L.cls;
-  cudaMemsetAsync(reinterpret_cast<char*>(S) + offsetof(dev::KryScalars, H), 0, sizeof(S->H), s);
   // beta = ||r||_2, v_0 = r / beta, which is also the first preconditioner input
-  KL(launch_k(dev::k_kdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, (const float*)L.r32, R, 1, S));
-  KL(launch_k(dev::k_kreduce, 1, KT, 0, s, 1, 2, 0, m, S));
-  KL(launch_k(dev::k_kscale, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, (const float*)L.r32, h->kv[0], L.r32,
+  KL(launch_k(dev::k_kdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, (const float*)L.r32, R, 1, dev::KryStep{2, 0, m, 0}, S));
+  KL(launch_k(dev::k_kscale, KGV, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, (const float*)L.r32, h->kv[0], L.r32,
               (const dev::KryScalars*)S));
+  const bool zero_first = zero_start(h);
   for (int j = 0; j < m; ++j) {
     // z_j = M v_j: the inner cycles from a zero guess on the right-hand side r32 = v_j
-    cudaMemsetAsync(L.u32[L.cur32], 0, L.npad * sizeof(float), s);
+    if (!zero_first) cudaMemsetAsync(L.u32[L.cur32], 0, L.npad * sizeof(float), s);
     for (int c = 0; c < std::max(1, h->par.inner_cycles); ++c) {
       ProfScope ps(h, CCM_PROF_VCYCLE, s);
+      h->zero_u_next = c == 0 && zero_first;
       if (c == 0 && h->par.cycle == 1) fmg<float>(h, s);
       else vcycle<float>(h, 0, s);
+      h->zero_u_next = false;
     }
     const float* z = L.u32[L.cur32];
     float* w = h->kv[j + 1];
-    // w = L z (regular stencil, then the fitted rows), z kept as z_j
+    // w = L z (regular stencil and fitted rows), z kept as z_j
     if (h->cross)
-      KL(launch_k(dev::k_kapply<true>, nt, KT, 0, s, tl, L.nx, L.ny, L.pitch, cl, z, w, h->kz[j], h->S32));
+      KL(launch_k(dev::k_kapply<true>, nrow + nt, KT, 0, s, tl, L.nx, L.ny, L.pitch, cl, z, w, h->kz[j], h->S32, nrow, L.n2,
+                  L.W, (const int32_t*)L.irr_cell, (const int32_t*)L.ell_col, (const float*)L.ell32));
     else
-      KL(launch_k(dev::k_kapply<false>, nt, KT, 0, s, tl, L.nx, L.ny, L.pitch, cl, z, w, h->kz[j], h->S32));
-    if (L.n2)
-      KL(launch_k(dev::k_rows<float, float, false, true>, ceil_div(L.n2, 128), 128, 0, s, L.n2, L.W,
-                  (const int32_t*)L.irr_cell, (const int32_t*)L.ell_col, (const float*)L.ell32, z, (const float*)nullptr, w,
-                  (const double*)nullptr, (const int32_t*)nullptr, (const double*)nullptr));
+      KL(launch_k(dev::k_kapply<false>, nrow + nt, KT, 0, s, tl, L.nx, L.ny, L.pitch, cl, z, w, h->kz[j], h->S32, nrow, L.n2,
+                  L.W, (const int32_t*)L.irr_cell, (const int32_t*)L.ell_col, (const float*)L.ell32));
     // classical Gram-Schmidt against v_0 .. v_j twice, each subtraction fused with the next
-    // reduction: the second pass's dot products, then ||w||^2
-    KL(launch_k(dev::k_kdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, (const float*)w, V, j + 1, S));
-    KL(launch_k(dev::k_kreduce, 1, KT, 0, s, j + 1, 0, j, m, S));
-    KL(launch_k(dev::k_ksubdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, w, V, j + 1, false, S));
-    KL(launch_k(dev::k_kreduce, 1, KT, 0, s, j + 1, 0, j, m, S));
-    KL(launch_k(dev::k_ksubdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, w, V, j + 1, true, S));
-    // h_{j+1,j} = ||w||, v_{j+1} = w / h_{j+1,j} (and the next preconditioner input)
-    KL(launch_k(dev::k_kreduce, 1, KT, 0, s, 1, 1, j, m, S));
-    KL(launch_k(dev::k_kscale, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, (const float*)w, w,
-                j + 1 < m ? L.r32 : (float*)nullptr, (const dev::KryScalars*)S));
+    // reduction: the second pass's dot products, then ||w||^2 and h_{j+1,j} = ||w||
+    KL(launch_k(dev::k_kdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, (const float*)w, V, j + 1, dev::KryStep{0, j, m, 1}, S));
+    KL(launch_k(dev::k_ksubdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, w, V, j + 1, false, dev::KryStep{0, j, m, 0}, S));
+    KL(launch_k(dev::k_ksubdot, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, w, V, j + 1, true, dev::KryStep{1, j, m, 0}, S));
+    // v_{j+1} = w / h_{j+1,j}, the next preconditioner input (the last one is not used)
+    if (j + 1 < m)
+      KL(launch_k(dev::k_kscale, KGV, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, (const float*)w, w, L.r32,
+                  (const dev::KryScalars*)S));
   }
-  KL(launch_k(dev::k_klsq, 1, 32, 0, s, m, S));
-  KL(launch_k(dev::k_kupdate, KG, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, Z, m, (const dev::KryScalars*)S, h->uhat));
+  KL(launch_k(dev::k_kupdate, KGV, KT, 0, s, tl, nt, L.nx, L.ny, L.pitch, cl, Z, m, (const dev::KryScalars*)S, h->uhat));
 }
 
 // One outer iteration on the stream (also the body captured into the iteration graph):
@@ -1836,7 +1841,7 @@ static void iteration_body(ccm_handle* h, bool fp64, cudaStream_t s, bool to_hos
     // without reading it (no clearing pass), and the last one adds its new values to u_hat
     // (no separate update pass)
     const bool persistent0 = L.smooth_ok[1] && h->persistent && h->par.smoother == 1 && h->par.ras_passes <= 1;
-    const bool zero_first = persistent0 && h->par.nu1 >= 1 && h->par.cycle == 0;
+    const bool zero_first = zero_start(h);
     if (!zero_first) cudaMemsetAsync(L.u32[L.cur32], 0, h->nb * np * sizeof(float), s);
     const int ncyc = std::max(1, h->par.inner_cycles);
     h->folded = false;
