@@ -51,6 +51,8 @@ template <typename T> struct Pair;
 template <> struct Pair<float> { using type = float2; };
 template <> struct Pair<double> { using type = double2; };
 
+__device__ __forceinline__ float2 pair(float a) { return make_float2(a, a); }
+
 // w[0..5] = row[0..5] as three aligned pair loads (row at an even element offset)
 template <typename T>
 __device__ __forceinline__ void load_six(const T* row, T (&w)[6]) {
@@ -137,57 +139,89 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
   nc = a.blk[4 * b + 1] - cs;
   es = a.blk[4 * b + 2];
   ne = a.blk[4 * b + 3] - es;
-  for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-    const int row = es + e;
-    const int q = a.cell[row];
-    if (!PRO && a.zero_u) {   // the old iterate is 0: the residual is r
+  if (!PRO && a.zero_u) {   // the old iterate is 0: the residual is r
+    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+      const int q = a.cell[es + e];
       sres[e] = rhs[q];
       sold[e] = (T)0;
       scell[e] = q;
-      continue;
     }
+    return;
+  }
+  // Two threads a row (a block has at most 256 / 2 rows at the default shape), each every other
+  // one of its coefficients.  The gathers' round trips are the launch's critical path on small
+  // levels, so each thread has up to eight in flight and none hangs on a branch: a column without a
+  // coarse parent reads cell 0, which lies in the zero ring, and adds nothing.
+  const int part = threadIdx.x & 1;
+  for (int e0 = 0; e0 < ne; e0 += blockDim.x / 2) {
+    const int e = e0 + (int)(threadIdx.x >> 1);
+    const bool on = e < ne;
+    const int row = es + (on ? e : 0);
+    const int q = a.cell[row];
     T acc = 0;
-#pragma unroll 15
-    for (int m = 0; m < a.W; ++m) {
-      const int cq = a.col[(long)m * a.n2 + row];
-      T v = CG ? __ldcg(u_old + cq) : u_old[cq];
-      if (PRO) {
-        const int pq = a.par[(long)m * a.n2 + row];
-        if (pq >= 0) v += ucs[pq];
+    for (int m0 = part; m0 < a.W; m0 += 16) {
+      int cq[8], pq[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const long o = (long)min(m0 + 2 * k, a.W - 1) * a.n2 + row;
+        cq[k] = a.col[o];
+        pq[k] = PRO ? a.par[o] : 0;
       }
-      acc += a.val[(long)m * a.n2 + row] * v;
+      T v[8], c[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = CG ? __ldcg(u_old + cq[k]) : u_old[cq[k]];
+        c[k] = PRO ? ucs[max(pq[k], 0)] : (T)0;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int m = m0 + 2 * k;
+        if (PRO && pq[k] >= 0) v[k] += c[k];
+        if (m < a.W) acc += a.val[(long)m * a.n2 + row] * v[k];
+      }
     }
-    sres[e] = rhs[q] - acc;
-    sold[e] = CG ? __ldcg(u_old + q) : u_old[q];
-    scell[e] = q;
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (on && part == 0) {
+      sres[e] = rhs[q] - acc;
+      sold[e] = CG ? __ldcg(u_old + q) : u_old[q];
+      scell[e] = q;
+    }
   }
 }
 
-// u_new = u_old + inv(L22[ext, ext]) sres on the block's core cells; As = the staged rows
-// [ne][nc] of the inverse, columns over lanes, extended rows over warps; the core cells and
-// their old values from scell and sold (no global round trip before the stores)
-template <typename T>
-__device__ __forceinline__ void block_apply(const T* As, const T* sres, const T* sold, const int* scell, int c0,
-                                            int nc, int ne, T* __restrict__ u_new, double* __restrict__ uhat,
-                                            T (*part)[32]) {
+// FP32: u_new = u_old + inv(L22[ext, ext]) sres on the block's core cells; As = the staged rows
+// [ne][nc] of the inverse, two columns a lane, extended rows over warps (two barriers for a
+// block of 64 core rows); the core cells and their old values from scell and sold (no global
+// round trip before the stores)
+__device__ __forceinline__ void block_apply(const float* As, const float* sres, const float* sold, const int* scell, int c0,
+                                            int nc, int ne, float* __restrict__ u_new, double* __restrict__ uhat,
+                                            float (*part)[64]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int cb = 0; cb < nc; cb += 32) {
-    const int c = cb + lane;
-    T acc = 0;
-    if (c < nc)
-      for (int e = warp; e < ne; e += 8) acc += As[e * nc + c] * sres[e];
-    part[warp][lane] = acc;
+  for (int cb = 0; cb < nc; cb += 64) {
+    if (cb) __syncthreads();      // part is free
+    const int c = cb + 2 * lane;
+    float2 acc = make_float2(0.0f, 0.0f);
+    if (c + 1 < nc && !(nc & 1)) {
+#pragma unroll 4
+      for (int e = warp; e < ne; e += 8) acc = __ffma2_rn(*reinterpret_cast<const float2*>(As + e * nc + c), pair(sres[e]), acc);
+    } else if (c < nc) {          // an odd number of columns: the rows' pairs are not aligned
+      for (int e = warp; e < ne; e += 8) {
+        acc.x += As[e * nc + c] * sres[e];
+        if (c + 1 < nc) acc.y += As[e * nc + c + 1] * sres[e];
+      }
+    }
+    *reinterpret_cast<float2*>(&part[warp][2 * lane]) = acc;
     __syncthreads();
-    if (warp == 0 && c < nc) {
-      T tot = 0;
+    const int t = cb + (int)threadIdx.x;
+    if (threadIdx.x < 64 && t < nc) {
+      float tot = 0;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) tot += part[w][lane];
-      const int q = scell[c0 + c];
-      const T v = sold[c0 + c] + tot;
+      for (int w = 0; w < 8; ++w) tot += part[w][threadIdx.x];
+      const int q = scell[c0 + t];
+      const float v = sold[c0 + t] + tot;
       u_new[q] = v;
       if (uhat) uhat[q] += (double)v;
     }
-    __syncthreads();
   }
 }
 
@@ -266,6 +300,51 @@ __device__ __forceinline__ void tile_stencil64(double* tile, unsigned* wmax, int
   if (on) q_rows<CROSS, HX>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
 }
 
+// FP32: h^2 L u at the cells (x0, y0 + k) and (x0 + 1, y0 + k), k = 0 .. 3, of a staged tile.
+// Issue slots bound this loop, so the two cells go through packed operations (two FMA an issue slot)
+// and the mixed term is factored: the x-derivative of each of the eight rows once (its weights 1
+// and 8 are exact) and four operations a cell, in place of 16 FMA a cell.  The nine taps of the
+// two second derivatives keep the order of a plain sum; odd taps would need the pairs at odd
+// columns and stay scalar.  Error against 64-bit sums, rms over smooth and rough fields: 0.52 to
+// 0.95 of the 25-tap FMA chain's, equal to it without the mixed term.
+// emit(k, Lu, u) with both cells' values.
+template <bool CROSS, class Emit>
+__device__ __forceinline__ void stencil32(const float* __restrict__ tile, int x0, int y0, const Stencil<float>& S,
+                                          Emit emit) {
+  float2 u[8], d[8], e[8], f[8];    // of a row: the cells' pair, its x-derivatives times 12, the pairs left and right of it
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    float w[6];
+    load_six(tile + (y0 + q) * HX + x0, w);
+    u[q] = make_float2(w[2], w[3]);
+    e[q] = make_float2(w[0], w[1]);
+    f[q] = make_float2(w[4], w[5]);
+    if (CROSS)
+      d[q] = __ffma2_rn(pair(8.0f), make_float2(w[3] - w[1], w[4] - w[2]), __ffma2_rn(pair(-1.0f), f[q], e[q]));
+    if (q < 4) continue;
+    const int k = q - 4, c = k + 2;
+    float2 s;
+    if (CROSS) {
+      const float2 g = __ffma2_rn(pair(8.0f), __ffma2_rn(pair(-1.0f), d[c - 1], d[c + 1]),
+                                  __ffma2_rn(pair(-1.0f), d[c + 2], d[c - 2]));
+      s = __ffma2_rn(pair(S.w[2]), u[c - 2], __fmul2_rn(pair(S.w[0]), g));
+    } else {
+      s = __fmul2_rn(pair(S.w[2]), u[c - 2]);
+    }
+    s = __ffma2_rn(pair(S.w[7]), u[c - 1], s);
+    s = __ffma2_rn(pair(S.w[10]), e[c], s);
+    s.x = fmaf(S.w[11], e[c].y, s.x);
+    s.y = fmaf(S.w[11], u[c].x, s.y);
+    s = __ffma2_rn(pair(S.w[12]), u[c], s);
+    s.x = fmaf(S.w[13], u[c].y, s.x);
+    s.y = fmaf(S.w[13], f[c].x, s.y);
+    s = __ffma2_rn(pair(S.w[14]), f[c], s);
+    s = __ffma2_rn(pair(S.w[17]), u[c + 1], s);
+    s = __ffma2_rn(pair(S.w[22]), u[c + 2], s);
+    emit(k, s, u[c]);
+  }
+}
+
 // SMO-1 on the regular cells of a staged 64 x 32 tile (halo box of u, box of r and class bytes
 // at the TileStage offsets of st; with PRO the coarse box too, whose parent values are first
 // added to the staged regular cells: the sweep then reads u + P uc)
@@ -332,65 +411,57 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
       put(kk, u.x + a.S.omega_d * (r2.x - s0), u.y + a.S.omega_d * (r2.y - s1));
     });
   } else {
-    // FP32: two adjacent cells (x0, x0 + 1) in four rows per thread: each staged row is read
-    // as three aligned pairs (x0 - 2 .. x0 + 3) and serves both cells' stencils, and the
-    // class bytes, right-hand sides and new values move in pairs
-    using V2 = typename Pair<T>::type;
+    // FP32: two adjacent cells (x0, x0 + 1) in four rows per thread; class bytes, right-hand sides
+    // and new values move in pairs.  A thread whose eight cells are all regular (most are) stores
+    // without looking at them one by one.
     const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
-    const int i0 = cx0 + x0;
-    // the new values of row kk's pair: into u_new, and added to u_hat when the sweep folds in
-    // the outer iteration's update
-    auto put = [&](int kk, T v0, T v1, uint32_t c2) {
-      const bool g0 = (c2 & 0xffu) == 1u, g1 = (c2 >> 8) == 1u && i0 + 1 < a.nx;
-      const long p = (long)(cy0 + y0 + kk + 2) * a.pitch + (i0 + 2);
-      if (g0 && g1) {
-        V2 o;
-        o.x = v0;
-        o.y = v1;
-        *reinterpret_cast<V2*>(u_new + p) = o;
-      } else {
-        if (g0) u_new[p] = v0;
-        if (g1) u_new[p + 1] = v1;
-      }
-      if (uhat) {
-        if (g0) uhat[p] += (double)v0;
-        if (g1) uhat[p + 1] += (double)v1;
-      }
-    };
+    const uint8_t* cp = ct + (y0 + 2) * CLX + x0 + 2;
+    uint32_t c2[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c2[k] = *reinterpret_cast<const uint16_t*>(cp + k * CLX);
+    const uint32_t all = c2[0] & c2[1] & c2[2] & c2[3];     // class bytes are 0 (empty, and outside the grid), 1, 2
+    const float* rp = rt + y0 * HX + x0 + 2;
+    float2 v[4];
     if (!PRO && a.zero_u) {
       // the old iterate is 0 (its tile was not copied): u_new = omega_d r on the regular cells
-      if (i0 < a.nx)
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y0 + kk + 2) * CLX + x0 + 2);
-          const V2 r2 = *reinterpret_cast<const V2*>(rt + (y0 + kk) * HX + x0 + 2);
-          put(kk, a.S.omega_d * r2.x, a.S.omega_d * r2.y, c2);
-        }
-      return;
+      for (int k = 0; k < 4; ++k) {
+        const float2 r2 = *reinterpret_cast<const float2*>(rp + k * HX);
+        v[k] = make_float2(a.S.omega_d * r2.x, a.S.omega_d * r2.y);
+      }
+    } else {
+      stencil32<CROSS>(tile, x0, y0, a.S, [&](int k, float2 s, float2 u) {
+        const float2 r2 = *reinterpret_cast<const float2*>(rp + k * HX);
+        v[k] = __ffma2_rn(pair(a.S.omega_d), __ffma2_rn(pair(-1.0f), s, r2), u);
+      });
     }
-    if (i0 < a.nx) {
-      T w[5][6];
+    // into u_new, and added to u_hat where the sweep folds in the outer iteration's update
+    const long p = (long)(cy0 + y0 + 2) * a.pitch + (cx0 + x0 + 2);
+    T* o = u_new + p;
+    double* h = uhat ? uhat + p : nullptr;
+    if (all == 0x0101u) {
+      double2 w[4];
+      if (h)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) load_six(tile + (y0 + q) * HX + x0, w[q]);
+        for (int k = 0; k < 4; ++k) w[k] = *reinterpret_cast<const double2*>(h + (long)k * a.pitch);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        load_six(tile + (y0 + kk + 4) * HX + x0, w[4]);
-        T acc0 = 0, acc1 = 0;
+      for (int k = 0; k < 4; ++k) *reinterpret_cast<float2*>(o + (long)k * a.pitch) = v[k];
+      if (h)
 #pragma unroll
-        for (int q = 0; q < 5; ++q)
+        for (int k = 0; k < 4; ++k)
+          *reinterpret_cast<double2*>(h + (long)k * a.pitch) = make_double2(w[k].x + (double)v[k].x, w[k].y + (double)v[k].y);
+    } else {
 #pragma unroll
-          for (int b = 0; b < 5; ++b) {
-            if (!CROSS && q != 2 && b != 2) continue;
-            acc0 += a.S.w[q * 5 + b] * w[q][b];
-            acc1 += a.S.w[q * 5 + b] * w[q][b + 1];
-          }
-        const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y0 + kk + 2) * CLX + x0 + 2);
-        const V2 r2 = *reinterpret_cast<const V2*>(rt + (y0 + kk) * HX + x0 + 2);
-        put(kk, w[2][2] + a.S.omega_d * (r2.x - acc0), w[2][3] + a.S.omega_d * (r2.y - acc1), c2);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int b = 0; b < 6; ++b) w[q][b] = w[q + 1][b];
+      for (int k = 0; k < 4; ++k) {
+        const long q = (long)k * a.pitch;
+        if ((c2[k] & 0xffu) == 1u) {
+          o[q] = v[k].x;
+          if (h) h[q] += (double)v[k].x;
+        }
+        if ((c2[k] >> 8) == 1u) {
+          o[q + 1] = v[k].y;
+          if (h) h[q + 1] += (double)v[k].y;
+        }
       }
     }
   }
@@ -403,7 +474,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
                                                 const __grid_constant__ CUtensorMap tuc, SmoothArgs<T> A) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
-  __shared__ T part[8][32];
+  __shared__ __align__(16) T part[8][sizeof(T) == 8 ? 32 : 64];
   __shared__ __align__(16) unsigned wmax[8];
   const SweepArgs<T>& a = A.a;
   // While the previous launch drains: pull the static fitted-row data (columns, coefficients,
@@ -485,7 +556,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
         const int e0 = half ? block_split(ne) : 0, e1 = half ? ne : block_split(ne);
         block_apply_part(As, sres, sold, scell, cs - es, nc, e0, e1, half == 1, acc, u_new, &part[0][0]);
       } else {
-        block_apply<T>(As, sres, sold, scell, cs - es, nc, ne, u_new, uhat, part);
+        block_apply(As, sres, sold, scell, cs - es, nc, ne, u_new, uhat, part);
       }
     } else {
       tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, u_new, uhat, wmax);
@@ -577,7 +648,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
                                                        const __grid_constant__ CUtensorMap tvol, RestrictArgs<T> A) {
   using S = RestrictStage<T>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(16) T res[JY][JX];      // residual of every fine cell of the tile (0 on empty cells)
+  __shared__ T res[JY][JX];      // residuals of the tile's irregular cells
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ __align__(16) unsigned wmax[8];
   const int G = gridDim.x;
@@ -641,20 +712,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
     // class bytes of this thread's two coarse cells (0 outside the coarse level), and in FP64
     // their children's volumes
     uint8_t cc[2];
-    T vv[2][4];
+    typename Pair<T>::type vv[2][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int c = threadIdx.x + h * 256;
-      const int I = cx0 / 2 + c % (JX / 2), J = cy0 / 2 + c / (JX / 2);
+      const int I = cx0 / 2 + (threadIdx.x & 31), J = cy0 / 2 + 2 * (threadIdx.x >> 5) + h;
       cc[h] = (I < A.nxc && J < A.nyc) ? A.clsc[(long)(J + 2) * A.pitchc + (I + 2)] : (uint8_t)0;
       if constexpr (!S::vbox)
         if (I < A.nxc && J < A.nyc) {
           const T* v = A.vol + (long)(2 * J + 2) * A.pitchf + (2 * I + 2);
-          const double2 va = *reinterpret_cast<const double2*>(v), vb = *reinterpret_cast<const double2*>(v + A.pitchf);
-          vv[h][0] = va.x;
-          vv[h][1] = va.y;
-          vv[h][2] = vb.x;
-          vv[h][3] = vb.y;
+          vv[h][0] = *reinterpret_cast<const double2*>(v);
+          vv[h][1] = *reinterpret_cast<const double2*>(v + A.pitchf);
         }
     }
     const bool ok = __syncthreads_and(wait_parity(&bar[sb], parity));
@@ -669,64 +736,42 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
     const T* rt = reinterpret_cast<const T*>(st + S::r_off);
     const uint8_t* ct = st + S::c_off;
     const T* vt = reinterpret_cast<const T*>(st + S::v_off);
-    if constexpr (sizeof(T) == 4) {
-      // two adjacent cells in four rows per thread, rows read as aligned pairs (as in k_smooth)
-      const int x0 = 2 * (threadIdx.x & 31), y1 = (threadIdx.x >> 5) * 4;
-      T w[5][6];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) load_six(tile + (y1 + q) * HX + x0, w[q]);
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        load_six(tile + (y1 + kk + 4) * HX + x0, w[4]);
-        T acc0 = 0, acc1 = 0;
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-#pragma unroll
-          for (int b = 0; b < 5; ++b) {
-            if (!CROSS && q != 2 && b != 2) continue;
-            acc0 += A.S.w[q * 5 + b] * w[q][b];
-            acc1 += A.S.w[q * 5 + b] * w[q][b + 1];
-          }
-        const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y1 + kk + 2) * CLX + x0 + 2);
-        const typename Pair<T>::type r2 = *reinterpret_cast<const typename Pair<T>::type*>(rt + (y1 + kk) * HX + x0 + 2);
-        const uint32_t cv0 = c2 & 0xffu, cv1 = c2 >> 8;
-        if (cv0 == 1u) res[y1 + kk][x0] = r2.x - acc0;
-        else if (cv0 == 0u) res[y1 + kk][x0] = (T)0;
-        if (cv1 == 1u) res[y1 + kk][x0 + 1] = r2.y - acc1;
-        else if (cv1 == 0u) res[y1 + kk][x0 + 1] = (T)0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int b = 0; b < 6; ++b) w[q][b] = w[q + 1][b];
+    // A thread's eight cells (two columns of four rows) are the children of two coarse cells, one
+    // above the other: their volume-weighted sums stay in registers; irregular cells' residuals
+    // come from shared memory.
+    const int x0 = 2 * (threadIdx.x & 31), y1 = (threadIdx.x >> 5) * 4;
+    using V2 = typename Pair<T>::type;
+    V2 rs[4];
+    auto resid = [&](int kk, T s0, T s1) {
+      const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y1 + kk + 2) * CLX + x0 + 2);
+      const V2 r2 = *reinterpret_cast<const V2*>(rt + (y1 + kk) * HX + x0 + 2);
+      V2 t;
+      t.x = r2.x - s0;
+      t.y = r2.y - s1;
+      if (c2 != 0x0101u) {
+        const uint32_t c0 = c2 & 0xffu, c1 = c2 >> 8;
+        if (c0 != 1u) t.x = c0 ? res[y1 + kk][x0] : (T)0;
+        if (c1 != 1u) t.y = c1 ? res[y1 + kk][x0 + 1] : (T)0;
       }
-    } else {
-      // FP64: the stencil in integer form, two columns and four rows per thread (as in k_smooth)
-      const int x0 = 2 * (threadIdx.x & 31), y1 = (threadIdx.x >> 5) * 4;
-      tile_stencil64<CROSS>(tile, wmax, x0, y1, true, A.S, A.Q, [&](int kk, double s0, double s1) {
-        const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y1 + kk + 2) * CLX + x0 + 2);
-        const double2 r2 = *reinterpret_cast<const double2*>(rt + (y1 + kk) * HX + x0 + 2);
-        const uint32_t cv0 = c2 & 0xffu, cv1 = c2 >> 8;
-        if (cv0 == 1u) res[y1 + kk][x0] = r2.x - s0;
-        else if (cv0 == 0u) res[y1 + kk][x0] = 0.0;
-        if (cv1 == 1u) res[y1 + kk][x0 + 1] = r2.y - s1;
-        else if (cv1 == 0u) res[y1 + kk][x0 + 1] = 0.0;
-      });
-    }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)       // (kk may be a run-time value: rs stays in registers)
+        if (j == kk) rs[j] = t;
+    };
+    if constexpr (sizeof(T) == 4)
+      stencil32<CROSS>(tile, x0, y1, A.S, [&](int kk, float2 s, float2) { resid(kk, s.x, s.y); });
+    else
+      tile_stencil64<CROSS>(tile, wmax, x0, y1, true, A.S, A.Q, resid);
     if (k + 1 < K) prefetch_tile_rows(A, n0, n1);
-    __syncthreads();
-    // 32 x 16 coarse cells, two per thread
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (cc[h] == 0) continue;
-      const int c = threadIdx.x + h * 256;
-      const int ci = c % (JX / 2), cj = c / (JX / 2);
-      const long pc = (long)(cy0 / 2 + cj + 2) * A.pitchc + (cx0 / 2 + ci + 2);
-      const T* v = vt + (2 * cj) * HX + 2 * ci + 2;
-      const T v0 = S::vbox ? v[0] : vv[h][0], v1 = S::vbox ? v[1] : vv[h][1], v2 = S::vbox ? v[HX] : vv[h][2],
-              v3 = S::vbox ? v[HX + 1] : vv[h][3];
-      const T s = v0 * res[2 * cj][2 * ci] + v1 * res[2 * cj][2 * ci + 1] + v2 * res[2 * cj + 1][2 * ci] +
-                  v3 * res[2 * cj + 1][2 * ci + 1];
-      const T sv = v0 + v1 + v2 + v3;
+      const long pc = (long)(cy0 / 2 + y1 / 2 + h + 2) * A.pitchc + (cx0 / 2 + x0 / 2 + 2);
+      const T* v = vt + (y1 + 2 * h) * HX + x0 + 2;
+      const V2 va = S::vbox ? *reinterpret_cast<const V2*>(v) : vv[h][0];
+      const V2 vb = S::vbox ? *reinterpret_cast<const V2*>(v + HX) : vv[h][1];
+      const V2 ra = rs[2 * h], rb = rs[2 * h + 1];
+      const T s = va.x * ra.x + va.y * ra.y + vb.x * rb.x + vb.y * rb.y;
+      const T sv = va.x + va.y + vb.x + vb.y;
       rcz[pc] = sv > (T)0 ? (T)4 * s / sv : (T)0;
       ucz[pc] = (T)0;
     }
