@@ -577,14 +577,32 @@ namespace dev {
 
 // ---- residual + restriction of a level (Alg. 2: the coarse right-hand side and a zero coarse
 // iterate) as one persistent launch over the fine 64 x 32 tiles that restriction visits.
-// A tile item's halo tile of u, its boxes of r and (FP32) of the cell volumes (68 x 32 over the
+// A tile item's halo tile of u, its boxes of r and (FP32) of the restriction weights (68 x 32 over the
 // tile's rows) and its class bytes (80 x 36) arrive by TMA in one of two stages while the
-// previous item computes.  In FP64 each thread loads the volumes of its coarse cells' children
+// previous item computes.  In FP64 each thread loads the weights of its coarse cells' children
 // into registers before the wait instead: without their box two CTAs per SM are resident, not
 // one.  The fitted rows of the tile's irregular cells (listed per tile:
 // row and position) are gathered from global memory before the wait, and so are the class
 // bytes of the coarse cells the thread restricts to; regular cells take the stencil from the
 // staged tile; then the 32 x 16 coarse cells get the volume-weighted 2 x 2 sums.
+// the weights 4 |C_k| / sum |C| of the volume-weighted sums (Sec. 4.1) over the children of every
+// coarse cell, once at set-up: two FP64 divisions a thread cost a tile of k_restrict_p 2.6 us
+__global__ void k_restrict_weights(int nxc, int nyc, int pitchf, const double* __restrict__ vol, double* __restrict__ w64,
+                                   float* __restrict__ w32) {
+  const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y;
+  if (I >= nxc || J >= nyc) return;
+  const long p = (long)(2 * J + 2) * pitchf + (2 * I + 2);
+  const double2 a = *reinterpret_cast<const double2*>(vol + p), b = *reinterpret_cast<const double2*>(vol + p + pitchf);
+  const double sv = a.x + a.y + b.x + b.y;
+  const double v[4] = {a.x, a.y, b.x, b.y};
+  for (int k = 0; k < 4; ++k) {
+    const double w = sv > 0 ? 4 * v[k] / sv : 0.0;
+    const long q = p + (k >> 1) * pitchf + (k & 1);
+    w64[q] = w;
+    w32[q] = (float)w;
+  }
+}
+
 template <typename T>
 struct RestrictArgs {
   const int32_t* tiles;
@@ -601,7 +619,7 @@ struct RestrictArgs {
   const uint8_t* clsc;
   T* rc;
   T* uc;
-  const T* vol;        // fine cell volumes
+  const T* wt;         // restriction weights of the fine cells (k_restrict_weights)
   Stencil<T> S;
   QStencil Q;
   int* err;
@@ -621,7 +639,7 @@ struct RestrictStage {
   static constexpr uint32_t c_bytes = HY * CLX;
   static constexpr uint32_t r_off = al(u_bytes);
   static constexpr uint32_t c_off = r_off + al(r_bytes);
-  static constexpr bool vbox = sizeof(T) == 4;     // the volumes arrive by TMA too
+  static constexpr bool vbox = sizeof(T) == 4;     // the weights arrive by TMA too
   static constexpr uint32_t v_off = c_off + al(c_bytes);
   static constexpr uint32_t bytes = al(v_off + (vbox ? r_bytes : 0));
   static constexpr uint32_t tx = u_bytes + (vbox ? 2 : 1) * r_bytes + c_bytes;
@@ -658,7 +676,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
   prefetch_tile_rows(A, n0, n1);
   // this CTA's right-hand side of the batch (blockIdx.y)
   const int z = blockIdx.y;
-  // tile t's copy into stage sb.  part 0: all of it; part 1: the class bytes and volumes,
+  // tile t's copy into stage sb.  part 0: all of it; part 1: the class bytes and weights,
   // which no launch writes, with the byte count of the whole tile (before the grid
   // dependency wait); part 2: the iterate and the right-hand side (after it)
   auto issue = [&](int t, int sb, int part) {
@@ -710,7 +728,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
       res[loc >> 6][loc & 63] = rf[cell] - acc;
     }
     // class bytes of this thread's two coarse cells (0 outside the coarse level), and in FP64
-    // their children's volumes
+    // their children's weights
     uint8_t cc[2];
     typename Pair<T>::type vv[2][2];
 #pragma unroll
@@ -719,7 +737,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
       cc[h] = (I < A.nxc && J < A.nyc) ? A.clsc[(long)(J + 2) * A.pitchc + (I + 2)] : (uint8_t)0;
       if constexpr (!S::vbox)
         if (I < A.nxc && J < A.nyc) {
-          const T* v = A.vol + (long)(2 * J + 2) * A.pitchf + (2 * I + 2);
+          const T* v = A.wt + (long)(2 * J + 2) * A.pitchf + (2 * I + 2);
           vv[h][0] = *reinterpret_cast<const double2*>(v);
           vv[h][1] = *reinterpret_cast<const double2*>(v + A.pitchf);
         }
@@ -770,9 +788,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
       const V2 va = S::vbox ? *reinterpret_cast<const V2*>(v) : vv[h][0];
       const V2 vb = S::vbox ? *reinterpret_cast<const V2*>(v + HX) : vv[h][1];
       const V2 ra = rs[2 * h], rb = rs[2 * h + 1];
-      const T s = va.x * ra.x + va.y * ra.y + vb.x * rb.x + vb.y * rb.y;
-      const T sv = va.x + va.y + vb.x + vb.y;
-      rcz[pc] = sv > (T)0 ? (T)4 * s / sv : (T)0;
+      rcz[pc] = va.x * ra.x + va.y * ra.y + vb.x * rb.x + vb.y * rb.y;
       ucz[pc] = (T)0;
     }
     __syncthreads();      // res and stage sb are free

@@ -53,7 +53,9 @@ struct DevLevel {
   size_t smooth_smem[2] = {0, 0};
   int smooth_grid[2] = {0, 0};
   int smooth_cap[2] = {0, 0};   // resident CTAs of the persistent sweep over the whole GPU
-  CUtensorMap tmv64, tmv32;     // 68 x 32 boxes over the cell volumes
+  double* rw64 = nullptr;       // restriction weights of the cells (levels with k_restrict_p)
+  float* rw32 = nullptr;
+  CUtensorMap tmv64, tmv32;     // 68 x 32 boxes over them
   bool restrict_ok[2] = {false, false};  // persistent restriction (k_restrict_p), [0] FP64, [1] FP32
   uint32_t restrict_stage[2] = {0, 0};
   int restrict_grid[2] = {0, 0};
@@ -592,7 +594,7 @@ void restrict_to(ccm_handle* H, DevLevel& F, DevLevel& C, cudaStream_t s) {
     A.clsc = C.cls;
     A.rc = R<T>(C);
     A.uc = U<T>(C);
-    A.vol = Vol<T>(F);
+    A.wt = sizeof(T) == 8 ? (const T*)F.rw64 : (const T*)F.rw32;
     A.S = stencil<T>(H);
     A.Q = H->Q;
     A.err = H->derr;
@@ -1236,8 +1238,6 @@ int upload_hierarchy(ccm_handle* h) {
       d.tma = make_tmap(&d.tm64[b], d.u64[b], d.pitch, d.rows, true, 1) &&
               make_tmap(&d.tm32[b], d.u32[b], d.pitch, d.rows, false, h->B);
     d.tma = d.tma && make_tmap(&d.tmcls, d.cls, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, dev::CLX, dev::HY) &&
-            make_tmap(&d.tmv64, d.vol64, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY) &&
-            make_tmap(&d.tmv32, d.vol32, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::HX, dev::JY) &&
             make_tmap(&d.tmr64, d.r64, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY, 1) &&
             make_tmap(&d.tmr32, d.r32, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::HX, dev::JY, h->B);
   }
@@ -1334,8 +1334,18 @@ int upload_hierarchy(ccm_handle* h) {
         d.tma_pro = make_tmap(&d.tmuc64[b], c.u64[b], c.pitch, c.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::UCX, dev::UCY, 1) &&
                     make_tmap(&d.tmuc32[b], c.u32[b], c.pitch, c.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::UCX, dev::UCY,
                               h->B);
-      // the persistent restriction: two stages of u, r, class bytes and volumes per tile
-      for (int k = 0; k < 2 && d.ntiles64r > 0; ++k) {
+      // the persistent restriction: two stages of u, r, class bytes and weights per tile
+      bool maps = d.ntiles64r > 0;
+      if (maps) {
+        d.rw64 = A.alloc<double>(d.npad);
+        d.rw32 = A.alloc<float>(d.npad);
+        if (A.err == cudaSuccess)
+          KL(dev::k_restrict_weights<<<dim3(ceil_div(hc.nx, 128), hc.ny), 128>>>(hc.nx, hc.ny, d.pitch, d.vol64, d.rw64, d.rw32));
+        maps = A.err == cudaSuccess &&
+               make_tmap(&d.tmv64, d.rw64, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY) &&
+               make_tmap(&d.tmv32, d.rw32, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::HX, dev::JY);
+      }
+      for (int k = 0; k < 2 && maps; ++k) {
         const uint32_t stage = k == 0 ? dev::RestrictStage<double>::bytes : dev::RestrictStage<float>::bytes;
         const size_t smem = 2 * (size_t)stage;
         int occ = 0;
