@@ -281,6 +281,12 @@ int ccm_apply_T(ccm_handle* h, const double* v, double* out_u, double* out_g, in
 int ccm_solve(ccm_handle* h, const double* f, const double* g, double* u, int nrhs,
               void* stream, ccm_stats* stats);
 
+/* ccm_solve from the zero initial guess: u is written only (uninitialised memory is fine), and
+ * the initial residual is r_hat itself, so neither the guess nor L of it is read or computed.
+ * Where a solve ends with CCM_ETIMEOUT, right-hand sides that it did not reach are set to 0. */
+int ccm_solve_zero(ccm_handle* h, const double* f, const double* g, double* u, int nrhs,
+                   void* stream, ccm_stats* stats);
+
 /* ccm_solve with HOST arrays: f [nrhs][ny][nx], g [nrhs][n_segments] (may be NULL) and u
  * [nrhs][ny][nx] (in: initial guess, out: solution) in host memory, same layouts.  Pinned host
  * memory (cudaHostAlloc, cudaHostRegister, a pinned torch tensor) is read and written by the
@@ -319,6 +325,9 @@ int ccm_solve_host(ccm_handle* h, const double* f, const double* g, double* u, i
 int ccm_group_create(ccm_handle* const* members, int count, void* stream, ccm_group** out);
 int ccm_group_solve(ccm_group* g, const double* const* f, const double* const* gb, double* const* u,
                     void* stream, ccm_stats* stats);
+/* ccm_group_solve from the guesses u0 (u0 or u0[k] NULL: zero), the solutions into u. */
+int ccm_group_solve_from(ccm_group* g, const double* const* f, const double* const* gb, const double* const* u0,
+                         double* const* u, void* stream, ccm_stats* stats);
 int ccm_group_query(const ccm_group* g, int* members, int* programmatic);
 void ccm_group_free(ccm_group* g);
 
@@ -331,6 +340,9 @@ void ccm_group_free(ccm_group* g);
  * dJ/df = lambda, dJ/dg = -N^T lambda (ccm_apply_T of lambda). */
 int ccm_solve_T(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void* stream,
                 ccm_stats* stats);
+/* ccm_solve_T from the zero initial guess (lambda is written only). */
+int ccm_solve_T_zero(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void* stream,
+                     ccm_stats* stats);
 
 /* ---- level components of the V-cycle (one call = one step of the path, for testing and
  *      composition).  Level arrays use the user layout of that level: [ny_m][nx_m] FP64

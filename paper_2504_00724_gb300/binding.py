@@ -93,8 +93,10 @@ _SIGS = {
     "ccm_apply": (I, [P, P, P, P, I, P]),
     "ccm_apply_T": (I, [P, P, P, P, I, P]),
     "ccm_solve": (I, [P, P, P, P, I, P, ctypes.POINTER(ccm_stats)]),
+    "ccm_solve_zero": (I, [P, P, P, P, I, P, ctypes.POINTER(ccm_stats)]),
     "ccm_solve_host": (I, [P, P, P, P, I, P, ctypes.POINTER(ccm_stats)]),
     "ccm_solve_T": (I, [P, P, P, I, P, ctypes.POINTER(ccm_stats)]),
+    "ccm_solve_T_zero": (I, [P, P, P, I, P, ctypes.POINTER(ccm_stats)]),
     "ccm_level_apply": (I, [P, I, P, P, P]),
     "ccm_level_smooth": (I, [P, I, P, P, I, P]),
     "ccm_level_restrict": (I, [P, I, P, P, P, P]),
@@ -121,6 +123,7 @@ _SIGS = {
     "ccm_profile_read": (I, [P, ctypes.POINTER(ctypes.c_double), I64P]),
     "ccm_group_create": (I, [P, I, P, ctypes.POINTER(P)]),
     "ccm_group_solve": (I, [P, P, P, P, P, ctypes.POINTER(ccm_stats)]),
+    "ccm_group_solve_from": (I, [P, P, P, P, P, P, ctypes.POINTER(ccm_stats)]),
     "ccm_group_query": (I, [P, ctypes.POINTER(I), ctypes.POINTER(I)]),
     "ccm_group_free": (None, [P]),
 }
@@ -306,9 +309,10 @@ class Solver:
     def solve(self, f, g=None, u0=None, stream=None, check=True):
         import torch
         nrhs = f.numel() // (self.nx * self.ny)
-        u = torch.zeros_like(f) if u0 is None else u0.clone()
+        u = torch.empty_like(f) if u0 is None else u0.clone()
         st = ccm_stats()
-        rc = lib().ccm_solve(self.h, _ptr(f), _ptr(g), _ptr(u), nrhs, _stream(stream), ctypes.byref(st))
+        fn = lib().ccm_solve_zero if u0 is None else lib().ccm_solve
+        rc = fn(self.h, _ptr(f), _ptr(g), _ptr(u), nrhs, _stream(stream), ctypes.byref(st))
         if check:
             _check(rc, "ccm_solve")
         return u, st
@@ -337,9 +341,10 @@ class Solver:
         """lambda with L^T lambda = rhs (adjoint solve)."""
         import torch
         nrhs = rhs.numel() // (self.nx * self.ny)
-        lam = torch.zeros_like(rhs) if lam0 is None else lam0.clone()
+        lam = torch.empty_like(rhs) if lam0 is None else lam0.clone()
         st = ccm_stats()
-        rc = lib().ccm_solve_T(self.h, _ptr(rhs), _ptr(lam), nrhs, _stream(stream), ctypes.byref(st))
+        fn = lib().ccm_solve_T_zero if lam0 is None else lib().ccm_solve_T
+        rc = fn(self.h, _ptr(rhs), _ptr(lam), nrhs, _stream(stream), ctypes.byref(st))
         if check:
             _check(rc, "ccm_solve_T")
         return lam, st
@@ -501,12 +506,14 @@ class Group:
         guess (None: zero).  Returns (solutions, per-member ccm_stats, return code)."""
         import torch
         n = len(self.solvers)
-        us = [torch.zeros_like(f) if (us is None or us[k] is None) else us[k].clone() for k, f in enumerate(fs)]
+        zero = [us is None or us[k] is None for k in range(n)]
+        us = [torch.empty_like(f) if zero[k] else us[k].clone() for k, f in enumerate(fs)]
         fa = (P * n)(*[_ptr(f) for f in fs])
         ua = (P * n)(*[_ptr(u) for u in us])
+        u0 = (P * n)(*[None if zero[k] else _ptr(u) for k, u in enumerate(us)])
         ga = None if gs is None else (P * n)(*[_ptr(g) for g in gs])
         st = (ccm_stats * n)()
-        rc = lib().ccm_group_solve(self.g, fa, ga, ua, _stream(stream), st)
+        rc = lib().ccm_group_solve_from(self.g, fa, ga, u0, ua, _stream(stream), st)
         if check:
             _check(rc, "ccm_group_solve")
         return us, list(st), rc

@@ -1031,60 +1031,127 @@ __global__ void k_unpack(int nx, int ny, int pitch, const uint8_t* __restrict__ 
   else if (!KEEP) dst[(long)j * nx + i] = 0.0;
 }
 
-// k_pack and k_unpack over the level's active 32 x 8 tiles (every non-empty cell lies in one;
-// on a domain that covers a fraction of the box the rest of the grid is not visited).  The
-// tiled unpack writes the non-empty cells only: a caller that wants 0 on the empty cells
-// clears the destination first.
-template <typename TD, typename TS>
-__global__ void k_pack_tiles(const int32_t* __restrict__ tiles, int nx, int ny, int pitch, const uint8_t* __restrict__ cls,
-                             const TS* __restrict__ src, TD* __restrict__ dst, double scale) {
-  const int i = tiles[2 * blockIdx.x] * TX + threadIdx.x, j = tiles[2 * blockIdx.x + 1] * TY + threadIdx.y;
-  if (i >= nx || j >= ny) return;
-  const long p = (long)(j + 2) * pitch + (i + 2);
-  if (cls[p] != 0) dst[p] = (TD)(scale * (double)src[(long)j * nx + i]);
+// |v| as the bit pattern of a non-negative double, NaN mapped to +Inf: non-negative doubles
+// order like their patterns, so a max-norm runs on the integer pipe
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+  return b > 0x7ff0000000000000ULL ? 0x7ff0000000000000ULL : b;
 }
 
-template <typename TS>
-__global__ void k_unpack_tiles(const int32_t* __restrict__ tiles, int nx, int ny, int pitch,
-                               const uint8_t* __restrict__ cls, const TS* __restrict__ src, double* __restrict__ dst,
-                               double scale) {
-  const int i = tiles[2 * blockIdx.x] * TX + threadIdx.x, j = tiles[2 * blockIdx.x + 1] * TY + threadIdx.y;
-  if (i >= nx || j >= ny) return;
-  const long p = (long)(j + 2) * pitch + (i + 2);
-  if (cls[p] != 0) dst[(long)j * nx + i] = scale * (double)src[p];
-}
+// The start of a solve: on every non-empty cell r_hat = h^2 f - nb g (g may be null), the initial
+// iterate (u null: 0) and ||r_hat||; with u null also what the initial residual r_hat - L 0 gives,
+// its FP32 image (r32) and its norm (norm0).  Memory bounds it: f (and u) read once, the level-0
+// arrays written once, for all right-hand sides (blockIdx.y) in one launch.  Empty cells of
+// the padded arrays are 0 from their allocation on and are not written.
+struct LoadArgs {
+  const int32_t* tiles;      // the active 32 x 8 tiles: every non-empty cell lies in one
+  int ntiles, nx, ny, pitch;
+  const uint8_t* cls;
+  const int32_t* rowmap;     // padded cell -> fitted row
+  const double* nb;
+  const int32_t* seg;
+  int nseg;
+  const double *f, *g, *u;   // [nrhs][ny][nx], [nrhs][nseg], [nrhs][ny][nx]
+  double scale;
+  double *r, *r2, *u0;       // r_hat, a second copy (or null), the iterate
+  float* r32;                // or null
+  unsigned long long *norm, *norm0;   // norm0 may be null
+  long bs;                   // batch stride of the padded arrays
+};
 
-// max |x| over the non-empty cells of the active 32 x 8 tiles (as k_absmax), CTAs striding
-// over the tiles; right-hand side blockIdx.y of a batch at stride bs
-template <typename T>
-__global__ void k_absmax_tiles(const int32_t* __restrict__ tiles, int ntiles, int nx, int ny, int pitch,
-                               const uint8_t* __restrict__ cls, const T* __restrict__ x,
-                               unsigned long long* __restrict__ out, long bs) {
-  pdl_enter();
-  x += blockIdx.y * bs;
-  out += blockIdx.y;
-  double m = 0.0;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int i = tiles[2 * t] * TX + threadIdx.x, j = tiles[2 * t + 1] * TY + threadIdx.y;
-    if (i < nx && j < ny) {
-      const long p = (long)(j + 2) * pitch + (i + 2);
-      if (cls[p] != 0) {
-        double v = fabs((double)x[p]);
-        if (!(v <= 1.7976931348623157e308)) v = __longlong_as_double(0x7ff0000000000000ULL);   // NaN -> Inf
-        m = fmax(m, v);
+__global__ void __launch_bounds__(TX* TY) k_load(LoadArgs A) {
+  constexpr int NT = 4;      // tiles a step, so that a thread has 4 cells' loads in flight
+  __shared__ unsigned long long wm[TY];
+  const int z = blockIdx.y;
+  const long nu = (long)A.nx * A.ny, bo = z * A.bs;
+  const double* f = A.f + z * nu;
+  const double* u = A.u ? A.u + z * nu : nullptr;
+  const double* g = A.g ? A.g + (long)z * A.nseg : nullptr;
+  unsigned long long m = 0;
+  for (int t0 = blockIdx.x; t0 < A.ntiles; t0 += NT * gridDim.x) {
+    long p[NT];
+    uint8_t c[NT];
+    double fv[NT], uv[NT];
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+      const int t = t0 + k * gridDim.x;
+      c[k] = 0;
+      if (t >= A.ntiles) continue;
+      const int i = A.tiles[2 * t] * TX + threadIdx.x, j = A.tiles[2 * t + 1] * TY + threadIdx.y;
+      if (i >= A.nx || j >= A.ny) continue;
+      p[k] = (long)(j + 2) * A.pitch + (i + 2);
+      c[k] = A.cls[p[k]];
+      const long q = (long)j * A.nx + i;
+      fv[k] = c[k] ? f[q] : 0.0;
+      uv[k] = c[k] && u ? u[q] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+      if (!c[k]) continue;
+      double v = A.scale * fv[k];
+      if (c[k] == 2 && g) {
+        const int row = A.rowmap[p[k]], sg = A.seg[row];
+        if (sg >= 0) v -= A.nb[row] * g[sg];
       }
+      A.r[bo + p[k]] = v;
+      if (A.r2) A.r2[bo + p[k]] = v;
+      A.u0[bo + p[k]] = uv[k];
+      if (A.r32) A.r32[bo + p[k]] = (float)v;
+      m = max(m, abs_bits(v));
     }
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (threadIdx.x == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (threadIdx.x == 0) wm[threadIdx.y] = m;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    for (int w = 1; w < TY; ++w) m = max(m, wm[w]);
+    atomicMax(A.norm + z, m);
+    if (A.norm0) atomicMax(A.norm0 + z, m);
+  }
 }
 
-// r_hat -= nb g on the rows that own a boundary segment
-__global__ void k_sub_boundary(int n2, const int32_t* __restrict__ cell, const double* __restrict__ nb,
-                               const int32_t* __restrict__ seg, const double* __restrict__ g, double* __restrict__ r) {
-  int row = blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= n2 || seg[row] < 0) return;
-  r[cell[row]] -= nb[row] * g[seg[row]];
+// The end of a solve: the iterates of all right-hand sides (blockIdx.z) into the caller's layout,
+// every cell written once (0 on empty cells), two cells of four rows a thread; vec: pairs of u
+// are aligned
+__global__ void __launch_bounds__(256) k_store(int nx, int ny, int pitch, const uint8_t* __restrict__ cls,
+                                               const double* __restrict__ src, long bs, double* __restrict__ u, int vec) {
+  const int i = 2 * (blockIdx.x * 32 + threadIdx.x), j0 = 4 * (blockIdx.y * 8 + threadIdx.y);
+  if (i >= nx) return;
+  src += blockIdx.z * bs;
+  u += blockIdx.z * (long)nx * ny;
+  uint32_t c[4];
+  double2 v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const long p = (long)(j0 + k + 2) * pitch + (i + 2);
+    c[k] = j0 + k < ny ? *reinterpret_cast<const uint16_t*>(cls + p) : 0u;
+    v[k] = make_double2(0.0, 0.0);
+    if (c[k]) v[k] = *reinterpret_cast<const double2*>(src + p);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (j0 + k >= ny) break;
+    if (!(c[k] & 0xffu)) v[k].x = 0.0;
+    if (!(c[k] >> 8)) v[k].y = 0.0;
+    double* o = u + (long)(j0 + k) * nx + i;
+    if (vec) {
+      *reinterpret_cast<double2*>(o) = v[k];
+    } else {
+      o[0] = v[k].x;
+      if (i + 1 < nx) o[1] = v[k].y;
+    }
+  }
+}
+
+// the non-empty cells alone, over the active 32 x 8 tiles (a destination across the host link),
+// for the right-hand sides blockIdx.y
+__global__ void k_unpack_tiles(const int32_t* __restrict__ tiles, int nx, int ny, int pitch,
+                               const uint8_t* __restrict__ cls, const double* __restrict__ src, long bs,
+                               double* __restrict__ dst) {
+  const int i = tiles[2 * blockIdx.x] * TX + threadIdx.x, j = tiles[2 * blockIdx.x + 1] * TY + threadIdx.y;
+  if (i >= nx || j >= ny) return;
+  const long p = (long)(j + 2) * pitch + (i + 2);
+  if (cls[p] != 0) dst[blockIdx.y * (long)nx * ny + (long)j * nx + i] = src[blockIdx.y * bs + p];
 }
 
 // max |x| over the non-empty cells (non-negative doubles order like their bit patterns)

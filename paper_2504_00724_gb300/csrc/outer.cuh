@@ -13,13 +13,6 @@
 namespace ccm {
 namespace dev {
 
-// |t| as the bit pattern of a non-negative double, NaN mapped to +Inf: non-negative doubles
-// order like their patterns, so the max-norm runs on the integer pipe
-__device__ __forceinline__ unsigned long long abs_bits(double t) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(t) & 0x7fffffffffffffffULL;
-  return b > 0x7ff0000000000000ULL ? 0x7ff0000000000000ULL : b;
-}
-
 // dynamic shared memory of k_resid (offsets are multiples of 128 bytes)
 struct ResidSmem {
   static constexpr uint32_t u_bytes = HY * HX * 8, r_bytes = JY * HX * 8, c_bytes = HY * CLX;

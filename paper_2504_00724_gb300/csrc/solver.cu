@@ -2051,32 +2051,59 @@ static bool log_enabled() {
   return on;
 }
 
-// r_hat = h^2 (f - N g) and the initial guess into slots [0, nb) of the level-0 FP64 arrays,
-// from right-hand sides [k0, k0 + nb) of the caller's arrays (g may be NULL: g = 0).  The
-// packing visits the active 32 x 8 tiles only.  ||r_hat|| of slot b goes to dnorm[B + b].
+// r_hat = h^2 (f - N g) and the initial iterate into slots [0, nb) of the level-0 FP64 arrays,
+// from right-hand sides [k0, k0 + nb) of the caller's arrays (g may be NULL: g = 0; u NULL: the
+// zero guess, for which the norms and FP32 image of the initial residual come along where the
+// outer residual kernel would give them: returns true in *resid).  ||r_hat|| of slot b goes to
+// dnorm[B + b].
 static int load_rhs(ccm_handle* h, const double* f, const double* g, const double* u, int k0, int nb, double* U0,
-                    cudaStream_t s) {
+                    bool* resid, cudaStream_t s) {
   DevLevel& L = h->L[0];
-  const long nu = (long)L.nx * L.ny, np = L.npad;
-  const dim3 tb(dev::TX, dev::TY);
-  CCM_CUDA(cudaMemsetAsync(h->rhat, 0, nb * np * sizeof(double), s));
-  CCM_CUDA(cudaMemsetAsync(U0, 0, nb * np * sizeof(double), s));
-  for (int b = 0; b < nb && L.ntiles; ++b) {
-    const long k = k0 + b;
-    KL(dev::k_pack_tiles<double, double><<<L.ntiles, tb, 0, s>>>(L.tiles, L.nx, L.ny, L.pitch, L.cls, f + k * nu,
-                                                                 h->rhat + b * np, L.h * L.h));
-    if (g && L.n2)
-      KL(dev::k_sub_boundary<<<ceil_div(L.n2, 128), 128, 0, s>>>(L.n2, L.irr_cell, L.nb, L.seg,
-                                                             g + k * h->info.n_segments, h->rhat + b * np));
-    KL(dev::k_pack_tiles<double, double><<<L.ntiles, tb, 0, s>>>(L.tiles, L.nx, L.ny, L.pitch, L.cls, u + k * nu,
-                                                                 U0 + b * np, 1.0));
-  }
-  if (h->par.precision == CCM_FP64) CCM_CUDA(cudaMemcpyAsync(L.r64, h->rhat, np * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  CCM_CUDA(cudaMemsetAsync(h->dnorm + h->B, 0, nb * sizeof(unsigned long long), s));
-  if (L.ntiles)
-    KL(launch_k(dev::k_absmax_tiles<double>, dim3(std::min(L.ntiles, 1216), nb), tb, 0, s, L.tiles, L.ntiles, L.nx, L.ny,
-                L.pitch, L.cls, (const double*)h->rhat, h->dnorm + h->B, np));
+  const long nu = (long)L.nx * L.ny;
+  const bool fp64 = h->par.precision == CCM_FP64;
+  *resid = !u && h->fused_outer;
+  CCM_CUDA(cudaMemsetAsync(h->dnorm, 0, 2 * h->B * sizeof(unsigned long long), s));
+  if (!L.ntiles) return CCM_OK;
+  dev::LoadArgs A{};
+  A.tiles = L.tiles;
+  A.ntiles = L.ntiles;
+  A.nx = L.nx;
+  A.ny = L.ny;
+  A.pitch = L.pitch;
+  A.cls = L.cls;
+  A.rowmap = L.rowmap;
+  A.nb = L.nb;
+  A.seg = L.seg;
+  A.nseg = h->info.n_segments;
+  A.f = f + k0 * nu;
+  A.g = g && L.n2 ? g + (long)k0 * A.nseg : nullptr;
+  A.u = u ? u + k0 * nu : nullptr;
+  A.scale = L.h * L.h;
+  A.r = h->rhat;
+  A.r2 = fp64 ? L.r64 : nullptr;
+  A.u0 = U0;
+  A.r32 = *resid && !fp64 ? L.r32 : nullptr;
+  A.norm = h->dnorm + h->B;
+  A.norm0 = *resid ? h->dnorm : nullptr;
+  A.bs = L.npad;
+  // one tile a CTA until the GPU is full (8 CTAs an SM), then up to four in flight in each
+  const int full = std::max(1, 1216 / nb);
+  KL(dev::k_load<<<dim3(std::min(L.ntiles, std::max(full, ceil_div(L.ntiles, 16))), nb), dim3(dev::TX, dev::TY), 0, s>>>(A));
   return CCM_OK;
+}
+
+// the iterates in slots [0, nb) of U0 into u; keep_empty: the empty cells of u keep their values
+static void store_solution(ccm_handle* h, const double* U0, double* u, int nb, bool keep_empty, cudaStream_t s) {
+  DevLevel& L = h->L[0];
+  if (keep_empty) {
+    if (L.ntiles)
+      KL(dev::k_unpack_tiles<<<dim3(L.ntiles, nb), dim3(dev::TX, dev::TY), 0, s>>>(L.tiles, L.nx, L.ny, L.pitch, L.cls, U0,
+                                                                                  L.npad, u));
+    return;
+  }
+  const int vec = (uintptr_t)u % 16 == 0 && L.nx % 2 == 0;
+  KL(dev::k_store<<<dim3(ceil_div(L.nx, 64), ceil_div(L.ny, 32), nb), dim3(32, 8), 0, s>>>(L.nx, L.ny, L.pitch, L.cls, U0,
+                                                                                          L.npad, u, vec));
 }
 
 // max |r_hat - L U0| of one right-hand side into dnorm[0] (no host synchronisation)
@@ -2098,14 +2125,14 @@ static void initial_residual(ccm_handle* h, const double* U0, cudaStream_t s) {
 
 namespace {
 
-// ccm_solve; keep_empty: the empty cells of u keep the values they had (ccm_solve_host)
-int solve_impl(ccm_handle* h, const double* f, const double* g, double* u, int nrhs, void* stream, ccm_stats* st,
-               bool keep_empty) {
+// ccm_solve from the initial guess u0 (NULL: zero; it may be u); keep_empty: the empty cells of u
+// keep the values they had (ccm_solve_host)
+int solve_impl(ccm_handle* h, const double* f, const double* g, const double* u0, double* u, int nrhs, void* stream,
+               ccm_stats* st, bool keep_empty) {
   if (!h || !f || !u || nrhs < 1) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   DevLevel& L = h->L[0];
-  const long nu = (long)L.nx * L.ny, np = L.npad;
-  dim3 pg(ceil_div(L.nx, 128), L.ny);
+  const long nu = (long)L.nx * L.ny;
   const bool fp64 = h->par.precision == CCM_FP64;
   const int bmax = fp64 ? 1 : h->bmax;
   int result = CCM_OK;
@@ -2121,14 +2148,15 @@ int solve_impl(ccm_handle* h, const double* f, const double* g, double* u, int n
     }
     ccm_handle::Graph& G = h->graph[fp64 ? 1 : 0];
     double* U0 = G.u0;
-    rc = load_rhs(h, f, g, u, k0, nb, U0, s);
+    bool resid = false;
+    rc = load_rhs(h, f, g, u0, k0, nb, U0, &resid, s);
     if (rc) {
       h->nb = 1;
       return rc;
     }
     // initial residual (one right-hand side at a time outside the fused mixed form); its norms
     // and ||r_hat|| come back in one synchronisation
-    initial_residual(h, U0, s);
+    if (!resid) initial_residual(h, U0, s);
     CCM_CUDA(cudaMemcpyAsync(h->hnorm, h->dnorm, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     CCM_CUDA(cudaMemcpyAsync(h->hnorm + h->B, h->dnorm + h->B, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     CCM_CUDA(cudaStreamSynchronize(s));
@@ -2176,13 +2204,7 @@ int solve_impl(ccm_handle* h, const double* f, const double* g, double* u, int n
     if (result == CCM_ETIMEOUT) {
     } else if (!std::isfinite(wr)) result = CCM_ENOTFINITE;
     else if (wr > h->par.rtol && result == CCM_OK) result = CCM_ENOCONV;
-    // the non-empty cells over the active tiles; without keep_empty the array is cleared first
-    for (int b = 0; b < nb; ++b) {
-      if (!keep_empty) CCM_CUDA(cudaMemsetAsync(u + (k0 + b) * nu, 0, nu * sizeof(double), s));
-      if (L.ntiles)
-        KL(dev::k_unpack_tiles<double><<<L.ntiles, dim3(dev::TX, dev::TY), 0, s>>>(L.tiles, L.nx, L.ny, L.pitch, L.cls,
-                                                                                 U0 + b * np, u + (k0 + b) * nu, 1.0));
-    }
+    store_solution(h, U0, u + k0 * nu, nb, keep_empty, s);
     local.iterations = it;
     local.rel_residual = wr;
     if (st) *st = local;
@@ -2192,7 +2214,12 @@ int solve_impl(ccm_handle* h, const double* f, const double* g, double* u, int n
       for (int j = 0; j <= std::min(it, 63); ++j)
         std::fprintf(stderr, "ccm_solve:   iteration %2d  rel. residual %.3e\n", j, local.history[j]);
     }
-    if (result == CCM_ETIMEOUT) break;
+    if (result == CCM_ETIMEOUT) {
+      // the right-hand sides not reached keep their initial guess
+      const int left = nrhs - k0 - nb;
+      if (!u0 && left > 0) CCM_CUDA(cudaMemsetAsync(u + (k0 + nb) * nu, 0, left * nu * sizeof(double), s));
+      break;
+    }
   }
   h->nb = 1;
   CCM_CUDA(cudaGetLastError());
@@ -2204,7 +2231,11 @@ int solve_impl(ccm_handle* h, const double* f, const double* g, double* u, int n
 extern "C" {
 
 int ccm_solve(ccm_handle* h, const double* f, const double* g, double* u, int nrhs, void* stream, ccm_stats* st) {
-  return solve_impl(h, f, g, u, nrhs, stream, st, false);
+  return solve_impl(h, f, g, u, u, nrhs, stream, st, false);
+}
+
+int ccm_solve_zero(ccm_handle* h, const double* f, const double* g, double* u, int nrhs, void* stream, ccm_stats* st) {
+  return solve_impl(h, f, g, nullptr, u, nrhs, stream, st, false);
 }
 
 }  // extern "C"
@@ -2389,6 +2420,11 @@ int ccm_group_create(ccm_handle* const* members, int count, void* stream, ccm_gr
 
 int ccm_group_solve(ccm_group* G, const double* const* f, const double* const* g, double* const* u, void* stream,
                     ccm_stats* st) {
+  return ccm_group_solve_from(G, f, g, u, u, stream, st);
+}
+
+int ccm_group_solve_from(ccm_group* G, const double* const* f, const double* const* g, const double* const* u0,
+                         double* const* u, void* stream, ccm_stats* st) {
   if (!G || !f || !u) return CCM_EINVAL;
   const int n = (int)G->m.size();
   for (int k = 0; k < n; ++k)
@@ -2398,10 +2434,11 @@ int ccm_group_solve(ccm_group* G, const double* const* f, const double* const* g
   for (int k = 0; k < n; ++k) {
     ccm_handle* h = G->m[k];
     h->nb = 1;
-    int rc = load_rhs(h, f[k], g ? g[k] : nullptr, u[k], 0, 1, G->u0[k], s);
+    bool resid = false;
+    int rc = load_rhs(h, f[k], g ? g[k] : nullptr, u0 ? u0[k] : nullptr, 0, 1, G->u0[k], &resid, s);
     if (rc) return rc;
     CCM_CUDA(cudaMemcpyAsync(G->rnorm + k, h->dnorm + h->B, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
-    initial_residual(h, G->u0[k], s);
+    if (!resid) initial_residual(h, G->u0[k], s);
   }
   CCM_CUDA(cudaGraphLaunch(G->exec, s));
   CCM_CUDA(cudaMemcpyAsync(G->h_iters, G->A.iters, n * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2410,10 +2447,7 @@ int ccm_group_solve(ccm_group* G, const double* const* f, const double* const* g
   CCM_CUDA(cudaMemcpyAsync(G->h_hist, G->A.hist, (long)n * dev::GROUP_HIST * sizeof(double), cudaMemcpyDeviceToHost, s));
   int result = CCM_OK;
   for (int k = 0; k < n; ++k) {
-    ccm_handle* h = G->m[k];
-    DevLevel& L = h->L[0];
-    dim3 pg(ceil_div(L.nx, 128), L.ny);
-    KL(dev::k_unpack<double><<<pg, 128, 0, s>>>(L.nx, L.ny, L.pitch, L.cls, G->u0[k], u[k], 1.0));
+    store_solution(G->m[k], G->u0[k], u[k], 1, false, s);
   }
   CCM_CUDA(cudaStreamSynchronize(s));
   long long total = 2;   // k_group_init and the last k_group_decide
@@ -2543,7 +2577,8 @@ int ccm_solve_host(ccm_handle* h, const double* f, const double* g, double* u, i
   if (!rc) rc = host_view(g, (size_t)h->info.n_segments * nrhs * sizeof(double), true, s, vg);
   if (!rc) rc = host_view(u, cells * sizeof(double), true, s, vu);
   if (!rc) {
-    rc = solve_impl(h, (const double*)vf.dev, (const double*)vg.dev, (double*)vu.dev, nrhs, stream, st, true);
+    rc = solve_impl(h, (const double*)vf.dev, (const double*)vg.dev, (const double*)vu.dev, (double*)vu.dev, nrhs, stream, st,
+                    true);
     // the solution in u (also after CCM_ENOCONV, where u holds the last iterate)
     const int rb = stage_back(vu, s);
     if (rc == CCM_OK || rc == CCM_ENOCONV) rc = rc ? rc : rb;
@@ -2555,8 +2590,8 @@ int ccm_solve_host(ccm_handle* h, const double* f, const double* g, double* u, i
   return rc;
 }
 
-int ccm_solve_T(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void* stream, ccm_stats* st) {
-  if (!h || !rhs || !lambda || nrhs < 1) return CCM_EINVAL;
+// the hierarchy of transposed operators, built on first use
+static int transposed(ccm_handle* h) {
   if (!h->adj) {
     std::unique_ptr<ccm_handle> t(new ccm_handle());
     t->par = h->par;
@@ -2579,7 +2614,19 @@ int ccm_solve_T(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void
     t->info.n_segments = 0;
     h->adj = t.release();
   }
+  return CCM_OK;
+}
+
+int ccm_solve_T(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void* stream, ccm_stats* st) {
+  if (!h || !rhs || !lambda || nrhs < 1) return CCM_EINVAL;
+  if (int rc = transposed(h)) return rc;
   return ccm_solve(h->adj, rhs, nullptr, lambda, nrhs, stream, st);
+}
+
+int ccm_solve_T_zero(ccm_handle* h, const double* rhs, double* lambda, int nrhs, void* stream, ccm_stats* st) {
+  if (!h || !rhs || !lambda || nrhs < 1) return CCM_EINVAL;
+  if (int rc = transposed(h)) return rc;
+  return ccm_solve_zero(h->adj, rhs, nullptr, lambda, nrhs, stream, st);
 }
 
 // ---- level components
