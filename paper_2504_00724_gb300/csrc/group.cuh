@@ -11,7 +11,7 @@
 // ones the single-problem solve takes on the host, per member.
 #pragma once
 
-#include <cuda_runtime.h>
+#include "kernels.cuh"
 
 namespace ccm {
 namespace dev {
@@ -90,6 +90,61 @@ __global__ void k_group_decide(GroupArgs A) {
     for (int k = 0; k < A.n; ++k) cudaGraphSetConditional(A.hk[k], (unsigned)A.act[k]);
     cudaGraphSetConditional(A.hw, (unsigned)any);
   }
+}
+
+// One problem's loop (ccm_solve): a WHILE conditional node whose body is one outer iteration and
+// k_loop_decide, so that a solve is one graph launch and the host waits once.  The worst of the
+// nb right-hand sides decides (a non-finite one first of all).
+struct LoopState {
+  int it, failed;          // outer iterations done; a bounded wait ran out
+  double rel;              // last relative residual
+  double hist[GROUP_HIST];
+};
+
+struct LoopArgs {
+  int nb, max_iter;
+  double rtol;
+  const unsigned long long* norm;    // bits of the residuals' max-norms
+  const unsigned long long* rnorm;   // bits of ||r_hat||
+  const int* err;
+  LoopState* st;
+  cudaGraphConditionalHandle hw;
+};
+
+constexpr int LOOP_THREADS = 128;
+
+template <bool INIT>
+__global__ void __launch_bounds__(LOOP_THREADS) k_loop_decide(LoopArgs A) {
+  __shared__ int bad;
+  __shared__ unsigned long long worst;
+  if (threadIdx.x == 0) {
+    bad = A.nb;
+    worst = 0;
+  }
+  __syncthreads();
+  if (!INIT) pdl_enter();
+  auto rel = [&](int k) {
+    const double r0 = bits_to_double(A.rnorm[k]);
+    return bits_to_double(A.norm[k]) / (r0 == 0.0 ? 1.0 : r0);
+  };
+  unsigned long long m = 0;
+  for (int k = threadIdx.x; k < A.nb; k += LOOP_THREADS) {
+    const double r = rel(k);
+    if (r <= 1.7976931348623157e308) m = max(m, (unsigned long long)__double_as_longlong(r));
+    else atomicMin(&bad, k);
+  }
+  atomicMax(&worst, m);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  LoopState& st = *A.st;
+  const int it = INIT ? 0 : st.it + 1;
+  const double w = bad < A.nb ? rel(bad) : bits_to_double(worst);
+  const int failed = !INIT && *A.err != 0;
+  st.it = it;
+  st.failed = failed;
+  st.rel = w;
+  if (it < GROUP_HIST && !failed) st.hist[it] = w;
+  cudaGraphSetConditional(A.hw, !failed && bad == A.nb && w > A.rtol && it < A.max_iter ? 1u : 0u);
 }
 
 }  // namespace dev

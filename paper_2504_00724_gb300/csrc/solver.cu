@@ -239,7 +239,10 @@ struct ccm_handle {
     std::vector<int> prof_pairs;      // indices into gprof_ev (pairs at 2k, 2k + 1)
     double* u0 = nullptr;             // the level-0 FP64 iterate the graph updates
     int nb = 1;                       // right-hand sides its launches cover
+    bool loop = false;                // the whole loop to the tolerance, else one outer iteration
   } graph[2];
+  dev::LoopState* loop_st = nullptr;  // of the loop graph, and its pinned copy
+  dev::LoopState* loop_h = nullptr;
 };
 
 namespace {
@@ -1410,12 +1413,14 @@ int upload_hierarchy(ccm_handle* h) {
   }
   h->dnorm = A.alloc<unsigned long long>(2 * h->B);   // [0, B) residual norms, [B, 2B) ||r_hat||
   h->derr = A.alloc<int>(1);
+  h->loop_st = A.alloc<dev::LoopState>(1);
   if (A.err != cudaSuccess) {
     A.release();
     return A.err == cudaErrorMemoryAllocation ? CCM_ENOMEM : CCM_ECUDA;
   }
   if (cudaMallocHost(&h->hnorm, 2 * h->B * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMallocHost(&h->herr, sizeof(int)) != cudaSuccess) {
+      cudaMallocHost(&h->herr, sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&h->loop_h, sizeof(dev::LoopState)) != cudaSuccess) {
     A.release();
     return CCM_ECUDA;
   }
@@ -1903,6 +1908,55 @@ static void iteration_body(ccm_handle* h, bool fp64, cudaStream_t s, bool to_hos
   cudaMemcpyAsync(h->herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, s);
 }
 
+// init { it = 0, condition }, WHILE(condition) { outer iteration; decide }.  A host that launches
+// each iteration waits for its norm first: about 12 us a time without work on the GPU.
+static bool capture_loop(ccm_handle* h, bool fp64, cudaStream_t s, ccm_handle::Graph& G) {
+  cudaGraph_t graph = nullptr, part = nullptr;
+  if (cudaGraphCreate(&graph, 0) != cudaSuccess) return false;
+  bool ok = false;
+  long long l0 = g_launches.load();
+  do {
+    dev::LoopArgs A{};
+    A.nb = h->nb;
+    A.max_iter = h->par.max_iter;
+    A.rtol = h->par.rtol;
+    A.norm = h->dnorm;
+    A.rnorm = h->dnorm + h->B;
+    A.err = h->derr;
+    A.st = h->loop_st;
+    if (cudaGraphConditionalHandleCreate(&A.hw, graph, 0, cudaGraphCondAssignDefault) != cudaSuccess) break;
+    void* kargs[] = {&A};
+    cudaKernelNodeParams kp{};
+    kp.func = (void*)dev::k_loop_decide<true>;
+    kp.gridDim = dim3(1);
+    kp.blockDim = dim3(dev::LOOP_THREADS);
+    kp.kernelParams = kargs;
+    cudaGraphNode_t init, loop;
+    if (cudaGraphAddKernelNode(&init, graph, nullptr, 0, &kp) != cudaSuccess) break;
+    cudaGraphNodeParams wp{};
+    wp.type = cudaGraphNodeTypeConditional;
+    wp.conditional.handle = A.hw;
+    wp.conditional.type = cudaGraphCondTypeWhile;
+    wp.conditional.size = 1;
+    if (cudaGraphAddNode(&loop, graph, &init, nullptr, 1, &wp) != cudaSuccess) break;
+    if (cudaStreamBeginCaptureToGraph(s, wp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+      break;
+    h->capturing = true;
+    iteration_body(h, fp64, s, false);
+    const cudaError_t e = KL(launch_k(dev::k_loop_decide<false>, 1, dev::LOOP_THREADS, 0, s, A));
+    h->capturing = false;
+    if (cudaStreamEndCapture(s, &part) != cudaSuccess || e != cudaSuccess) break;
+    ok = cudaGraphInstantiate(&G.exec, graph, 0) == cudaSuccess;
+    if (!ok) G.exec = nullptr;
+  } while (false);
+  G.launches = g_launches.load() - l0;
+  g_launches.fetch_sub(G.launches);
+  cudaGraphDestroy(graph);
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 static int capture_iteration(ccm_handle* h, bool fp64, cudaStream_t user) {
   ccm_handle::Graph& G = h->graph[fp64 ? 1 : 0];
   if (G.exec && G.nb == h->nb) return CCM_OK;
@@ -1919,23 +1973,31 @@ static int capture_iteration(ccm_handle* h, bool fp64, cudaStream_t user) {
   // sweeps per level; odd counts are handled inside the body (fp64) or by resetting the
   // level-0 FP32 buffer at the start of every replay (mixed)
   const int cur64 = h->L[0].cur64;
-  cudaGraph_t graph;
-  CCM_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  h->capturing = true;
-  size_t ev0 = h->gprof_ev.size();
-  long long l0 = g_launches.load();
-  iteration_body(h, fp64, s);
-  G.launches = g_launches.load() - l0;
-  g_launches.fetch_sub(G.launches);
-  h->capturing = false;
-  cudaError_t e = cudaStreamEndCapture(s, &graph);
-  if (e != cudaSuccess) return CCM_ECUDA;
-  for (size_t k = ev0; k < h->gprof_ev.size(); k += 2) G.prof_pairs.push_back((int)k);
-  e = cudaGraphInstantiate(&G.exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {
-    G.exec = nullptr;
-    return CCM_ECUDA;
+  G.loop = false;
+  // Profiled launches carry event nodes, which conditional bodies cannot hold; a runtime that
+  // rejects programmatic edges in them gets one launch per iteration, too
+  if (h->prof_class == 0 && capture_loop(h, fp64, s, G)) {
+    G.loop = true;
+  } else {
+    h->L[0].cur64 = cur64;
+    cudaGraph_t graph;
+    CCM_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    h->capturing = true;
+    size_t ev0 = h->gprof_ev.size();
+    long long l0 = g_launches.load();
+    iteration_body(h, fp64, s);
+    G.launches = g_launches.load() - l0;
+    g_launches.fetch_sub(G.launches);
+    h->capturing = false;
+    cudaError_t e = cudaStreamEndCapture(s, &graph);
+    if (e != cudaSuccess) return CCM_ECUDA;
+    for (size_t k = ev0; k < h->gprof_ev.size(); k += 2) G.prof_pairs.push_back((int)k);
+    e = cudaGraphInstantiate(&G.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+      G.exec = nullptr;
+      return CCM_ECUDA;
+    }
   }
   h->L[0].cur64 = cur64;
   G.u0 = fp64 ? h->L[0].u64[cur64] : h->uhat;
@@ -2157,54 +2219,71 @@ int solve_impl(ccm_handle* h, const double* f, const double* g, const double* u0
     // initial residual (one right-hand side at a time outside the fused mixed form); its norms
     // and ||r_hat|| come back in one synchronisation
     if (!resid) initial_residual(h, U0, s);
-    CCM_CUDA(cudaMemcpyAsync(h->hnorm, h->dnorm, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    CCM_CUDA(cudaMemcpyAsync(h->hnorm + h->B, h->dnorm + h->B, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    CCM_CUDA(cudaStreamSynchronize(s));
-    for (int b = 0; b < nb; ++b) {
-      std::memcpy(&rnorm[b], &h->hnorm[h->B + b], sizeof(double));
-      if (rnorm[b] == 0) rnorm[b] = 1;
-      std::memcpy(&rel[b], &h->hnorm[b], sizeof(double));
-    }
-    // the worst right-hand side of the group decides; stats report it
-    auto worst = [&]() {
-      double w = 0;
-      for (int b = 0; b < nb; ++b) {
-        const double r = rel[b] / rnorm[b];
-        if (!std::isfinite(r)) return r;
-        w = std::max(w, r);
-      }
-      return w;
-    };
-    double wr = worst();
     ccm_stats local{};
-    local.history[0] = wr;
+    double wr = 0;
     int it = 0;
-    while (std::isfinite(wr) && wr > h->par.rtol && it < h->par.max_iter) {
+    if (G.loop) {
       CCM_CUDA(cudaGraphLaunch(G.exec, s));
-      g_launches.fetch_add(G.launches);
+      CCM_CUDA(cudaMemcpyAsync(h->loop_h, h->loop_st, sizeof(dev::LoopState), cudaMemcpyDeviceToHost, s));
+      store_solution(h, U0, u + k0 * nu, nb, keep_empty, s);
       CCM_CUDA(cudaStreamSynchronize(s));
-      for (int b = 0; b < nb; ++b) std::memcpy(&rel[b], &h->hnorm[b], sizeof(double));
-      wr = worst();
-      ++it;
-      if (*h->herr) {
+      const dev::LoopState& o = *h->loop_h;
+      it = o.it;
+      wr = o.rel;
+      std::copy_n(o.hist, std::min(it - o.failed, dev::GROUP_HIST - 1) + 1, local.history);
+      g_launches.fetch_add(1 + it * G.launches);
+      if (o.failed) {
         result = CCM_ETIMEOUT;
-        *h->herr = 0;
         cudaMemsetAsync(h->derr, 0, sizeof(int), s);
-        break;
       }
-      if (it < 64) local.history[it] = wr;
-      for (int p : G.prof_pairs) {
-        float t = 0;
-        if (cudaEventElapsedTime(&t, h->gprof_ev[p], h->gprof_ev[p + 1]) == cudaSuccess) {
-          h->prof_ms += t;
-          h->prof_n += 1;
+    } else {
+      CCM_CUDA(cudaMemcpyAsync(h->hnorm, h->dnorm, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+      CCM_CUDA(cudaMemcpyAsync(h->hnorm + h->B, h->dnorm + h->B, nb * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+      CCM_CUDA(cudaStreamSynchronize(s));
+      for (int b = 0; b < nb; ++b) {
+        std::memcpy(&rnorm[b], &h->hnorm[h->B + b], sizeof(double));
+        if (rnorm[b] == 0) rnorm[b] = 1;
+        std::memcpy(&rel[b], &h->hnorm[b], sizeof(double));
+      }
+      // the worst right-hand side of the group decides; stats report it
+      auto worst = [&]() {
+        double w = 0;
+        for (int b = 0; b < nb; ++b) {
+          const double r = rel[b] / rnorm[b];
+          if (!std::isfinite(r)) return r;
+          w = std::max(w, r);
+        }
+        return w;
+      };
+      wr = worst();
+      local.history[0] = wr;
+      while (std::isfinite(wr) && wr > h->par.rtol && it < h->par.max_iter) {
+        CCM_CUDA(cudaGraphLaunch(G.exec, s));
+        g_launches.fetch_add(G.launches);
+        CCM_CUDA(cudaStreamSynchronize(s));
+        for (int b = 0; b < nb; ++b) std::memcpy(&rel[b], &h->hnorm[b], sizeof(double));
+        wr = worst();
+        ++it;
+        if (*h->herr) {
+          result = CCM_ETIMEOUT;
+          *h->herr = 0;
+          cudaMemsetAsync(h->derr, 0, sizeof(int), s);
+          break;
+        }
+        if (it < 64) local.history[it] = wr;
+        for (int p : G.prof_pairs) {
+          float t = 0;
+          if (cudaEventElapsedTime(&t, h->gprof_ev[p], h->gprof_ev[p + 1]) == cudaSuccess) {
+            h->prof_ms += t;
+            h->prof_n += 1;
+          }
         }
       }
+      store_solution(h, U0, u + k0 * nu, nb, keep_empty, s);
     }
     if (result == CCM_ETIMEOUT) {
     } else if (!std::isfinite(wr)) result = CCM_ENOTFINITE;
     else if (wr > h->par.rtol && result == CCM_OK) result = CCM_ENOCONV;
-    store_solution(h, U0, u + k0 * nu, nb, keep_empty, s);
     local.iterations = it;
     local.rel_residual = wr;
     if (st) *st = local;
@@ -2841,6 +2920,7 @@ void ccm_free(ccm_handle* h) {
   h->arena.release();
   if (h->hnorm) cudaFreeHost(h->hnorm);
   if (h->herr) cudaFreeHost(h->herr);
+  if (h->loop_h) cudaFreeHost(h->loop_h);
   delete h;
 }
 
