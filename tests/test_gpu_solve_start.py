@@ -31,9 +31,10 @@ def test_zero_guess_equals_an_array_of_zeros(name, precision, batch, nrhs):
     s = P.Solver(make(), coarsest=coarsest, precision=precision, batch=batch, max_iter=4, rtol=1e-13)
     try:
         f, g, live = inputs(s, nrhs)
+        zero = torch.zeros((), dtype=torch.float64, device="cuda")
         for gb in (g, None):
             a, sa = s.solve(f, gb, check=False)
-            b, sb = s.solve(f, gb, u0=torch.where(live, 0.0, 3.0).expand(f.shape), check=False)
+            b, sb = s.solve(f, gb, u0=torch.where(live, zero, zero + 3).expand(f.shape).contiguous(), check=False)
             assert sa.iterations == sb.iterations and list(sa.history) == list(sb.history)
             assert torch.equal(a, b) and not a[:, ~live].any() and a.abs().max() > 0
     finally:
@@ -41,7 +42,7 @@ def test_zero_guess_equals_an_array_of_zeros(name, precision, batch, nrhs):
 
 
 def test_zero_and_non_finite_right_hand_sides():
-    s = P.Solver(W.disk_minus(96), max_iter=20)
+    s = P.Solver(W.disk_minus(128), max_iter=20)
     try:
         f, g, live = inputs(s, 1)
         u, st = s.solve(torch.zeros_like(f))
