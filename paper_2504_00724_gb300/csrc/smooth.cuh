@@ -158,6 +158,7 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
     const bool on = e < ne;
     const int row = es + (on ? e : 0);
     const int q = a.cell[row];
+    const T rq = rhs[q], uq = CG ? __ldcg(u_old + q) : u_old[q];    // (with the gathers in flight)
     T acc = 0;
     for (int m0 = part; m0 < a.W; m0 += 16) {
       int cq[8], pq[8];
@@ -182,8 +183,8 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
     }
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (on && part == 0) {
-      sres[e] = rhs[q] - acc;
-      sold[e] = CG ? __ldcg(u_old + q) : u_old[q];
+      sres[e] = rq - acc;
+      sold[e] = uq;
       scell[e] = q;
     }
   }
