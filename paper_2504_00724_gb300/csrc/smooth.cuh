@@ -33,6 +33,8 @@ namespace dev {
 // that one CTA per SM is resident instead of two
 template <typename T>
 constexpr int BLOCK_PARTS = sizeof(T) == 8 ? 2 : 1;
+// right-hand sides of a batch that share block items (FP32; 256 threads update 64 core rows of 4)
+constexpr int BATCH_SHARE = 4;
 // extended rows of the first part (even: the second part's copy starts on 16 bytes)
 __host__ __device__ constexpr int block_split(int ne) { return (ne / 2 + 1) & ~1; }
 
@@ -40,7 +42,8 @@ template <typename T>
 struct SmoothArgs {
   SweepArgs<T> a;      // level arrays, stencil, iterates, blocks (chunks == 1)
   int nbi;             // block items (= a.nblk)
-  int nitems;          // nbi + a.ntiles
+  int nitems;          // nbi + a.ntiles: items of one right-hand side
+  int nb;              // right-hand sides of the launch (grid y: groups of R of them)
   uint32_t stage;      // bytes per stage (multiple of 128)
   int max_ext;         // most extended rows of a block (the per-row scratch after the stages)
 };
@@ -96,9 +99,8 @@ __device__ __forceinline__ bool wait_parity(uint64_t* bar, uint32_t parity) {
 // of a tile (iterate, right-hand side, coarse iterate), after it.
 template <typename T, bool PRO>
 __device__ __forceinline__ void smooth_issue(const SmoothArgs<T>& A, const CUtensorMap* tin, const CUtensorMap* tr,
-                                             const CUtensorMap* tcls, const CUtensorMap* tuc, int item, int half,
+                                             const CUtensorMap* tcls, const CUtensorMap* tuc, int z, int item, int half,
                                              unsigned char* st, uint64_t* bar, int part = 0) {
-  const int z = blockIdx.y;      // right-hand side of the batch
   const SweepArgs<T>& a = A.a;
   if (item < A.nbi) {
     if (part == 2) return;
@@ -194,34 +196,48 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
 // [ne][nc] of the inverse, two columns a lane, extended rows over warps (two barriers for a
 // block of 64 core rows); the core cells and their old values from scell and sold (no global
 // round trip before the stores)
-__device__ __forceinline__ void block_apply(const float* As, const float* sres, const float* sold, const int* scell, int c0,
-                                            int nc, int ne, float* __restrict__ u_new, double* __restrict__ uhat,
-                                            float (*part)[64]) {
+// for nr <= R right-hand sides, sres and sold of one `slot` values after the other's, u_new and
+// uhat `bs` apart
+template <int R>
+__device__ __forceinline__ void block_apply(const float* As, const float* sres, const float* sold, int slot, const int* scell,
+                                            int c0, int nc, int ne, int nr, float* __restrict__ u_new,
+                                            double* __restrict__ uhat, long bs, float (*part)[8][64]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int cb = 0; cb < nc; cb += 64) {
     if (cb) __syncthreads();      // part is free
     const int c = cb + 2 * lane;
-    float2 acc = make_float2(0.0f, 0.0f);
+    float2 acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = make_float2(0.0f, 0.0f);
     if (c + 1 < nc && !(nc & 1)) {
 #pragma unroll 4
-      for (int e = warp; e < ne; e += 8) acc = __ffma2_rn(*reinterpret_cast<const float2*>(As + e * nc + c), pair(sres[e]), acc);
-    } else if (c < nc) {          // an odd number of columns: the rows' pairs are not aligned
       for (int e = warp; e < ne; e += 8) {
-        acc.x += As[e * nc + c] * sres[e];
-        if (c + 1 < nc) acc.y += As[e * nc + c + 1] * sres[e];
+        const float2 m = *reinterpret_cast<const float2*>(As + e * nc + c);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (R == 1 || r < nr) acc[r] = __ffma2_rn(m, pair(sres[r * slot + e]), acc[r]);
       }
+    } else if (c < nc) {          // an odd number of columns: the rows' pairs are not aligned
+      for (int e = warp; e < ne; e += 8)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (R > 1 && r >= nr) continue;
+          acc[r].x += As[e * nc + c] * sres[r * slot + e];
+          if (c + 1 < nc) acc[r].y += As[e * nc + c + 1] * sres[r * slot + e];
+        }
     }
-    *reinterpret_cast<float2*>(&part[warp][2 * lane]) = acc;
+#pragma unroll
+    for (int r = 0; r < R; ++r) *reinterpret_cast<float2*>(&part[r][warp][2 * lane]) = acc[r];
     __syncthreads();
-    const int t = cb + (int)threadIdx.x;
-    if (threadIdx.x < 64 && t < nc) {
+    const int r = threadIdx.x >> 6, l = threadIdx.x & 63, t = cb + l;
+    if (r < nr && t < nc) {
       float tot = 0;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) tot += part[w][threadIdx.x];
+      for (int w = 0; w < 8; ++w) tot += part[r][w][l];
       const int q = scell[c0 + t];
-      const float v = sold[c0 + t] + tot;
-      u_new[q] = v;
-      if (uhat) uhat[q] += (double)v;
+      const float v = sold[r * slot + c0 + t] + tot;
+      u_new[r * bs + q] = v;
+      if (uhat) uhat[r * bs + q] += (double)v;
     }
   }
 }
@@ -468,14 +484,18 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
   }
 }
 
-template <typename T, bool CROSS, bool PRO>
+// R: right-hand sides of a batch that share a CTA's items (grid y: groups of R).  A block item
+// serves all of them with one copy of its inverse rows (28 KB; one right-hand side at a time
+// these copies were two fifths of a sweep's L2 reads), then come the tile items of the first, the
+// second, ...
+template <typename T, bool CROSS, bool PRO, int R = 1>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __grid_constant__ CUtensorMap tin,
                                                 const __grid_constant__ CUtensorMap tr,
                                                 const __grid_constant__ CUtensorMap tcls,
                                                 const __grid_constant__ CUtensorMap tuc, SmoothArgs<T> A) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[2];
-  __shared__ __align__(16) T part[8][sizeof(T) == 8 ? 32 : 64];
+  __shared__ __align__(16) T part[R][8][sizeof(T) == 8 ? 32 : 64];
   __shared__ __align__(16) unsigned wmax[8];
   const SweepArgs<T>& a = A.a;
   // While the previous launch drains: pull the static fitted-row data (columns, coefficients,
@@ -496,38 +516,41 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
     if (threadIdx.x == 0) prefetch_l1(a.blk_off + b);
   }
   const int G = gridDim.x;
-  const int K = (A.nitems - (int)blockIdx.x + G - 1) / G;   // items of this CTA (>= 1)
+  const int z0 = blockIdx.y * R, nr = R == 1 ? 1 : min(R, A.nb - z0);
+  const int nitems = R == 1 ? A.nitems : A.nbi + nr * a.ntiles;
+  if (R > 1 && (int)blockIdx.x >= nitems) return;           // (the last group may be a small one)
+  const int K = (nitems - (int)blockIdx.x + G - 1) / G;     // items of this CTA (>= 1)
   // its block items come first and take BLOCK_PARTS steps of the ring each: NB block steps in
   // all, K steps with the tiles'
   constexpr int BP = BLOCK_PARTS<T>;
   const int kb = (int)blockIdx.x < A.nbi ? (A.nbi - 1 - (int)blockIdx.x) / G + 1 : 0;
   const int NB = BP * kb, KS = K + (BP - 1) * kb;
   auto item_of = [&](int k) { return (int)blockIdx.x + (k < NB ? k / BP : k - NB + kb) * G; };
+  // the right-hand side and the item among its own of a group's item
+  auto rhs_of = [&](int item) { return R == 1 || item < A.nbi ? z0 : z0 + (item - A.nbi) / a.ntiles; };
+  auto own_of = [&](int item) { return R == 1 || item < A.nbi ? item : A.nbi + (item - A.nbi) % a.ntiles; };
+  auto issue = [&](int k, int half, int sb, int part) {
+    const int item = item_of(k);
+    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, rhs_of(item), own_of(item), half, smem_raw + sb * A.stage, &bar[sb], part);
+  };
   // also before the wait: the copy barriers, and the parts of the first two items' copies
   // that no earlier launch writes (the rest follows the wait)
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
-    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(0), 0, smem_raw, &bar[0], 1);
-    if (KS > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(1), 1, smem_raw + A.stage, &bar[1], 1);
+    issue(0, 0, 0, 1);
+    if (KS > 1) issue(1, 1, 1, 1);
   }
   __syncthreads();
   pdl_enter();
-  // this CTA's right-hand side of the batch (blockIdx.y)
-  const long bo = (long)blockIdx.y * a.bs;
-  const T* __restrict__ u_old = a.u_old + bo;
-  T* __restrict__ u_new = a.u_new + bo;
-  double* __restrict__ uhat = a.uhat ? a.uhat + bo : nullptr;
-  const T* __restrict__ rhs = a.r + bo;
-  const T* __restrict__ ucs = PRO ? a.uc + (long)blockIdx.y * a.bsc : nullptr;
-  // per extended row of a block item: residual, old value, cell (three slots of max_ext)
+  // per extended row of a block item: residual, old value, cell (slots of max_ext, the first two for each right-hand side)
   const uint32_t slot = (uint32_t)(((long)A.max_ext * sizeof(T) + 15) & ~15L);
   T* sres = reinterpret_cast<T*>(smem_raw + 2 * A.stage);
-  T* sold = reinterpret_cast<T*>(smem_raw + 2 * A.stage + slot);
-  int* scell = reinterpret_cast<int*>(smem_raw + 2 * A.stage + 2 * slot);
+  T* sold = reinterpret_cast<T*>(smem_raw + 2 * A.stage + R * slot);
+  int* scell = reinterpret_cast<int*>(smem_raw + 2 * A.stage + 2 * R * slot);
   if (threadIdx.x == 0) {
-    smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(0), 0, smem_raw, &bar[0], 2);
-    if (KS > 1) smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(1), 1, smem_raw + A.stage, &bar[1], 2);
+    issue(0, 0, 0, 2);
+    if (KS > 1) issue(1, 1, 1, 2);
   }
   T acc = 0;                     // BP == 2: a block's product, carried from its first half to its second
   int cs = 0, nc = 0, ne = 0, es = 0;
@@ -537,9 +560,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
     const uint32_t parity = (k >> 1) & 1;
     int cx0 = 0, cy0 = 0;
     if (item < A.nbi) {
-      if (half == 0) block_residuals<T, PRO, false>(a, item, u_old, rhs, ucs, sres, sold, scell, cs, nc, ne, es);
+      if (half == 0)
+        for (int r = 0; r < nr; ++r) {
+          const long bo = (long)(z0 + r) * a.bs;
+          block_residuals<T, PRO, false>(a, item, a.u_old + bo, a.r + bo, PRO ? a.uc + (long)(z0 + r) * a.bsc : nullptr,
+                                         sres + r * (slot / sizeof(T)), sold + r * (slot / sizeof(T)), scell, cs, nc, ne, es);
+        }
     } else {
-      const int t = item - A.nbi;       // the tile's origin, read before the wait
+      const int t = own_of(item) - A.nbi;       // the tile's origin, read before the wait
       cx0 = a.tiles[2 * t] * JX;
       cy0 = a.tiles[2 * t + 1] * JY;
     }
@@ -555,17 +583,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
       const T* As = reinterpret_cast<const T*>(smem_raw + sb * A.stage);
       if constexpr (BP == 2) {
         const int e0 = half ? block_split(ne) : 0, e1 = half ? ne : block_split(ne);
-        block_apply_part(As, sres, sold, scell, cs - es, nc, e0, e1, half == 1, acc, u_new, &part[0][0]);
+        block_apply_part(As, sres, sold, scell, cs - es, nc, e0, e1, half == 1, acc, a.u_new + z0 * a.bs, &part[0][0][0]);
       } else {
-        block_apply(As, sres, sold, scell, cs - es, nc, ne, u_new, uhat, part);
+        block_apply<R>(As, sres, sold, (int)(slot / sizeof(T)), scell, cs - es, nc, ne, nr, a.u_new + z0 * a.bs,
+                       a.uhat ? a.uhat + z0 * a.bs : nullptr, a.bs, part);
       }
     } else {
-      tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, u_new, uhat, wmax);
+      const long bo = rhs_of(item) * a.bs;
+      tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, a.u_new + bo, a.uhat ? a.uhat + bo : nullptr, wmax);
     }
     __syncthreads();      // stage sb is free
     if (threadIdx.x == 0 && k + 2 < KS) {
       fence_proxy_async();
-      smooth_issue<T, PRO>(A, &tin, &tr, &tcls, &tuc, item_of(k + 2), k % BP, smem_raw + sb * A.stage, &bar[sb]);
+      issue(k + 2, k % BP, sb, 0);
     }
   }
 }

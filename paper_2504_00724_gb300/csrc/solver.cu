@@ -409,6 +409,7 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   a.uc = C ? U<T>(*C) : nullptr;
   A.nbi = L.nblk;
   A.nitems = L.nblk + L.ntiles64;
+  A.nb = H->nb;
   A.stage = L.smooth_stage[k];
   A.max_ext = std::max(1, L.max_ext);
   const bool l0f = &L == &H->L[0] && sizeof(T) == 4;
@@ -424,16 +425,26 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   a.bs = L.npad;
   a.bsc = C ? C->npad : 0;
   // with a batch, fewer CTAs per right-hand side so that the whole launch stays resident
-  const dim3 grid(persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], H->nb, H->launch_cap), H->nb);
+  const int ctas = persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], H->nb, H->launch_cap);
   const size_t smem = L.smooth_smem[k];
-  if (C) {
-    const CUtensorMap& tu = TmUc<T>(L, *C);
-    if (H->cross) KL(launch_k(dev::k_smooth<T, true, true>, grid, 256, smem, s, tm, tr, L.tmcls, tu, A));
-    else KL(launch_k(dev::k_smooth<T, false, true>, grid, 256, smem, s, tm, tr, L.tmcls, tu, A));
-  } else {
-    if (H->cross) KL(launch_k(dev::k_smooth<T, true, false>, grid, 256, smem, s, tm, tr, L.tmcls, tm, A));
-    else KL(launch_k(dev::k_smooth<T, false, false>, grid, 256, smem, s, tm, tr, L.tmcls, tm, A));
+  const CUtensorMap& tu = C ? TmUc<T>(L, *C) : tm;
+  auto go = [&](auto kernel, dim3 grid) { KL(launch_k(kernel, grid, 256, smem, s, tm, tr, L.tmcls, tu, A)); };
+  if constexpr (sizeof(T) == 4) {
+    constexpr int R = dev::BATCH_SHARE;
+    if (H->nb >= R) {       // groups of R right-hand sides, with the CTAs of R
+      const dim3 grid(std::min(ctas * R, A.nbi + R * L.ntiles64), ceil_div(H->nb, R));
+      if (C && H->cross) go(dev::k_smooth<T, true, true, R>, grid);
+      else if (C) go(dev::k_smooth<T, false, true, R>, grid);
+      else if (H->cross) go(dev::k_smooth<T, true, false, R>, grid);
+      else go(dev::k_smooth<T, false, false, R>, grid);
+      return;
+    }
   }
+  const dim3 grid(ctas, H->nb);
+  if (C && H->cross) go(dev::k_smooth<T, true, true>, grid);
+  else if (C) go(dev::k_smooth<T, false, true>, grid);
+  else if (H->cross) go(dev::k_smooth<T, true, false>, grid);
+  else go(dev::k_smooth<T, false, false>, grid);
 }
 
 template <typename T>
@@ -1010,8 +1021,10 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
     if (k == 0 && d.max_core > 128) continue;
     const size_t blk = ((size_t)ext * d.max_core * es + 15) & ~(size_t)15;
     const size_t stage = (std::max(tile, blk) + 127) & ~(size_t)127;
-    // two stages, then per extended row of a block: its residual, old value and cell
-    const size_t smem = 2 * stage + 3 * (((size_t)std::max(1, d.max_ext) * es + 15) & ~(size_t)15);
+    // two stages, then per extended row of a block: its residual and old value (of each
+    // right-hand side that shares the item) and its cell
+    const int share = k == 1 && h->B >= dev::BATCH_SHARE ? dev::BATCH_SHARE : 1;
+    const size_t smem = 2 * stage + (2 * share + 1) * (((size_t)std::max(1, d.max_ext) * es + 15) & ~(size_t)15);
     if (smem > 200 * 1024) continue;
     int occ = 0;
     if (k == 0) {
@@ -1026,6 +1039,15 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
       for (auto g : {h->cross ? dev::k_smooth<float, true, false> : dev::k_smooth<float, false, false>})
         cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (share > 1) {
+        constexpr int R = dev::BATCH_SHARE;
+        auto gp = h->cross ? dev::k_smooth<float, true, true, R> : dev::k_smooth<float, false, true, R>;
+        auto gn = h->cross ? dev::k_smooth<float, true, false, R> : dev::k_smooth<float, false, false, R>;
+        for (auto g : {gp, gn}) cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        int o = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, gp, 256, smem);
+        occ = std::min(occ, o);
+      }
     }
     if (occ < 1 || nsm < 1) continue;
     d.smooth_ok[k] = true;
