@@ -37,6 +37,8 @@ struct ApplyArgs {
   long nseg;
   double scale;              // 1 / h^2
   bool vec;                  // out rows start on 16 bytes
+  bool uvec;                 // u rows start on 16 bytes
+  const uint8_t* act;        // per 64 x 32 tile of the box: it holds a non-empty cell
   Stencil<double> S;
   QStencil Q;
 };
@@ -48,8 +50,9 @@ __device__ __forceinline__ long cell_at(int p, int pitch, long stride) {
 }
 
 // out = L u + N g (TRANS: the regular cells' part of L^T v on every non-empty cell, and N^T v).
-// Bound by memory at large sizes: star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134
-// MB written.
+// star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134 MB written (26 us at the copy rate):
+// 66 us, bound by the integer stencil's issue slots (85 us with the classes loaded first and cell by
+// cell, so that a tile took two round trips and 10 loads a thread in place of 5).
 template <bool CROSS, bool TRANS>
 __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
   __shared__ __align__(16) double tile[HY * HX];
@@ -77,19 +80,6 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
   }
   const int t = blockIdx.x - A.nrow;
   const int cx0 = (t % A.tx) * JX, cy0 = (t / A.tx) * JY;
-  // classes of the staged slots (threadIdx.x + 256 k of the 68 x 36 tile with its halo)
-  constexpr int N = (HY * HX + 255) / 256;
-  bool on[N];
-  bool any = false;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const int idx = threadIdx.x + 256 * k, y = idx / HX, x = idx - y * HX;
-    const int i = cx0 + x - 2, j = cy0 + y - 2;
-    const bool in = idx < HY * HX && (unsigned)i < (unsigned)A.nx && (unsigned)j < (unsigned)A.ny;
-    const uint8_t c = in ? A.cls[(long)(j + 2) * A.pitch + i + 2] : (uint8_t)0;
-    on[k] = TRANS ? c == 1 : c != 0;
-    any |= c != 0;
-  }
   const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
   const int i0 = cx0 + x0;
   auto put = [&](int kk, double s0, double s1, uint32_t c2) {
@@ -106,25 +96,53 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
       if (g1) o[1] = v1;
     }
   };
-  if (!__syncthreads_or(any)) {
+  if (!A.act[t]) {
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) put(kk, 0.0, 0.0, 0u);
     return;
   }
-  uint32_t c2[4];
+  uint32_t c2[2] = {0, 0};      // the classes of two rows' pairs each
 #pragma unroll
   for (int kk = 0; kk < 4; ++kk) {
     const int j = cy0 + y0 + kk;
-    c2[kk] = (i0 < A.nx && j < A.ny) ? *reinterpret_cast<const uint16_t*>(A.cls + (long)(j + 2) * A.pitch + i0 + 2) : 0u;
+    if (i0 < A.nx && j < A.ny)
+      c2[kk >> 1] |= (uint32_t)*reinterpret_cast<const uint16_t*>(A.cls + (long)(j + 2) * A.pitch + i0 + 2) << (16 * (kk & 1));
   }
+  // the 68 x 36 tile with its halo, in pairs of cells; classes and values are loaded together (the
+  // values of cells that do not count are dropped afterwards)
+  const auto counts = [](uint32_t c) { return TRANS ? c == 1u : c != 0u; };
+  constexpr int NP = HY * HX / 2;
+  if (A.uvec) {
+    constexpr int N = (NP + 255) / 256;
+    double2 v[N];
+    uint32_t c[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const int idx = threadIdx.x + 256 * k, y = idx / HX, x = idx - y * HX;
-    if (idx < HY * HX) tile[idx] = on[k] ? u[(cy0 + y - 2) * A.u.stride + (cx0 + x - 2)] : 0.0;
+    for (int k = 0; k < N; ++k) {
+      const int idx = threadIdx.x + 256 * k, y = idx / (HX / 2), i = cx0 - 2 + 2 * (idx - y * (HX / 2)), j = cy0 - 2 + y;
+      const bool in = idx < NP && (unsigned)i < (unsigned)A.nx && (unsigned)j < (unsigned)A.ny;
+      c[k] = in ? *reinterpret_cast<const uint16_t*>(A.cls + (long)(j + 2) * A.pitch + i + 2) : 0u;
+      v[k] = in ? *reinterpret_cast<const double2*>(u + j * A.u.stride + i) : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const int idx = threadIdx.x + 256 * k;
+      if (!counts(c[k] & 0xffu)) v[k].x = 0.0;
+      if (!counts(c[k] >> 8)) v[k].y = 0.0;
+      if (idx < NP) *reinterpret_cast<double2*>(tile + 2 * idx) = v[k];
+    }
+  } else {
+#pragma unroll 5
+    for (int idx = threadIdx.x; idx < HY * HX; idx += 256) {
+      const int y = idx / HX, i = cx0 + idx - y * HX - 2, j = cy0 + y - 2;
+      const bool in = (unsigned)i < (unsigned)A.nx && (unsigned)j < (unsigned)A.ny;
+      const uint32_t c = in ? A.cls[(long)(j + 2) * A.pitch + i + 2] : 0u;
+      tile[idx] = counts(c) ? u[j * A.u.stride + i] : 0.0;
+    }
+    __syncthreads();
   }
-  // each thread reads back its own slots first (tile_stencil64's maximum), so no barrier here
+  // with pairs each thread reads back its own slots first (tile_stencil64's maximum): no barrier
   tile_stencil64<CROSS>(tile, wmax, x0, y0, true, A.S, A.Q, [&](int kk, double s0, double s1) {
-    put(kk, s0, s1, kk == 0 ? c2[0] : kk == 1 ? c2[1] : kk == 2 ? c2[2] : c2[3]);
+    put(kk, s0, s1, ((kk < 2 ? c2[0] : c2[1]) >> (16 * (kk & 1))) & 0xffffu);
   });
 }
 

@@ -133,19 +133,24 @@ __device__ __forceinline__ unsigned q_cta_max(unsigned m, unsigned* wmax) {
   return max(max(max(a.x, a.y), max(a.z, a.w)), max(max(b.x, b.y), max(b.z, b.w)));
 }
 
-// this thread's slots threadIdx.x + 256 k of a staged tile of n doubles, and their largest word
+// this thread's pairs threadIdx.x + 256 k of a staged tile of n pairs of doubles, and their largest
+// word
 template <int N>
 struct QSlots {
-  unsigned hi[N], lo[N];
+  unsigned hi[2 * N], lo[2 * N];
   __device__ __forceinline__ unsigned load(const double* tile, int n) {
     unsigned m = 0;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int idx = threadIdx.x + 256 * k;
-      const unsigned long long b = idx < n ? (unsigned long long)__double_as_longlong(tile[idx]) : 0ull;
-      hi[k] = (unsigned)(b >> 32);
-      lo[k] = (unsigned)b;
-      m = max(m, q_word(hi[k], lo[k]));
+      const double2 v = idx < n ? *reinterpret_cast<const double2*>(tile + 2 * idx) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(j ? v.y : v.x);
+        hi[2 * k + j] = (unsigned)(b >> 32);
+        lo[2 * k + j] = (unsigned)b;
+        m = max(m, q_word(hi[2 * k + j], lo[2 * k + j]));
+      }
     }
     return m;
   }
@@ -153,7 +158,9 @@ struct QSlots {
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int idx = threadIdx.x + 256 * k;
-      if (idx < n) q[idx] = q_fixed(hi[k], lo[k], E);
+      if (idx < n)
+        *reinterpret_cast<longlong2*>(q + 2 * idx) =
+            make_longlong2(q_fixed(hi[2 * k], lo[2 * k], E), q_fixed(hi[2 * k + 1], lo[2 * k + 1], E));
     }
   }
 };

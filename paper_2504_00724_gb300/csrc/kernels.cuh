@@ -1042,7 +1042,8 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 // iterate (u null: 0) and ||r_hat||; with u null also what the initial residual r_hat - L 0 gives,
 // its FP32 image (r32) and its norm (norm0).  Memory bounds it: f (and u) read once, the level-0
 // arrays written once, for all right-hand sides (blockIdx.y) in one launch.  Empty cells of
-// the padded arrays are 0 from their allocation on and are not written.
+// the padded arrays are 0 from their allocation on and are not written.  star 4096^2: 47 us cold (147 MB;
+// the clearing, packing, norm and residual passes it replaced: 230 us), k_store 28 us.
 struct LoadArgs {
   const int32_t* tiles;      // the active 32 x 8 tiles: every non-empty cell lies in one
   int ntiles, nx, ny, pitch;

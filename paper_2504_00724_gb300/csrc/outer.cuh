@@ -111,8 +111,16 @@ __global__ void __launch_bounds__(256, 3) k_resid(const __grid_constant__ CUtens
       }
     });
   }
+  // one atomic a CTA, and none where the norm is already larger (all of them hit one word)
+  __shared__ unsigned long long wm[8];
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(A.norm + z, m);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = max(m, wm[w]);
+    if (m > *(volatile unsigned long long*)(A.norm + z)) atomicMax(A.norm + z, m);
+  }
 }
 
 // u_hat += e on the non-empty cells of the 32 x 8 tiles that hold one

@@ -34,6 +34,8 @@ namespace dev {
 template <typename T>
 constexpr int BLOCK_PARTS = sizeof(T) == 8 ? 2 : 1;
 // right-hand sides of a batch that share block items (FP32; 256 threads update 64 core rows of 4)
+// disk 512^2, 64 right-hand sides: 22.6 ms a solve without, 20.1 with; below four the launch is not
+// bound by L2 and keeps its CTAs apart
 constexpr int BATCH_SHARE = 4;
 // extended rows of the first part (even: the second part's copy starts on 16 bytes)
 __host__ __device__ constexpr int block_split(int ne) { return (ne / 2 + 1) & ~1; }
@@ -153,7 +155,8 @@ __device__ __forceinline__ void block_residuals(const SweepArgs<T>& a, int b, co
   // Two threads a row (a block has at most 256 / 2 rows at the default shape), each every other
   // one of its coefficients.  The gathers' round trips are the launch's critical path on small
   // levels, so each thread has up to eight in flight and none hangs on a branch: a column without a
-  // coarse parent reads cell 0, which lies in the zero ring, and adds nothing.
+  // coarse parent reads cell 0, which lies in the zero ring, and adds nothing (one thread a row and a
+  // branch a coefficient: a PRO sweep of a small level took 11.8 us cold, now 7.1).
   const int part = threadIdx.x & 1;
   for (int e0 = 0; e0 < ne; e0 += blockDim.x / 2) {
     const int e = e0 + (int)(threadIdx.x >> 1);
@@ -304,14 +307,15 @@ __device__ __forceinline__ void fp64_rows(const double* __restrict__ tile, int x
 template <bool CROSS, class Emit>
 __device__ __forceinline__ void tile_stencil64(double* tile, unsigned* wmax, int x0, int y0, bool on,
                                                const Stencil<double>& S, const QStencil& Q, Emit emit) {
-  QSlots<(HY * HX + 255) / 256> v;
-  const int E = q_scale(q_cta_max(v.load(tile, HY * HX), wmax), Q);
+  constexpr int NP = HY * HX / 2;
+  QSlots<(NP + 255) / 256> v;
+  const int E = q_scale(q_cta_max(v.load(tile, NP), wmax), Q);
   if (E < 0) {
     if (on) fp64_rows<CROSS>(tile, x0, y0, S, emit);
     return;
   }
   long long* q = reinterpret_cast<long long*>(tile);
-  v.store(q, HY * HX, E);
+  v.store(q, NP, E);
   __syncthreads();
   const int e = E - 1022 + Q.cexp;
   if (on) q_rows<CROSS, HX>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
@@ -324,7 +328,8 @@ __device__ __forceinline__ void tile_stencil64(double* tile, unsigned* wmax, int
 // two second derivatives keep the order of a plain sum; odd taps would need the pairs at odd
 // columns and stay scalar.  Error against 64-bit sums, rms over smooth and rough fields: 0.52 to
 // 0.95 of the 25-tap FMA chain's, equal to it without the mixed term.
-// emit(k, Lu, u) with both cells' values.
+// emit(k, Lu, u) with both cells' values.  A sweep of the star 4096^2's finest level, cold: 22.5 us
+// with the 25-tap sum and a class test a cell, 20.2 us with this and one test for eight cells.
 template <bool CROSS, class Emit>
 __device__ __forceinline__ void stencil32(const float* __restrict__ tile, int x0, int y0, const Stencil<float>& S,
                                           Emit emit) {

@@ -39,6 +39,7 @@ struct DevLevel {
   int32_t* tiles = nullptr;
   int ntiles64 = 0;
   int32_t* tiles64 = nullptr;
+  uint8_t* act64 = nullptr;     // per 64 x 32 tile of the box: it holds a non-empty cell
   int ntiles64r = 0;            // fine 64 x 32 tiles that restriction to level m + 1 visits
   int32_t* tiles64r = nullptr;
   bool stage_blocks = false;    // SMO-2 block inverses fit in shared memory (bulk-staged kernel)
@@ -908,6 +909,8 @@ void launch_apply(ccm_handle* H, DevLevel& L, dev::Grid<const double*> u, dev::G
   A.nseg = H->info.n_segments;
   A.scale = scale;
   A.vec = ((uintptr_t)out.p % 16) == 0 && out.stride % 2 == 0 && (out.batch % 2 == 0 || nrhs == 1);
+  A.uvec = ((uintptr_t)u.p % 16) == 0 && u.stride % 2 == 0 && (u.batch % 2 == 0 || nrhs == 1);
+  A.act = L.act64;
   A.S = H->S64;
   A.Q = H->Q;
   const int tiles = out.p ? A.tx * ceil_div(L.ny, dev::JY) : 0;
@@ -1244,6 +1247,13 @@ int upload_hierarchy(ccm_handle* h) {
       for (size_t k = 0; k < rc.size(); ++k) rc[k] = hl.irr_cell[hl.tr_row[k]];
       d.tr_rcell = A.upload(rc);
       d.tr_val = A.upload(hl.tr_val);
+    }
+    {
+      const int tx = ceil_div(hl.nx, dev::JX);
+      std::vector<uint8_t> act((size_t)tx * ceil_div(hl.ny, dev::JY), 0);
+      for (size_t k = 0; k + 1 < hl.tiles.size(); k += 2)
+        act[(size_t)(hl.tiles[k + 1] * dev::TY / dev::JY) * tx + hl.tiles[k] * dev::TX / dev::JX] = 1;
+      d.act64 = A.upload(act);
     }
     d.ntiles64 = (int)hl.tiles64.size() / 2;
     if (d.ntiles64) d.tiles64 = A.upload(hl.tiles64);
