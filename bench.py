@@ -61,7 +61,7 @@ KERNEL_SOURCES = ("kernels.cuh", "smooth.cuh", "outer.cuh")
 NCU_TRAFFIC = {        # class name -> (source hash, bytes per launch)
     "fp32 sweep, level 0 (SMO-1 regular cells + SMO-2 blocks)": ("e9d37767504660f2", 69.69e6),
     "fp32 residual + restriction, level 0": ("e9d37767504660f2", 76.64e6),
-    "outer residual, level 0 (regular cells, float-float)": ("e9d37767504660f2", 95.72e6),
+    "outer residual, level 0": ("e9d37767504660f2", 95.72e6),
 }
 
 
@@ -710,9 +710,8 @@ def main():
     ms, nl = prof_res
     if nl:
         # the outer residual reads u_hat, r_hat (FP64) and the class byte and writes the FP32
-        # image of the residual per regular cell (8 + 8 + 1 + 4 B); it runs in float-float
-        # arithmetic at this tolerance
-        classes.append(("outer residual, level 0 (regular cells, float-float)", ms, ms / nl, nl, "hbm",
+        # image of the residual per regular cell (8 + 8 + 1 + 4 B)
+        classes.append(("outer residual, level 0", ms, ms / nl, nl, "hbm",
                         n_reg * 21.0, "GB/s"))
     roof = None
     if classes:

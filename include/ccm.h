@@ -267,16 +267,16 @@ int ccm_apply_T(ccm_handle* h, const double* v, double* out_u, double* out_g, in
 
 /* Solve L u = f - N g (eq. PoissonResidualForm) by V-cycles (Alg. 2) to rtol.  One outer
  * iteration (CCM_FP64: one FP64 V-cycle; CCM_MIXED: inner_cycles FP32 V-cycles on the FP32
- * image of the FP64 residual, then u += e in FP64) runs as one CUDA graph, captured on the
- * first call; the FP64 residual norm is read back after every outer iteration.
+ * image of the FP64 residual, then u += e in FP64) is captured on the first call as the body of
+ * one CUDA graph that loops on the device until the FP64 residual norm meets rtol.
  * f: device [nrhs][ny][nx] cell averages; g: device [nrhs][n_segments] (NULL: g = 0);
  * u: device [nrhs][ny][nx], in: initial guess, out: solution.  CCM_MIXED handles with
  * ccm_info.batch > 1 advance up to that many right-hand sides per graph replay, until the
  * worst of them meets rtol (the others iterate on).  stats (host, nullable) receives the
  * outer iteration count of the last group and, per iteration, the largest relative residual
  * of its right-hand sides.
- * Synchronises the stream once per outer iteration (the convergence test).  The first call
- * captures the graphs, so make it outside any caller's stream capture.
+ * Synchronises the stream once (a profiled solve, ccm_profile: once per outer iteration).  The
+ * first call captures the graphs, so make it outside any caller's stream capture.
  * Errors: CCM_ENOCONV (u holds the last iterate), CCM_ENOTFINITE, CCM_ECUDA. */
 int ccm_solve(ccm_handle* h, const double* f, const double* g, double* u, int nrhs,
               void* stream, ccm_stats* stats);
