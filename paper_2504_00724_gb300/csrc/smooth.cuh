@@ -23,6 +23,7 @@
 // bounded) for every copy still in flight, and the CTA leaves, all threads together.
 #pragma once
 
+#include "blocks.cuh"
 #include "kernels.cuh"
 
 namespace ccm {
@@ -37,8 +38,6 @@ constexpr int BLOCK_PARTS = sizeof(T) == 8 ? 2 : 1;
 // disk 512^2, 64 right-hand sides: 22.6 ms a solve without, 20.1 with; below four the launch is not
 // bound by L2 and keeps its CTAs apart
 constexpr int BATCH_SHARE = 4;
-// extended rows of the first part (even: the second part's copy starts on 16 bytes)
-__host__ __device__ constexpr int block_split(int ne) { return (ne / 2 + 1) & ~1; }
 
 template <typename T>
 struct SmoothArgs {
@@ -110,9 +109,9 @@ __device__ __forceinline__ void smooth_issue(const SmoothArgs<T>& A, const CUten
     const int nc = a.blk[4 * b + 1] - a.blk[4 * b], ne = a.blk[4 * b + 3] - a.blk[4 * b + 2];
     const int e0 = BLOCK_PARTS<T> == 2 && half ? block_split(ne) : 0;
     const int e1 = BLOCK_PARTS<T> == 2 && !half ? block_split(ne) : ne;
-    const uint32_t abytes = (uint32_t)(((long)(e1 - e0) * nc * sizeof(T) + 15) & ~15L);
+    const uint32_t abytes = block_copy_bytes(e1 - e0, nc, sizeof(T));
     mbar_expect_tx(bar, abytes);
-    if (abytes) bulk_load(st, a.inv + a.blk_off[b] + (long)e0 * nc, abytes, bar);   // (a block of 1 or 2 rows: an empty half)
+    if (abytes) bulk_load(st, a.inv + a.blk_off[b] + (long)e0 * nc, abytes, bar);   // (a block of 1 or 2 rows: an empty second part)
   } else {
     using S = TileStage<T>;
     const int t = item - A.nbi;

@@ -1019,10 +1019,9 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   for (int k = 0; k < 2 && d.tma && one_chunk && nitems > 0; ++k) {
     const size_t es = k == 0 ? sizeof(double) : sizeof(float);
     const size_t tile = k == 0 ? dev::TileStage<double>::bytes(true) : dev::TileStage<float>::bytes(true);
-    // the rows of a block item that one stage takes (all in FP32, half in FP64)
-    const int ext = k == 0 ? std::max(2, dev::block_split(d.max_ext)) : d.max_ext;
     if (k == 0 && d.max_core > 128) continue;
-    const size_t blk = ((size_t)ext * d.max_core * es + 15) & ~(size_t)15;
+    // the rows of a block item that one stage takes (all in FP32, half in FP64)
+    const size_t blk = dev::block_stage_bytes(d.max_ext, d.max_core, (int)es, k == 0);
     const size_t stage = (std::max(tile, blk) + 127) & ~(size_t)127;
     // two stages, then per extended row of a block: its residual and old value (of each
     // right-hand side that shares the item) and its cell
