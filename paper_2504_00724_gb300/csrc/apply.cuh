@@ -49,7 +49,7 @@ __device__ __forceinline__ long cell_at(int p, int pitch, long stride) {
   return (j - 2) * stride + (i - 2);
 }
 
-// out = L u + N g (TRANS: the regular cells' part of L^T v on every non-empty cell, and N^T v).
+// out = L u + N g (TRANS: L^T v on the cells that no fitted row's stencil reaches, and N^T v).
 // star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134 MB written (26 us at the copy rate):
 // 66 us, bound by the integer stencil's issue slots (85 us with the classes loaded first and cell by
 // cell, so that a tile took two round trips and 10 loads a thread in place of 5).
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
   auto put = [&](int kk, double s0, double s1, uint32_t c2) {
     const int j = cy0 + y0 + kk;
     if (j >= A.ny || i0 >= A.nx) return;
-    // forward: the fitted rows' cells are written by their own CTAs
-    const bool g0 = TRANS || (c2 & 0xffu) != 2u, g1 = (TRANS || (c2 >> 8) != 2u) && i0 + 1 < A.nx;
+    // the fitted rows' cells are written by their own CTAs, or (TRANS) by k_rows_T
+    const bool g0 = (c2 & 0xffu) != 2u, g1 = (c2 >> 8) != 2u && i0 + 1 < A.nx;
     const double v0 = (c2 & 0xffu) ? A.scale * s0 : 0.0, v1 = (c2 >> 8) ? A.scale * s1 : 0.0;
     double* o = out + (long)j * A.out.stride + i0;
     if (A.vec && g0 && g1) {
@@ -146,19 +146,51 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
   });
 }
 
-// out += the fitted rows' part of L^T v, by the transposed CSR (one thread per column cell; the
-// entry's row is given by its cell)
-__global__ void k_rows_T(int ncol, const int32_t* __restrict__ ptr, const int32_t* __restrict__ ccell,
-                         const int32_t* __restrict__ rcell, const double* __restrict__ val, Grid<const double*> v,
-                         Grid<double*> out, int pitch, double scale) {
+// L^T v at the cells that the fitted rows' stencils reach (every irregular cell is one): the regular
+// cells' part, sum_d w_d v[c + d] over the regular c + d (the stencil is point-symmetric), and the
+// fitted rows' by the transposed CSR (its entries' rows are given by their cells), scaled together,
+// over what k_apply wrote there.  One thread per cell; its classes and row range, which no launch
+// writes, before the wait.  (Adding the scaled fitted part to k_apply's scaled part instead rounds once
+// more, an eighth more error; disk 1408^2, 4 vectors, whole call: 67.3 us that way, 70.0 this.)
+struct RowsTArgs {
+  int n;                     // cells
+  const int32_t* ptr;
+  const int32_t* cell;       // padded
+  const int32_t* rcell;      // padded
+  const double* val;
+  const uint8_t* cls;        // padded
+  int pitch;
+  double scale;
+  Grid<const double*> v;
+  Grid<double*> out;
+  Stencil<double> S;
+};
+
+template <bool CROSS>
+__global__ void __launch_bounds__(128) k_rows_T(RowsTArgs A) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int e0 = k < ncol ? ptr[k] : 0, e1 = k < ncol ? ptr[k + 1] : 0;
+  const bool on = k < A.n;
+  const int c = on ? A.cell[k] : 2 * A.pitch + 2, e0 = on ? A.ptr[k] : 0, e1 = on ? A.ptr[k + 1] : 0;
+  uint32_t reg = 0;          // bit 5 (dj + 2) + di + 2: a regular cell
+#pragma unroll
+  for (int dj = -2; dj <= 2; ++dj)
+#pragma unroll
+    for (int di = -2; di <= 2; ++di) {
+      if (!CROSS && dj != 0 && di != 0) continue;
+      reg |= (uint32_t)(A.cls[c + (long)dj * A.pitch + di] == 1) << (5 * (dj + 2) + di + 2);
+    }
   pdl_enter();
-  if (k >= ncol) return;
-  const double* vz = v.p + blockIdx.y * v.batch;
-  double acc = 0;
-  for (int e = e0; e < e1; ++e) acc += val[e] * vz[cell_at(rcell[e], pitch, v.stride)];
-  out.p[blockIdx.y * out.batch + cell_at(ccell[k], pitch, out.stride)] += scale * acc;
+  if (!on) return;
+  const double* v = A.v.p + blockIdx.y * A.v.batch;
+  const long p = cell_at(c, A.pitch, A.v.stride);
+  double w[25], acc = 0, rows = 0;
+#pragma unroll
+  for (int t = 0; t < 25; ++t) w[t] = reg >> t & 1 ? v[p + (t / 5 - 2) * A.v.stride + t % 5 - 2] : 0.0;
+#pragma unroll
+  for (int t = 0; t < 25; ++t)
+    if (CROSS || t / 5 == 2 || t % 5 == 2) acc += A.S.w[t] * w[t];
+  for (int e = e0; e < e1; ++e) rows += A.val[e] * v[cell_at(A.rcell[e], A.pitch, A.v.stride)];
+  A.out.p[blockIdx.y * A.out.batch + cell_at(c, A.pitch, A.out.stride)] = A.scale * (acc + rows);
 }
 
 }  // namespace dev

@@ -1763,12 +1763,24 @@ int ccm_apply_T(ccm_handle* h, const double* v, double* out_u, double* out_g, in
   const long nu = (long)L.nx * L.ny, ns = h->info.n_segments;
   const double sc = 1.0 / (L.h * L.h);
   auto rows_T = [&](dev::Grid<const double*> vv, dev::Grid<double*> o, int n, double scale) {
+    dev::RowsTArgs A{};
+    A.n = L.ncolT;
+    A.ptr = L.tr_ptr;
+    A.cell = L.tr_cell;
+    A.rcell = L.tr_rcell;
+    A.val = L.tr_val;
+    A.cls = L.cls;
+    A.pitch = L.pitch;
+    A.scale = scale;
+    A.v = vv;
+    A.out = o;
+    A.S = h->S64;
     for (int k = 0; k < n && L.ncolT; k += 65535) {
-      KL(launch_k(dev::k_rows_T, dim3(ceil_div(L.ncolT, 128), std::min(n - k, 65535)), 128, 0, s, L.ncolT,
-                  (const int32_t*)L.tr_ptr, (const int32_t*)L.tr_cell, (const int32_t*)L.tr_rcell, (const double*)L.tr_val,
-                  vv, o, L.pitch, scale));
-      vv.p += 65535 * vv.batch;
-      o.p += 65535 * o.batch;
+      const dim3 grid(ceil_div(L.ncolT, 128), std::min(n - k, 65535));
+      if (h->cross) KL(launch_k(dev::k_rows_T<true>, grid, 128, 0, s, A));
+      else KL(launch_k(dev::k_rows_T<false>, grid, 128, 0, s, A));
+      A.v.p += 65535 * A.v.batch;
+      A.out.p += 65535 * A.out.batch;
     }
   };
   if (!overlap(out_u, nrhs * nu, v, nrhs * nu) && !overlap(out_g, nrhs * ns, v, nrhs * nu)) {
