@@ -234,7 +234,8 @@ int ccm_boundary_averages(const ccm_handle* h, ccm_grad_fn g, void* ctx, double*
 
 /* out = L u + N g (eq. PoissonLinearDiscretization) on the finest level, physical units.
  * u, out: device [nrhs][ny][nx] FP64; g: device [nrhs][n_segments] FP64 (may be NULL: g = 0).
- * Runs in FP64 (regular stencil, Sec. 3.2; fitted irregular rows, eq. goalOfApproximation). */
+ * Runs in FP64 (regular stencil, Sec. 3.2; fitted irregular rows, eq. goalOfApproximation): every
+ * cell's error is relative to that cell's own terms, also beside much larger values. */
 int ccm_apply(ccm_handle* h, const double* u, const double* g, double* out, int nrhs, void* stream);
 
 /* Allocation-free operator application.  Same result as ccm_apply with nrhs = 1
@@ -346,7 +347,9 @@ int ccm_solve_T_zero(ccm_handle* h, const double* rhs, double* lambda, int nrhs,
 
 /* ---- level components of the V-cycle (one call = one step of the path, for testing and
  *      composition).  Level arrays use the user layout of that level: [ny_m][nx_m] FP64
- *      device arrays with nx_m = nx >> m, values in physical units of level m. */
+ *      device arrays with nx_m = nx >> m, values in physical units of level m.  In FP64 a cell's
+ *      error is relative to its own terms.  (Inside the solves, ccm_vcycle and ccm_fmg the FP64
+ *      stencil's rounding is relative to the largest value of a 68 x 36 tile, 2^-60 of it.) */
 
 /* out = L^(m) u on level m (no boundary term). */
 int ccm_level_apply(ccm_handle* h, int level, const double* u, double* out, void* stream);

@@ -49,13 +49,46 @@ __device__ __forceinline__ long cell_at(int p, int pitch, long stride) {
   return (j - 2) * stride + (i - 2);
 }
 
+// two cells (i, j), (i + 1, j) of the result from their sums; c2: their classes
+__device__ __forceinline__ void apply_put(const ApplyArgs& A, double* __restrict__ out, int i, int j, uint32_t c2, double s0,
+                                          double s1) {
+  if (j >= A.ny || i >= A.nx) return;
+  // the fitted rows' cells are written by their own CTAs, or (transpose) by k_rows_T
+  const bool g0 = (c2 & 0xffu) != 2u, g1 = (c2 >> 8) != 2u && i + 1 < A.nx;
+  const double v0 = (c2 & 0xffu) ? A.scale * s0 : 0.0, v1 = (c2 >> 8) ? A.scale * s1 : 0.0;
+  double* o = out + (long)j * A.out.stride + i;
+  if (A.vec && g0 && g1) {
+    *reinterpret_cast<double2*>(o) = make_double2(v0, v1);
+  } else {
+    if (g0) o[0] = v0;
+    if (g1) o[1] = v1;
+  }
+}
+
+// the classes of the pairs of rows 2 k, 2 k + 1 are the halves of c2[k]
+__device__ __forceinline__ uint32_t pair_class(uint32_t ca, uint32_t cb, int kk) {
+  return ((kk < 2 ? ca : cb) >> (16 * (kk & 1))) & 0xffffu;
+}
+
+// a thread's cells that the integer form does not serve well; a call, so that this rare path takes no
+// registers from the common one
+template <bool CROSS>
+__device__ __noinline__ void apply_few(const ApplyArgs& A, const double* tile, const long long* ints, double* out, int cx0,
+                                       int cy0, uint32_t ca, uint32_t cb) {
+  const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
+  few_cells<CROSS>(tile, ints, x0, y0, A.S, A.Q, [&](int kk, int j) { return (pair_class(ca, cb, kk) >> (8 * j) & 0xffu) == 1u; },
+                   [&](int kk, int j, double s) { out[(long)(cy0 + y0 + kk) * A.out.stride + cx0 + x0 + j] = A.scale * s; });
+}
+
 // out = L u + N g (TRANS: L^T v on the cells that no fitted row's stencil reaches, and N^T v).
 // star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134 MB written (26 us at the copy rate):
-// 66 us, bound by the integer stencil's issue slots (85 us with the classes loaded first and cell by
-// cell, so that a tile took two round trips and 10 loads a thread in place of 5).
+// 71 us; without the look at the cells' sums 66 us (4 us of the difference its tests, which follow the
+// results, the rest the cells that fail them); with the classes loaded first and cell by cell, so that
+// a tile took two round trips and 10 loads a thread in place of 5, 85 us.
 template <bool CROSS, bool TRANS>
-__global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
+__global__ void __launch_bounds__(256, 3) k_apply(const __grid_constant__ ApplyArgs A) {
   __shared__ __align__(16) double tile[HY * HX];
+  __shared__ __align__(16) long long ints[HY * HX];
   __shared__ __align__(16) unsigned wmax[8];
   const int z = blockIdx.y;
   pdl_enter();
@@ -82,23 +115,9 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
   const int cx0 = (t % A.tx) * JX, cy0 = (t / A.tx) * JY;
   const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
   const int i0 = cx0 + x0;
-  auto put = [&](int kk, double s0, double s1, uint32_t c2) {
-    const int j = cy0 + y0 + kk;
-    if (j >= A.ny || i0 >= A.nx) return;
-    // the fitted rows' cells are written by their own CTAs, or (TRANS) by k_rows_T
-    const bool g0 = (c2 & 0xffu) != 2u, g1 = (c2 >> 8) != 2u && i0 + 1 < A.nx;
-    const double v0 = (c2 & 0xffu) ? A.scale * s0 : 0.0, v1 = (c2 >> 8) ? A.scale * s1 : 0.0;
-    double* o = out + (long)j * A.out.stride + i0;
-    if (A.vec && g0 && g1) {
-      *reinterpret_cast<double2*>(o) = make_double2(v0, v1);
-    } else {
-      if (g0) o[0] = v0;
-      if (g1) o[1] = v1;
-    }
-  };
   if (!A.act[t]) {
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) put(kk, 0.0, 0.0, 0u);
+    for (int kk = 0; kk < 4; ++kk) apply_put(A, out, i0, cy0 + y0 + kk, 0u, 0.0, 0.0);
     return;
   }
   uint32_t c2[2] = {0, 0};      // the classes of two rows' pairs each
@@ -141,9 +160,10 @@ __global__ void __launch_bounds__(256, 3) k_apply(ApplyArgs A) {
     __syncthreads();
   }
   // with pairs each thread reads back its own slots first (tile_stencil64's maximum): no barrier
-  tile_stencil64<CROSS>(tile, wmax, x0, y0, true, A.S, A.Q, [&](int kk, double s0, double s1) {
-    put(kk, s0, s1, ((kk < 2 ? c2[0] : c2[1]) >> (16 * (kk & 1))) & 0xffffu);
-  });
+  tile_stencil64<CROSS, true>(
+      tile, ints, wmax, x0, y0, true, A.S, A.Q,
+      [&](int kk, double s0, double s1) { apply_put(A, out, i0, cy0 + y0 + kk, pair_class(c2[0], c2[1], kk), s0, s1); },
+      [&] { apply_few<CROSS>(A, tile, ints, out, cx0, cy0, c2[0], c2[1]); });
 }
 
 // L^T v at the cells that the fitted rows' stencils reach (every irregular cell is one): the regular

@@ -5,25 +5,38 @@
 // bound every FP64 pass over a level (9.4 us per 64 x 32 tile and SM).  Integer adds run at
 // half the FP32 rate or better, so the stencil runs on fixed-point images of the staged values:
 //
-//   q = round(u 2^(57 - s)),  2^s the power of two above the largest |u| of the staged tile,
-//   Lap  = 16 (q_-1 + q_+1) - (q_-2 + q_+2) - 30 q_0      (eq. stdLap times 12; |Lap| < 2^63),
-//   Grad = (q_-2 - q_+2) + 8 (q_+1 - q_-1)                (eq. stdGrad times 12),
-//   h^2 L u = 2^.. (hi(A Lap_x) + hi(C Lap_y) + hi(B Grad_y(Grad_x / 8))),
+//   q = round(u 2^(60 - s)),  2^s the power of two above the largest |u| of the staged tile,
+//   Lap  = (q_-1 + q_+1 - 2 q_0) - (q_-2 + q_+2 - 2 q_0) / 16    (eq. stdLap times 12 / 16),
+//   Grad = (q_+1 - q_-1) + (q_-2 - q_+2) / 8                      (eq. stdGrad times 12 / 8),
+//   h^2 L u = 2^.. (hi(A Lap_x) + hi(C Lap_y) + hi(B Grad_y(Grad_x))),
 //
-// with A = a / 12, C = c / 12, B = 8 b / 144 as 62-bit integers on one common power of two and
-// hi() the upper half of the 128-bit product.  Lap and Grad are exact in q; what is rounded is
-// q (to 2^-58 of the tile's largest value; a value within 2^4 of the largest not at all),
-// Grad_x / 8, the three products and the conversion to FP64, each below that.  The FP64 sum
-// rounds every partial sum to 2^-53 of terms of the size of 30/12 u.  Errors against 128-bit
-// sums, relative 2-norm, FP64 / integer: plane waves 4e-12 / 6e-14, N(0, 1) values 1.6e-16 /
-// 4.8e-17, values that fall by e^40 over the tile 9.2e-16 / 9.4e-16.  Where |u| in a cell's
-// window is far below the tile's largest value the error stays 2^-58 of that value.  Tiles
-// that hold an infinity or a NaN, or whose largest value is outside 2^-800 .. 2^700, take the
+// with A = 16 a / 12, C = 16 c / 12, B = 64 b / 144 as 63-bit integers on one common power of two
+// and hi() the upper half of the 128-bit product.  All of it stays below 2^63 for |q| < 2^60.  What
+// is rounded is q (to 2^-61 of 2^s; a value within 2^7 of the largest not at all), the sixteenths
+// and the eighths, the three products and the conversion to FP64.
+//
+// These errors are relative to the tile's largest value, those of an FP64 sum to the cell's own
+// terms.  A pass whose results are the operator's values themselves (apply.cuh, a single sweep or
+// restriction) keeps the doubles beside the integers and looks at every cell (LOCAL): where the sum of
+// its |w u| is so small, against the tile's largest value, that their bound exceeds 3 2^-53 of that
+// sum (near a spike, in the tail of a narrow kernel, at some zeros of a smooth field: in one warp of 14
+// at most), the FP64 sum replaces the result (q_few).  Errors relative to a cell's sum of |w u| over the
+// tiles of random plane waves on 64^2 .. 4096^2 grids against 64-bit mantissas, rms / worst: FP64 sum
+// 4.5e-17 / 2.0e-16, this 0.1 - 0.6e-17 / 1.7e-16.  (q on 57 bits, Lap and Grad whole and no look at the
+// cell: 0.3 - 1.4e-17 / 1.0e-15, and no correct digit left in cells 2^-58 below the tile's largest.)
+//
+// Inside a solve no cell is looked at: everywhere in the tile the error is below the FP64 rounding
+// at its largest value, which the max-norm of the residual and the elliptic coupling of the cells see
+// just as well, and corrections that fall by decades within a tile are common on coarse levels (with
+// the look at every cell a star 1024^2 FP64 solve takes 12.7 ms, without 4.0).
+//
+// Tiles that hold an infinity or a NaN, or whose largest value is outside 2^-800 .. 2^700, take the
 // FP64 sum, and so do operators with a coefficient outside 2^-100 .. 2^100.
 #pragma once
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #ifdef __CUDACC__
 #define CCM_HD __host__ __device__ __forceinline__
@@ -35,14 +48,19 @@ namespace ccm {
 namespace dev {
 
 struct QStencil {
-  long long A = 0, C = 0, B = 0;   // a / 12, c / 12, b / 18 times 2^k
+  long long A = 0, C = 0, B = 0;   // 16 a / 12, 16 c / 12, 64 b / 144 times 2^k
   int cexp = 0;                    // the sum of the upper products times 2^(E - 1022 + cexp) is h^2 L u
   int ok = 0;                      // the coefficients are in range
+  // least sum of |w u| over 2^s for which the integer form is as accurate as the FP64 sum, the
+  // weights of the axis taps (centre, x +- 1, x +- 2, y +- 1, y +- 2), and the upper word of the
+  // centre's q for which its term alone is as much
+  float least = 0, wc = 0, wx1 = 0, wx2 = 0, wy1 = 0, wy2 = 0;
+  unsigned near = 0;
 };
 
 inline QStencil q_stencil(double a, double b, double c) {
   QStencil S;
-  const long double A = (long double)a / 12.0L, C = (long double)c / 12.0L, B = (long double)b / 18.0L;
+  const long double A = 16.0L * a / 12.0L, C = 16.0L * c / 12.0L, B = 64.0L * b / 144.0L;
   long double m = std::fabs(A);
   if (std::fabs(C) > m) m = std::fabs(C);
   if (std::fabs(B) > m) m = std::fabs(B);
@@ -50,12 +68,33 @@ inline QStencil q_stencil(double a, double b, double c) {
   int e = 0;
   std::frexp((double)m, &e);                    // m < 2^e (a rounding up to 2^e only widens it)
   if (e < -100 || e > 100) return S;
-  const int k = 62 - e;
-  S.A = (long long)std::llround(std::ldexp(A, k));
-  S.C = (long long)std::llround(std::ldexp(C, k));
-  S.B = (long long)std::llround(std::ldexp(B, k));
-  S.cexp = 64 - k - 57;
+  const int k = 63 - e;
+  const auto fix = [&](long double v) {
+    const long double t = std::ldexp(v, k);
+    return t >= 9223372036854775807.0L ? 9223372036854775807LL : t <= -9223372036854775807.0L ? -9223372036854775807LL
+                                                                                             : (long long)std::llround(t);
+  };
+  S.A = fix(A);
+  S.C = fix(C);
+  S.B = fix(B);
+  S.cexp = 64 - k - 60;
   S.ok = 1;
+  // The bound on the error in units of 2^(s - 60): the values' rounding, half a unit in every tap
+  // (64 / 12 in all along x and along y, 324 / 144 of the mixed term); the sixteenths' floors, times 16 / 12,
+  // up along x and down along y; the eighths' (at most 1.125 and 1 units, times 64 / 144); the products'
+  // floors, of 2^(1 + e): one down and one up, and another down with the mixed term.
+  const double ax = std::fabs(a), cy = std::fabs(c), bm = std::fabs(b), n = std::ldexp(1.0, -e);
+  const double bound = n * ((ax + cy) * 64 / 24 + (ax > cy ? ax : cy) * 16 / 12 + bm * (324.0 / 288 + 2.125 * 64 / 144)) +
+                       (b != 0 ? 4.0 : 2.0);
+  const double least = bound / (128.0 * 3);     // bound 2^-60 <= 3 2^-53 least, with 2^-e taken out
+  S.least = (float)(least * 1.0001);             // (its own and the sums' roundings in FP32)
+  S.wc = (float)(30.0 / 12 * n * std::fabs(a + c));
+  S.wx1 = (float)(16.0 / 12 * n * ax);
+  S.wx2 = (float)(1.0 / 12 * n * ax);
+  S.wy1 = (float)(16.0 / 12 * n * cy);
+  S.wy2 = (float)(1.0 / 12 * n * cy);
+  const double near = S.wc > 0 ? std::ceil(S.least / S.wc * 268435456.0) : 4e9;     // |q| >= 2^32 near
+  S.near = near < 4e9 ? (unsigned)near : 0xffffffffu;
   return S;
 }
 
@@ -71,7 +110,7 @@ CCM_HD int q_scale(unsigned m, const QStencil& S) {
 CCM_HD long long q_fixed(unsigned hi, unsigned lo, int E) {
   const unsigned mh = (hi << 11) | (lo >> 21) | 0x80000000u, ml = lo << 11;
   const unsigned long long m = ((unsigned long long)mh << 32) | ml;   // 1.f times 2^63
-  const unsigned sh = (unsigned)(E - (int)((hi >> 20) & 0x7ffu)) + 6u;
+  const unsigned sh = (unsigned)(E - (int)((hi >> 20) & 0x7ffu)) + 3u;
   unsigned long long q;
 #ifdef __CUDA_ARCH__
   asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m), "r"(sh));            // 0 from 64 on (zeros: 220 and up)
@@ -85,18 +124,35 @@ CCM_HD long long q_fixed(unsigned hi, unsigned lo, int E) {
 
 CCM_HD long long q_lap(long long m2, long long m1, long long c, long long p1, long long p2) {
   const long long c2 = c + c;
-  return (m1 + p1 - c2) * 16 - (m2 + p2 - c2);
+  return (m1 + p1 - c2) - ((m2 + p2 - c2) >> 4);
 }
-CCM_HD long long q_grad(long long m2, long long m1, long long p1, long long p2) { return (m2 - p2) + (p1 - m1) * 8; }
-CCM_HD long long q_grad8(long long m2, long long m1, long long p1, long long p2) {   // rounded eighth
-  return (q_grad(m2, m1, p1, p2) + 4) >> 3;
-}
+CCM_HD long long q_grad(long long m2, long long m1, long long p1, long long p2) { return (p1 - m1) + ((m2 - p2) >> 3); }
+CCM_HD long long q_grad8(long long m2, long long m1, long long p1, long long p2) { return q_grad(m2, m1, p1, p2); }
 CCM_HD long long q_hi(long long x, long long y) {
 #ifdef __CUDA_ARCH__
   return __mul64hi(x, y);
 #else
   return (long long)(((__int128)x * y) >> 64);
 #endif
+}
+
+// hi(A Lap_x) + hi(C Lap_y) from hx = hi(A Lap_x) and Lap_y of the negated values, so that the floors
+// along y go up where those along x go down and cancel on average (and zeros give 0)
+CCM_HD long long q_lap_neg(long long m2, long long m1, long long c, long long p1, long long p2) {
+  const long long c2 = c + c;
+  return (c2 - m1 - p1) - ((c2 - m2 - p2) >> 4);
+}
+CCM_HD long long q_axes(long long hx, long long neg_y, const QStencil& S) { return hx - q_hi(neg_y, S.C); }
+
+// |q| 2^-60 from the upper word of q, rounded down (a lone unit of it is 2^-28)
+CCM_HD float q_part(long long q) {
+  const int v = (int)(q >> 32);
+  return (float)(v ^ (v >> 31)) * 3.7252902984619140625e-9f;
+}
+// the sum of |w u| 2^-s over a cell's axis taps, a lower bound on all its taps' (c, and the sums of q_part at
+// x +- 1, x +- 2, y +- 1, y +- 2)
+CCM_HD float q_sum(const QStencil& S, float c, float x1, float x2, float y1, float y2) {
+  return S.wc * c + S.wx1 * x1 + S.wx2 * x2 + S.wy1 * y1 + S.wy2 * y2;
 }
 
 // x times 2^e as a double, rounded to nearest (ties away), for e that keeps it in the normal range
@@ -169,16 +225,22 @@ struct QSlots {
 // x0 even, on a staged tile q [.][ROW] of integers whose cell (0, 0) is at (2, 2): two columns
 // and four rows a thread, each staged row read as aligned pairs that serve both columns; the
 // rows' Lap_x and Grad_x are formed as a row enters and kept until their cells are complete.
-// emit(k, s0, s1).
-template <bool CROSS, int ROW, class Emit>
-__device__ __forceinline__ void q_rows(const long long* __restrict__ q, int x0, int y0, const QStencil& S, Emit emit) {
+// emit(k, s0, s1).  With LOCAL the result says whether every cell's own value alone is large enough
+// for the integer form (on the upper words, which are in registers: 2 operations a cell).
+template <bool CROSS, int ROW, bool LOCAL, class Emit>
+__device__ __forceinline__ bool q_rows(const long long* __restrict__ q, int x0, int y0, const QStencil& S, Emit emit) {
   long long c[2][8], d[2][8], X[2][4];
+  unsigned least = 0xffffffffu;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const longlong2* row = reinterpret_cast<const longlong2*>(q + (y0 + r) * ROW + x0);
     const longlong2 b = row[1];
     c[0][r] = b.x;
     c[1][r] = b.y;
+    if (LOCAL && r >= 2 && r < 6) {
+      const int v0 = (int)(b.x >> 32), v1 = (int)(b.y >> 32);
+      least = min(least, min((unsigned)(v0 ^ (v0 >> 31)), (unsigned)(v1 ^ (v1 >> 31))));
+    }
     if (CROSS || (r >= 2 && r < 6)) {
       const longlong2 a = row[0], e = row[2];
       if (CROSS) {
@@ -194,12 +256,57 @@ __device__ __forceinline__ void q_rows(const long long* __restrict__ q, int x0, 
       long long s[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        s[j] = X[j][r - 4] + q_hi(q_lap(c[j][r - 4], c[j][r - 3], c[j][r - 2], c[j][r - 1], c[j][r]), S.C);
+        s[j] = q_axes(X[j][r - 4], q_lap_neg(c[j][r - 4], c[j][r - 3], c[j][r - 2], c[j][r - 1], c[j][r]), S);
         if (CROSS) s[j] += q_hi(q_grad(d[j][r - 4], d[j][r - 3], d[j][r - 1], d[j][r]), S.B);
       }
       emit(r - 4, s[0], s[1]);
     }
   }
+  return !LOCAL || least >= S.near;
+}
+
+// Of these cells those whose sum of |w u| is too small for the integer form (bit 2 k + j: cell
+// (x0 + j, y0 + k)), less those of `skip`: first from the integers, then, as the integers of small values
+// are 0 too, without the cells whose taps are all 0 in the tile of doubles
+template <bool CROSS, int ROW>
+__device__ __forceinline__ unsigned q_few(const long long* __restrict__ q, const double* __restrict__ tile, int x0, int y0,
+                                          const QStencil& S, unsigned skip) {
+  float b[8][2], x1[4][2], x2[4][2];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const longlong2* row = reinterpret_cast<const longlong2*>(q + (y0 + r) * ROW + x0);
+    const longlong2 m = row[1];
+    b[r][0] = q_part(m.x);
+    b[r][1] = q_part(m.y);
+    if (r < 2 || r > 5) continue;
+    const longlong2 a = row[0], e = row[2];
+    const float a1 = q_part(a.y), e0 = q_part(e.x);
+    x1[r - 2][0] = a1 + b[r][1];
+    x1[r - 2][1] = b[r][0] + e0;
+    x2[r - 2][0] = q_part(a.x) + e0;
+    x2[r - 2][1] = a1 + q_part(e.y);
+  }
+  unsigned few = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      if (q_sum(S, b[k + 2][j], x1[k][j], x2[k][j], b[k + 1][j] + b[k + 3][j], b[k][j] + b[k + 4][j]) < S.least)
+        few |= 1u << (2 * k + j);
+  few &= ~skip;
+  for (unsigned m = few; m; m &= m - 1) {
+    const int t = __ffs(m) - 1;
+    const double* c = tile + (y0 + (t >> 1) + 2) * ROW + x0 + (t & 1) + 2;
+    bool any = c[0] != 0.0 || c[-1] != 0.0 || c[1] != 0.0 || c[-ROW] != 0.0 || c[ROW] != 0.0;
+    if (!any)
+#pragma unroll
+      for (int dj = -2; dj <= 2; ++dj)
+#pragma unroll
+        for (int di = -2; di <= 2; ++di)
+          if (CROSS || dj == 0 || di == 0) any |= c[dj * ROW + di] != 0.0;
+    if (!any) few &= ~(1u << t);
+  }
+  return few;
 }
 #endif
 

@@ -4,8 +4,8 @@
 //
 // GB300 issues FP64 at 1/64 of the FP32 rate, so the regular stencil runs in integer form
 // (fixed.cuh) on the TMA-staged tiles: 2 FP64 operations a cell are left (r_hat - L u_hat and
-// its rounding to FP32) of 19.  The kernel serves every tolerance: its error is below that of
-// the FP64 sum.
+// its rounding to FP32) of 19.  The kernel serves every tolerance: its error anywhere in a tile is below
+// the rounding of an FP64 sum at the tile's largest values.
 #pragma once
 
 #include "smooth.cuh"
@@ -93,7 +93,8 @@ __global__ void __launch_bounds__(256, 3) k_resid(const __grid_constant__ CUtens
     const int x0 = 2 * (threadIdx.x & 31), y0 = (threadIdx.x >> 5) * 4;
     const int i0 = cx0 + x0;
     float* r32 = A.r32 ? A.r32 + (long)z * A.bs : nullptr;
-    tile_stencil64<CROSS>(ut, wmax, x0, y0, i0 < A.nx, A.S, A.Q, [&](int kk, double s0, double s1) {
+    tile_stencil64<CROSS, false>(ut, reinterpret_cast<long long*>(ut), wmax, x0, y0, i0 < A.nx, A.S, A.Q,
+                                 [&](int kk, double s0, double s1) {
       const uint32_t c2 = *reinterpret_cast<const uint16_t*>(ct + (y0 + kk + 2) * CLX + x0 + 2);
       const double2 r2 = *reinterpret_cast<const double2*>(rt + (y0 + kk) * HX + x0 + 2);
       const double t0 = r2.x - s0, t1 = r2.y - s1;
@@ -109,7 +110,7 @@ __global__ void __launch_bounds__(256, 3) k_resid(const __grid_constant__ CUtens
           if (g1) r32[p + 1] = (float)t1;
         }
       }
-    });
+    }, [] {});
   }
   // one atomic a CTA, and none where the norm is already larger (all of them hit one word)
   __shared__ unsigned long long wm[8];

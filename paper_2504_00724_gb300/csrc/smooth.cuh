@@ -267,57 +267,75 @@ __device__ __forceinline__ void block_apply_part(const double* As, const double*
   }
 }
 
-// FP64 sum of the stencil on a staged tile in factored form (the x-derivative of each entering
-// row and 13 FMA per cell): the tiles that the integer form does not take
-template <bool CROSS, class Emit>
-__device__ __forceinline__ void fp64_rows(const double* __restrict__ tile, int x0, int y0, const Stencil<double>& S,
-                                          Emit emit) {
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    double s[2];
-#pragma unroll 1
-    for (int j = 0; j < 2; ++j) {
-      const double* c = tile + (y0 + k + 2) * HX + x0 + j + 2;
-      double acc = S.cc * c[0];
-      acc = fma(S.lx[0], c[-2], acc);
-      acc = fma(S.lx[1], c[-1], acc);
-      acc = fma(S.lx[3], c[1], acc);
-      acc = fma(S.lx[4], c[2], acc);
-      acc = fma(S.ly[0], c[-2 * HX], acc);
-      acc = fma(S.ly[1], c[-HX], acc);
-      acc = fma(S.ly[3], c[HX], acc);
-      acc = fma(S.ly[4], c[2 * HX], acc);
-      if (CROSS)
-        for (int dj = 0; dj < 5; ++dj) {
-          const double* r = c + (dj - 2) * HX;
-          if (dj != 2) acc = fma(S.gy[dj], S.gx[0] * r[-2] + S.gx[1] * r[-1] + S.gx[3] * r[1] + S.gx[4] * r[2], acc);
-        }
-      s[j] = acc;
+// FP64 sum of the stencil at a cell c of a staged tile, in factored form (the x-derivative of each row
+// and 13 FMA): the cells that the integer form does not take
+template <bool CROSS>
+__device__ __forceinline__ double fp64_sum(const double* __restrict__ c, const Stencil<double>& S) {
+  double acc = S.cc * c[0];
+  acc = fma(S.lx[0], c[-2], acc);
+  acc = fma(S.lx[1], c[-1], acc);
+  acc = fma(S.lx[3], c[1], acc);
+  acc = fma(S.lx[4], c[2], acc);
+  acc = fma(S.ly[0], c[-2 * HX], acc);
+  acc = fma(S.ly[1], c[-HX], acc);
+  acc = fma(S.ly[3], c[HX], acc);
+  acc = fma(S.ly[4], c[2 * HX], acc);
+  if (CROSS)
+    for (int dj = 0; dj < 5; ++dj) {
+      const double* r = c + (dj - 2) * HX;
+      if (dj != 2) acc = fma(S.gy[dj], S.gx[0] * r[-2] + S.gx[1] * r[-1] + S.gx[3] * r[1] + S.gx[4] * r[2], acc);
     }
-    emit(k, s[0], s[1]);
-  }
+  return acc;
 }
 
 // h^2 L u at the cells (x0, y0 + k) and (x0 + 1, y0 + k), k = 0 .. 3, of a staged tile of doubles
-// for all 256 threads of a CTA (x0, y0: two columns and four rows a thread): in integer form,
-// the tile's values replaced by their integers in place, or as an FP64 sum where that does not
-// apply (see fixed.cuh).  emit(k, Lu0, Lu1) only where on.  Barriers inside; a thread that needs
-// the tile's own values reads them before the call.
-template <bool CROSS, class Emit>
-__device__ __forceinline__ void tile_stencil64(double* tile, unsigned* wmax, int x0, int y0, bool on,
-                                               const Stencil<double>& S, const QStencil& Q, Emit emit) {
+// for all 256 threads of a CTA (x0, y0: two columns and four rows a thread): in integer form, or as
+// an FP64 sum where that does not apply (see fixed.cuh).  The integers go to q, with LOCAL an array
+// beside the tile, else the tile itself.  emit(k, Lu0, Lu1) only where on.  With LOCAL few() is called
+// afterwards by a thread with a cell whose own value is small; it looks at the cells' sums and replaces
+// what it must (few_cells).  Barriers inside; without LOCAL a thread that needs the tile's
+// own values reads them before the call.
+template <bool CROSS, bool LOCAL, class Emit, class Few>
+__device__ __forceinline__ void tile_stencil64(double* tile, long long* q, unsigned* wmax, int x0, int y0, bool on,
+                                               const Stencil<double>& S, const QStencil& Q, Emit emit, Few few) {
   constexpr int NP = HY * HX / 2;
   QSlots<(NP + 255) / 256> v;
-  const int E = q_scale(q_cta_max(v.load(tile, NP), wmax), Q);
+  const unsigned m = q_cta_max(v.load(tile, NP), wmax);
+  const int E = q_scale(m, Q);
   if (E < 0) {
-    if (on) fp64_rows<CROSS>(tile, x0, y0, S, emit);
+    if (on)
+#pragma unroll 1
+      for (int k = 0; k < 4; ++k) {
+        double s[2];
+#pragma unroll 1
+        for (int j = 0; j < 2; ++j) s[j] = fp64_sum<CROSS>(tile + (y0 + k + 2) * HX + x0 + j + 2, S);
+        emit(k, s[0], s[1]);
+      }
     return;
   }
-  long long* q = reinterpret_cast<long long*>(tile);
   v.store(q, NP, E);
   __syncthreads();
   const int e = E - 1022 + Q.cexp;
-  if (on) q_rows<CROSS, HX>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
+  if (on) {
+    const bool ok = q_rows<CROSS, HX, LOCAL>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
+    if (LOCAL && !ok && m != 0) few();
+  }
+}
+
+// FP64 sums for those of a thread's cells that the caller needs and whose sum of |w u| is too small for
+// the integer form: one(k, j, Lu), need(k, j): cell (x0 + j, y0 + k)
+template <bool CROSS, class Need, class One>
+__device__ __forceinline__ void few_cells(const double* tile, const long long* q, int x0, int y0, const Stencil<double>& S,
+                                          const QStencil& Q, Need need, One one) {
+  unsigned skip = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) skip |= need(t >> 1, t & 1) ? 0u : 1u << t;
+  if (skip == 255u) return;
+  const unsigned few = q_few<CROSS, HX>(q, tile, x0, y0, Q, skip);
+#pragma unroll 1
+  for (int t = 0; t < 8; ++t)
+    if (few >> t & 1)
+      one(t >> 1, t & 1, fp64_sum<CROSS>(tile + (y0 + (t >> 1) + 2) * HX + x0 + (t & 1) + 2, S));
 }
 
 // FP32: h^2 L u at the cells (x0, y0 + k) and (x0 + 1, y0 + k), k = 0 .. 3, of a staged tile.
@@ -369,8 +387,8 @@ __device__ __forceinline__ void stencil32(const float* __restrict__ tile, int x0
 // SMO-1 on the regular cells of a staged 64 x 32 tile (halo box of u, box of r and class bytes
 // at the TileStage offsets of st; with PRO the coarse box too, whose parent values are first
 // added to the staged regular cells: the sweep then reads u + P uc)
-template <typename T, bool CROSS, bool PRO>
-__device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char* st, int cx0, int cy0,
+template <typename T, bool CROSS, bool PRO, bool LOCAL>
+__device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char* st, long long* q, int cx0, int cy0,
                                            T* __restrict__ u_new, double* __restrict__ uhat, unsigned* wmax) {
   using S = TileStage<T>;
   T* tile = reinterpret_cast<T*>(st);
@@ -426,11 +444,19 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
     V2 c[4];
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) c[kk] = *reinterpret_cast<const V2*>(tile + (y0 + kk + 2) * HX + x0 + 2);
-    tile_stencil64<CROSS>(tile, wmax, x0, y0, i0 < a.nx, a.S, a.Q, [&](int kk, double s0, double s1) {
+    if (!LOCAL) q = reinterpret_cast<long long*>(tile);
+    const auto emit = [&](int kk, double s0, double s1) {
       const V2 r2 = *reinterpret_cast<const V2*>(rt + (y0 + kk) * HX + x0 + 2);
       const V2 u = kk == 0 ? c[0] : kk == 1 ? c[1] : kk == 2 ? c[2] : c[3];
       put(kk, u.x + a.S.omega_d * (r2.x - s0), u.y + a.S.omega_d * (r2.y - s1));
-    });
+    };
+    const auto need = [&](int kk, int j) { return ct[(y0 + kk + 2) * CLX + x0 + j + 2] == 1; };
+    const auto one = [&](int kk, int j, double s) {      // (a needed cell: regular, in the grid)
+      const double u = tile[(y0 + kk + 2) * HX + x0 + j + 2], r = rt[(y0 + kk) * HX + x0 + j + 2];
+      u_new[(long)(cy0 + y0 + kk + 2) * a.pitch + (i0 + j + 2)] = u + a.S.omega_d * (r - s);
+    };
+    tile_stencil64<CROSS, LOCAL>(tile, q, wmax, x0, y0, i0 < a.nx, a.S, a.Q, emit,
+                                 [&] { if constexpr (LOCAL) few_cells<CROSS>(tile, q, x0, y0, a.S, a.Q, need, one); });
   } else {
     // FP32: two adjacent cells (x0, x0 + 1) in four rows per thread; class bytes, right-hand sides
     // and new values move in pairs.  A thread whose eight cells are all regular (most are) stores
@@ -492,7 +518,9 @@ __device__ __forceinline__ void tile_sweep(const SweepArgs<T>& a, unsigned char*
 // serves all of them with one copy of its inverse rows (28 KB; one right-hand side at a time
 // these copies were two fifths of a sweep's L2 reads), then come the tile items of the first, the
 // second, ...
-template <typename T, bool CROSS, bool PRO, int R = 1>
+// LOCAL (FP64, one sweep by itself): the regular cells' stencil as accurate cell by cell as an FP64
+// sum (tile_stencil64), with the integers after the blocks' scratch; that leaves one CTA an SM
+template <typename T, bool CROSS, bool PRO, int R = 1, bool LOCAL = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __grid_constant__ CUtensorMap tin,
                                                 const __grid_constant__ CUtensorMap tr,
                                                 const __grid_constant__ CUtensorMap tcls,
@@ -552,6 +580,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
   T* sres = reinterpret_cast<T*>(smem_raw + 2 * A.stage);
   T* sold = reinterpret_cast<T*>(smem_raw + 2 * A.stage + R * slot);
   int* scell = reinterpret_cast<int*>(smem_raw + 2 * A.stage + 2 * R * slot);
+  long long* ints = reinterpret_cast<long long*>(smem_raw + 2 * A.stage + (2 * R + 1) * slot);     // LOCAL
   if (threadIdx.x == 0) {
     issue(0, 0, 0, 2);
     if (KS > 1) issue(1, 1, 1, 2);
@@ -594,7 +623,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
       }
     } else {
       const long bo = rhs_of(item) * a.bs;
-      tile_sweep<T, CROSS, PRO>(a, smem_raw + sb * A.stage, cx0, cy0, a.u_new + bo, a.uhat ? a.uhat + bo : nullptr, wmax);
+      tile_sweep<T, CROSS, PRO, LOCAL>(a, smem_raw + sb * A.stage, ints, cx0, cy0, a.u_new + bo,
+                                       a.uhat ? a.uhat + bo : nullptr, wmax);
     }
     __syncthreads();      // stage sb is free
     if (threadIdx.x == 0 && k + 2 < KS) {
@@ -694,7 +724,7 @@ __device__ __forceinline__ void prefetch_tile_rows(const RestrictArgs<T>& A, int
   }
 }
 
-template <typename T, bool CROSS>
+template <typename T, bool CROSS, bool LOCAL = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(const __grid_constant__ CUtensorMap tin,
                                                        const __grid_constant__ CUtensorMap tr,
                                                        const __grid_constant__ CUtensorMap tcls,
@@ -812,8 +842,18 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_restrict_p(cons
     };
     if constexpr (sizeof(T) == 4)
       stencil32<CROSS>(tile, x0, y1, A.S, [&](int kk, float2 s, float2) { resid(kk, s.x, s.y); });
-    else
-      tile_stencil64<CROSS>(tile, wmax, x0, y1, true, A.S, A.Q, resid);
+    else {
+      long long* ints = reinterpret_cast<long long*>(LOCAL ? smem_raw + 2 * A.stage : st);
+      const auto need = [&](int kk, int j) { return ct[(y1 + kk + 2) * CLX + x0 + j + 2] == 1; };
+      const auto one = [&](int kk, int j, double s) {
+        const double t = rt[(y1 + kk) * HX + x0 + j + 2] - s;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k == kk) (j ? rs[k].y : rs[k].x) = t;
+      };
+      tile_stencil64<CROSS, LOCAL>(tile, ints, wmax, x0, y1, true, A.S, A.Q, resid,
+                                   [&] { if constexpr (LOCAL) few_cells<CROSS>(tile, ints, x0, y1, A.S, A.Q, need, one); });
+    }
     if (k + 1 < K) prefetch_tile_rows(A, n0, n1);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

@@ -233,6 +233,7 @@ struct ccm_handle {
   // fold_next (level 0), it also adds its new values to u_hat (the outer iteration's update).
   // fold_last marks the last inner cycle; folded reports that a sweep took the update.
   bool zero_u_next = false, fold_next = false, fold_last = false, folded = false;
+  bool local = false;          // the FP64 pass being issued is a call of its own: accurate cell by cell
   long long cap_launches = 0;
   struct Graph {
     cudaGraphExec_t exec = nullptr;
@@ -249,6 +250,17 @@ struct ccm_handle {
 namespace {
 
 inline int ceil_div(long a, long b) { return (int)((a + b - 1) / b); }
+
+// dynamic shared memory that the FP64 passes take more where they are accurate cell by cell (the tile's
+// integers beside its doubles)
+constexpr size_t LOCAL_SMEM = dev::HY * dev::HX * sizeof(long long);
+
+// the FP64 passes issued while it lives are calls of their own, not part of a cycle
+struct LocalScope {
+  ccm_handle* h;
+  explicit LocalScope(ccm_handle* h) : h(h) { h->local = true; }
+  ~LocalScope() { h->local = false; }
+};
 
 // CTAs per right-hand side of a persistent launch: every item gets its own CTA up to the
 // resident capacity shared by the nb right-hand sides, and at most the handle's launch cap
@@ -442,6 +454,15 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
     }
   }
   const dim3 grid(ctas, H->nb);
+  if constexpr (sizeof(T) == 8)
+    if (H->local) {
+      auto go_local = [&](auto kernel) { KL(launch_k(kernel, grid, 256, smem + LOCAL_SMEM, s, tm, tr, L.tmcls, tu, A)); };
+      if (C && H->cross) go_local(dev::k_smooth<T, true, true, 1, true>);
+      else if (C) go_local(dev::k_smooth<T, false, true, 1, true>);
+      else if (H->cross) go_local(dev::k_smooth<T, true, false, 1, true>);
+      else go_local(dev::k_smooth<T, false, false, 1, true>);
+      return;
+    }
   if (C && H->cross) go(dev::k_smooth<T, true, true>, grid);
   else if (C) go(dev::k_smooth<T, false, true>, grid);
   else if (H->cross) go(dev::k_smooth<T, true, false>, grid);
@@ -619,6 +640,13 @@ void restrict_to(ccm_handle* H, DevLevel& F, DevLevel& C, cudaStream_t s) {
     const CUtensorMap& tv = kk == 0 ? F.tmv64 : F.tmv32;
     const size_t smem = 2 * (size_t)A.stage;
     const dim3 rgrid(persistent_ctas(F.restrict_grid[kk], F.restrict_cap[kk], H->nb, H->launch_cap), H->nb);
+    if constexpr (sizeof(T) == 8)
+      if (H->local) {
+        auto go = [&](auto kernel) { KL(launch_k(kernel, rgrid, 256, smem + LOCAL_SMEM, s, TmU<T>(F), TmR<T>(F), F.tmcls, tv, A)); };
+        if (H->cross) go(dev::k_restrict_p<T, true, true>);
+        else go(dev::k_restrict_p<T, false, true>);
+        return;
+      }
     if (H->cross)
       KL(launch_k(dev::k_restrict_p<T, true>, rgrid, 256, smem, s, TmU<T>(F), TmR<T>(F), F.tmcls, tv, A));
     else
@@ -1033,8 +1061,11 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
       auto fn = h->cross ? dev::k_smooth<double, true, true> : dev::k_smooth<double, false, true>;
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
-      for (auto g : {h->cross ? dev::k_smooth<double, true, false> : dev::k_smooth<double, false, false>})
-        cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      auto gn = h->cross ? dev::k_smooth<double, true, false> : dev::k_smooth<double, false, false>;
+      cudaFuncSetAttribute(gn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      auto lp = h->cross ? dev::k_smooth<double, true, true, 1, true> : dev::k_smooth<double, false, true, 1, true>;
+      auto ln = h->cross ? dev::k_smooth<double, true, false, 1, true> : dev::k_smooth<double, false, false, 1, true>;
+      for (auto g : {lp, ln}) cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + LOCAL_SMEM);
     } else {
       auto fn = h->cross ? dev::k_smooth<float, true, true> : dev::k_smooth<float, false, true>;
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -1387,6 +1418,8 @@ int upload_hierarchy(ccm_handle* h) {
           auto fn = h->cross ? dev::k_restrict_p<double, true> : dev::k_restrict_p<double, false>;
           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
+          auto lo = h->cross ? dev::k_restrict_p<double, true, true> : dev::k_restrict_p<double, false, true>;
+          cudaFuncSetAttribute(lo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + LOCAL_SMEM));
         } else {
           auto fn = h->cross ? dev::k_restrict_p<float, true> : dev::k_restrict_p<float, false>;
           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2774,6 +2807,7 @@ int ccm_level_apply(ccm_handle* h, int level, const double* u, double* out, void
 int ccm_level_smooth(ccm_handle* h, int level, double* u, const double* r, int precision, void* stream) {
   if (check_level(h, level) || !u || !r || level == (int)h->L.size() - 1) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  const LocalScope local(h);
   DevLevel& L = h->L[level];
   dim3 pg(ceil_div(L.nx, 128), L.ny);
   if (precision == CCM_FP64) {
@@ -2792,6 +2826,7 @@ int ccm_level_smooth(ccm_handle* h, int level, double* u, const double* r, int p
 int ccm_level_restrict(ccm_handle* h, int level, const double* u, const double* r, double* rc, void* stream) {
   if (check_level(h, level) || level == (int)h->L.size() - 1 || !u || !r || !rc) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  const LocalScope local(h);
   DevLevel& F = h->L[level];
   DevLevel& C = h->L[level + 1];
   load_level<double>(h, F, u, r, s);
@@ -2821,6 +2856,7 @@ int ccm_level_prolong_smooth(ccm_handle* h, int level, double* u, const double* 
                              void* stream) {
   if (check_level(h, level) || level == (int)h->L.size() - 1 || !u || !uc || !r) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  const LocalScope local(h);
   DevLevel& F = h->L[level];
   DevLevel& C = h->L[level + 1];
   dim3 pg(ceil_div(F.nx, 128), F.ny);
