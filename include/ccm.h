@@ -433,6 +433,11 @@ int ccm_fmg(ccm_handle* h, double* u, const double* r, int precision, void* stre
  * returns, so the context stays usable.  Returns CCM_ETIMEOUT (the expected outcome; the error
  * word is cleared again), CCM_OK if the wait did not run out, or CCM_ECUDA.  Blocking. */
 int ccm_wait_selftest(ccm_handle* h, void* stream);
+/* Test of the path without memory: the next `count` requests for set-up scratch on the device (the
+ * small levels' matrix of any handle, at set-up and in ccm_set_cycle_params and ccm_set_smo2_blocks)
+ * report that there is none.  Such a handle first tries with less, then runs the levels' sweeps; no
+ * call fails for it.  Host-only.  Errors: CCM_EINVAL. */
+int ccm_fail_scratch(int count);
 
 /* ---- accounting and profiling (not part of the method).
  * ccm_launch_count: kernels launched by this library in this process so far (all handles).

@@ -120,6 +120,7 @@ _SIGS = {
     "ccm_apply_noalloc": (I, [P, P, P, P, P]),
     "ccm_profile": (I, [P, I]),
     "ccm_wait_selftest": (I, [P, P]),
+    "ccm_fail_scratch": (I, [I]),
     "ccm_profile_read": (I, [P, ctypes.POINTER(ctypes.c_double), I64P]),
     "ccm_group_create": (I, [P, I, P, ctypes.POINTER(P)]),
     "ccm_group_solve": (I, [P, P, P, P, P, ctypes.POINTER(ccm_stats)]),

@@ -146,6 +146,17 @@ struct Arena {
     bytes += n * (long)sizeof(T);
     return (T*)p;
   }
+  // the same for what the caller can do without: null where there is no room, and no error
+  template <typename T>
+  T* try_alloc(long n) {
+    const cudaError_t before = err;
+    T* p = alloc<T>(n);
+    if (before == cudaSuccess && err == cudaErrorMemoryAllocation) {
+      err = cudaSuccess;
+      cudaGetLastError();
+    }
+    return p;
+  }
   // give one earlier allocation back (nullptr: nothing)
   void free(void* p) {
     if (!p) return;
@@ -1092,6 +1103,15 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   cudaGetLastError();
 }
 
+// set-up scratch; ccm_fail_scratch makes the next requests report that there is no memory
+std::atomic<int> g_fail_scratch{0};
+cudaError_t scratch_malloc(void** p, size_t bytes) {
+  int n = g_fail_scratch.load();
+  while (n > 0)
+    if (g_fail_scratch.compare_exchange_weak(n, n - 1)) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 // unknowns up to which the small levels' part of a V-cycle is applied as a dense matrix.  FP32
 // V-cycle of the star 256^2 (1.2k unknowns at 64^2): 108 -> 54 us.  At 3.7k unknowns (55 MB) a
 // single solve still gains (three ellipses 1024^2: 148 -> 137 us a V-cycle), but twelve problems
@@ -1101,9 +1121,11 @@ constexpr int DENSE_MAX = 2048;
 // (Re)build the dense matrix of the V-cycle from the first level below the finest with at most
 // DENSE_MAX unknowns, for the handle's cycle parameters and SMO-2 blocks.  Block-Jacobi smoother
 // only, and not where the caller asked for the cluster cycle.  A rebuilt matrix keeps its place
-// (the level does not depend on either).  Synchronises the device.
+// (the level does not depend on either).  Where there is no memory for it or for its set-up the
+// handle is left without one and the levels' sweeps run; that is no error.  Synchronises the device.
 int build_dense(ccm_handle* h) {
   ccm_handle::Dense& D = h->dense;
+  D.m = -1;
   Arena& A = h->arena;
   const int nl = (int)h->H.levels.size();
   if (h->par.smoother != 1 || h->par.ras_passes > 1 || h->par.coarse_n > 0) return CCM_OK;
@@ -1157,11 +1179,18 @@ int build_dense(ccm_handle* h) {
   a.n = n;
   a.S = h->S64;
   a.stride = (off + 15) & ~15L;
-  if (D.m < 0) {
-    D.cell = A.upload(cell);
+  if (!D.cell) {
     D.ld = (n + 3) & ~3;
-    if (h->par.precision == CCM_FP64) D.m64 = A.alloc<double>((long)n * D.ld);
-    else D.m32 = A.alloc<float>((long)n * D.ld);
+    D.cell = A.try_alloc<int32_t>(n);
+    if (h->par.precision == CCM_FP64) D.m64 = A.try_alloc<double>((long)n * D.ld);
+    else D.m32 = A.try_alloc<float>((long)n * D.ld);
+    if (A.err != cudaSuccess) return CCM_ECUDA;
+    if (!D.cell || !(D.m64 || D.m32)) {
+      for (void* p : {(void*)D.cell, (void*)D.m64, (void*)D.m32}) A.free(p);
+      D = {};
+      return CCM_OK;
+    }
+    if (cudaMemcpy(D.cell, cell.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) return CCM_ECUDA;
   }
   a.ld = D.ld;
   a.cell = D.cell;
@@ -1169,10 +1198,20 @@ int build_dense(ccm_handle* h) {
   a.out32 = D.m32;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
-  const int ctas = std::min(n, std::max(1, 2 * nsm));
-  if (A.err == cudaSuccess) A.err = cudaMalloc(&a.scratch, (size_t)ctas * a.stride * sizeof(double));
-  if (A.err != cudaSuccess) return A.err == cudaErrorMemoryAllocation ? CCM_ENOMEM : CCM_ECUDA;
-  cudaError_t e = cudaMemset(a.scratch, 0, (size_t)ctas * a.stride * sizeof(double));
+  // two CTAs an SM, or as many as there is scratch for
+  int ctas = std::min(n, std::max(1, 2 * nsm));
+  cudaError_t e = scratch_malloc((void**)&a.scratch, (size_t)ctas * a.stride * sizeof(double));
+  while (e == cudaErrorMemoryAllocation && ctas > 1) {
+    cudaGetLastError();
+    ctas = (ctas + 1) / 2;
+    e = scratch_malloc((void**)&a.scratch, (size_t)ctas * a.stride * sizeof(double));
+  }
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return CCM_OK;
+  }
+  if (e != cudaSuccess) return CCM_ECUDA;
+  e = cudaMemset(a.scratch, 0, (size_t)ctas * a.stride * sizeof(double));
   if (e == cudaSuccess) {
     if (h->cross) KL(dev::k_dense_columns<true><<<ctas, dev::DENSE_THREADS>>>(a));
     else KL(dev::k_dense_columns<false><<<ctas, dev::DENSE_THREADS>>>(a));
@@ -2115,6 +2154,12 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap) {
     t->info.device_bytes = t->arena.bytes;
   }
   return cudaDeviceSynchronize() == cudaSuccess ? CCM_OK : CCM_ECUDA;
+}
+
+int ccm_fail_scratch(int count) {
+  if (count < 0) return CCM_EINVAL;
+  g_fail_scratch.store(count);
+  return CCM_OK;
 }
 
 int ccm_set_launch_cap(ccm_handle* h, int max_ctas) {
