@@ -312,7 +312,10 @@ int ccm_solve_host(ccm_handle* h, const double* f, const double* g, double* u, i
  * convergence test moves from the host to the device.
  * ccm_group_create captures every member's iteration (it synchronises `stream` and uses
  * each member's private capture stream; call it outside any stream capture, after
- * ccm_set_cycle_params).  members[] is copied; the handles must outlive the group, and no
+ * ccm_set_cycle_params).  The group keeps that cycle: a later ccm_set_cycle_params or
+ * ccm_set_smo2_blocks of a member changes the member's own solves only (the memory that the group
+ * reads is given back by the first such call after the group is freed, or with the member).
+ * members[] is copied; the handles must outlive the group, and no
  * other call may use them while a group solve is in flight.  Errors: CCM_EINVAL (NULL, a
  * handle given twice), CCM_ENOMEM, CCM_ECUDA (the runtime rejected the graph).
  * ccm_group_solve: f[k], u[k] device [ny_k][nx_k] and g[k] device [n_segments_k] (g or

@@ -226,6 +226,9 @@ struct ccm_handle {
     double* m64 = nullptr;
     float* m32 = nullptr;
   } dense;
+  std::shared_ptr<int> groups = std::make_shared<int>(0);   // shared with the groups that captured this handle
+  bool matrix_captured = false, blocks_captured = false;   // a group's graph reads the current ones
+  std::vector<void*> kept;     // replaced ones that a group's graph may still read
   int launch_cap = 0;          // > 0: at most this many CTAs per right-hand side in the persistent kernels
   // GMRES(kry_m) correction of the mixed outer iteration (0: plain iterative refinement)
   int kry_m = 0;
@@ -1015,12 +1018,37 @@ bool make_tmap(CUtensorMap* map, void* base, int pitch, int rows, bool fp64, int
                    fp64 ? 8 : 4, dev::HX, dev::HY, depth);
 }
 
-// device copies of level m's SMO-2 blocks (the ones of a previous call are given back)
-int upload_blocks(ccm_handle* h, int m) {
+// A group's graph keeps the cycle that it captured: what it reads of a handle's matrix and SMO-2 blocks
+// is set aside when they change (the handle gets new memory for them), until a later change finds no
+// group left or the handle is freed.
+void drop_kept(ccm_handle* h) {
+  if (h->groups.use_count() > 1) return;
+  for (void* p : h->kept) h->arena.free(p);
+  h->kept.clear();
+  h->matrix_captured = h->blocks_captured = false;
+}
+
+void set_matrix_aside(ccm_handle* h) {
+  drop_kept(h);
+  if (!h->matrix_captured) return;
+  auto& D = h->dense;
+  for (void* p : {(void*)D.m64, (void*)D.m32})
+    if (p) h->kept.push_back(p);
+  D.m = -1;
+  D.m64 = nullptr;
+  D.m32 = nullptr;
+  h->matrix_captured = false;
+}
+
+// device copies of level m's SMO-2 blocks (the ones of a previous call are given back, or kept)
+int upload_blocks(ccm_handle* h, int m, bool keep = false) {
   Arena& A = h->arena;
   const HostLevel& hl = h->H.levels[m];
   DevLevel& d = h->L[m];
-  for (void* p : {(void*)d.order, (void*)d.blk, (void*)d.blk_off, (void*)d.inv64, (void*)d.inv32}) A.free(p);
+  for (void* p : {(void*)d.order, (void*)d.blk, (void*)d.blk_off, (void*)d.inv64, (void*)d.inv32}) {
+    if (keep && p) h->kept.push_back(p);
+    else A.free(p);
+  }
   d.order = d.blk = nullptr;
   d.blk_off = nullptr;
   d.inv64 = nullptr;
@@ -1179,17 +1207,13 @@ int build_dense(ccm_handle* h) {
   a.n = n;
   a.S = h->S64;
   a.stride = (off + 15) & ~15L;
-  if (!D.cell) {
+  if (!D.cell || !(D.m64 || D.m32)) {
     D.ld = (n + 3) & ~3;
-    D.cell = A.try_alloc<int32_t>(n);
-    if (h->par.precision == CCM_FP64) D.m64 = A.try_alloc<double>((long)n * D.ld);
-    else D.m32 = A.try_alloc<float>((long)n * D.ld);
+    if (!D.cell) D.cell = A.try_alloc<int32_t>(n);
+    if (h->par.precision == CCM_FP64 && !D.m64) D.m64 = A.try_alloc<double>((long)n * D.ld);
+    if (h->par.precision != CCM_FP64 && !D.m32) D.m32 = A.try_alloc<float>((long)n * D.ld);
     if (A.err != cudaSuccess) return CCM_ECUDA;
-    if (!D.cell || !(D.m64 || D.m32)) {
-      for (void* p : {(void*)D.cell, (void*)D.m64, (void*)D.m32}) A.free(p);
-      D = {};
-      return CCM_OK;
-    }
+    if (!D.cell || !(D.m64 || D.m32)) return CCM_OK;
     if (cudaMemcpy(D.cell, cell.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) return CCM_ECUDA;
   }
   a.ld = D.ld;
@@ -2138,18 +2162,22 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap) {
   for (ccm_handle* t : {h, h->adj}) {
     if (!t) continue;
     drop_graphs(t);
+    drop_kept(t);
+    const bool keep = t->blocks_captured;
+    t->blocks_captured = false;
     const int nl = (int)t->H.levels.size();
     for (int m = 0; m + 1 < nl; ++m) {
       HostLevel& hl = t->H.levels[m];
       if (hl.n2 == 0 || hl.n2 <= t->par.ras_exact) continue;
       std::string err;
       int rc = build_smo2_blocks(hl, block, overlap, t->par.nthreads, err);
-      if (!rc) rc = upload_blocks(t, m);
+      if (!rc) rc = upload_blocks(t, m, keep);
       if (rc) return rc;
       configure_sweep(t, t->L[m], nsm);
     }
     t->par.ras_block = block;
     t->par.ras_overlap = overlap;
+    set_matrix_aside(t);
     if (int rc = build_dense(t)) return rc;
     t->info.device_bytes = t->arena.bytes;
   }
@@ -2217,6 +2245,7 @@ int ccm_set_cycle_params(ccm_handle* h, double omega, int nu1, int nu2, int inne
       t->S64.omega_d = omega / w22;
       t->S32.omega_d = (float)(omega / w22);
     }
+    set_matrix_aside(t);
     if (int rc = build_dense(t)) return rc;
     t->info.device_bytes = t->arena.bytes;
   }
@@ -2444,6 +2473,7 @@ int ccm_solve_zero(ccm_handle* h, const double* f, const double* g, double* u, i
 
 struct ccm_group {
   std::vector<ccm_handle*> m;
+  std::vector<std::shared_ptr<int>> held;   // the members keep what the graph reads while these live
   std::vector<double*> u0;            // per member: the level-0 FP64 iterate its iteration updates
   std::vector<long long> launches;    // per member: kernel launches of one outer iteration
   cudaGraphExec_t exec = nullptr;
@@ -2603,6 +2633,10 @@ int ccm_group_create(ccm_handle* const* members, int count, void* stream, ccm_gr
       cudaMallocHost(&G->h_hist, (long)n * dev::GROUP_HIST * sizeof(double)) != cudaSuccess) {
     ccm_group_free(G.release());
     return CCM_ENOMEM;
+  }
+  for (ccm_handle* h : G->m) {
+    G->held.push_back(h->groups);
+    h->matrix_captured = h->blocks_captured = true;
   }
   int rc = build_group_graph(G.get(), s);
   if (rc == CCM_ECUDA) {
