@@ -49,11 +49,13 @@ struct DevLevel {
   CUtensorMap tmuc64[2], tmuc32[2];  // 36 x 18 boxes over level m + 1's u buffers
   bool tma_pro = false;         // the maps above exist: prolongation fuses into the sweep
   CUtensorMap tmr64, tmr32;     // 68 x 32 boxes over r
-  bool smooth_ok[2] = {false, false};  // persistent sweep (k_smooth) usable, [0] FP64, [1] FP32
-  uint32_t smooth_stage[2] = {0, 0};
-  size_t smooth_smem[2] = {0, 0};
-  int smooth_grid[2] = {0, 0};
-  int smooth_cap[2] = {0, 0};   // resident CTAs of the persistent sweep over the whole GPU
+  // persistent sweep (k_smooth) usable, and its launch shape: [0] FP64, [1] FP32, [2] FP32 with block
+  // items shared by BATCH_SHARE right-hand sides
+  bool smooth_ok[3] = {false, false, false};
+  uint32_t smooth_stage[3] = {0, 0, 0};
+  size_t smooth_smem[3] = {0, 0, 0};
+  int smooth_grid[3] = {0, 0, 0};
+  int smooth_cap[3] = {0, 0, 0};   // resident CTAs of the persistent sweep over the whole GPU
   double* rw64 = nullptr;       // restriction weights of the cells (levels with k_restrict_p)
   float* rw32 = nullptr;
   CUtensorMap tmv64, tmv32;     // 68 x 32 boxes over them
@@ -407,7 +409,7 @@ template <> const CUtensorMap& TmR<float>(const DevLevel& L) { return L.tmr32; }
 // the persistent sweep (k_smooth): SMO-2 block items and TMA tile items in one launch
 template <typename T>
 void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
-  const int k = sizeof(T) == 8 ? 0 : 1;
+  const int k = sizeof(T) == 8 ? 0 : H->nb >= dev::BATCH_SHARE && L.smooth_ok[2] ? 2 : 1;
   dev::SmoothArgs<T> A{};
   dev::SweepArgs<T>& a = A.a;
   a.tiles = L.tiles64;
@@ -458,7 +460,7 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   auto go = [&](auto kernel, dim3 grid) { KL(launch_k(kernel, grid, 256, smem, s, tm, tr, L.tmcls, tu, A)); };
   if constexpr (sizeof(T) == 4) {
     constexpr int R = dev::BATCH_SHARE;
-    if (H->nb >= R) {       // groups of R right-hand sides, with the CTAs of R
+    if (k == 2) {           // groups of R right-hand sides, with the CTAs of R
       const dim3 grid(std::min(ctas * R, A.nbi + R * L.ntiles64), ceil_div(H->nb, R));
       if (C && H->cross) go(dev::k_smooth<T, true, true, R>, grid);
       else if (C) go(dev::k_smooth<T, false, true, R>, grid);
@@ -1075,15 +1077,17 @@ int upload_blocks(ccm_handle* h, int m, bool keep = false) {
 
 // launch shape of a level's persistent sweep: two stages that hold a tile item or a block item,
 // one CTA-wide item at a time (blocks with more core rows than one CTA covers keep the older
-// path), as many CTAs as stay resident
+// path), as many CTAs as stay resident.  A handle with a batch keeps the shape of single right-hand
+// sides beside that of shared block items, whose scratch is four times as large.
 void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   const size_t need = (size_t)d.max_ext * d.max_core * sizeof(double) + d.max_ext * sizeof(double) + 16;
   d.stage_blocks = d.nblk > 0 && need <= 200 * 1024;
   const int rows_per_cta = d.nblk >= 16 ? std::max(1, d.max_core) : 64;
   const bool one_chunk = d.nblk == 0 || d.max_core <= rows_per_cta;
   const int nitems = d.nblk + d.ntiles64;
-  for (int k = 0; k < 2; ++k) d.smooth_ok[k] = false;
-  for (int k = 0; k < 2 && d.tma && one_chunk && nitems > 0; ++k) {
+  for (int k = 0; k < 3; ++k) d.smooth_ok[k] = false;
+  constexpr int R = dev::BATCH_SHARE;
+  for (int k = 0; k < (h->B >= R ? 3 : 2) && d.tma && one_chunk && nitems > 0; ++k) {
     const size_t es = k == 0 ? sizeof(double) : sizeof(float);
     const size_t tile = k == 0 ? dev::TileStage<double>::bytes(true) : dev::TileStage<float>::bytes(true);
     if (k == 0 && d.max_core > 128) continue;
@@ -1092,34 +1096,29 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
     const size_t stage = (std::max(tile, blk) + 127) & ~(size_t)127;
     // two stages, then per extended row of a block: its residual and old value (of each
     // right-hand side that shares the item) and its cell
-    const int share = k == 1 && h->B >= dev::BATCH_SHARE ? dev::BATCH_SHARE : 1;
+    const int share = k == 2 ? R : 1;
     const size_t smem = 2 * stage + (2 * share + 1) * (((size_t)std::max(1, d.max_ext) * es + 15) & ~(size_t)15);
     if (smem > 200 * 1024) continue;
     int occ = 0;
-    if (k == 0) {
-      auto fn = h->cross ? dev::k_smooth<double, true, true> : dev::k_smooth<double, false, true>;
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
-      auto gn = h->cross ? dev::k_smooth<double, true, false> : dev::k_smooth<double, false, false>;
-      cudaFuncSetAttribute(gn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      auto lp = h->cross ? dev::k_smooth<double, true, true, 1, true> : dev::k_smooth<double, false, true, 1, true>;
-      auto ln = h->cross ? dev::k_smooth<double, true, false, 1, true> : dev::k_smooth<double, false, false, 1, true>;
-      for (auto g : {lp, ln}) cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024 + LOCAL_SMEM);
+    const auto take = [&](auto pro, auto plain, size_t more) {   // PRO takes the most registers
+      cudaFuncSetAttribute(pro, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024 + more));
+      cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024 + more));
+      if (!more) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pro, 256, smem);
+    };
+    if (k == 0 && h->cross) {
+      take(dev::k_smooth<double, true, true>, dev::k_smooth<double, true, false>, 0);
+      take(dev::k_smooth<double, true, true, 1, true>, dev::k_smooth<double, true, false, 1, true>, LOCAL_SMEM);
+    } else if (k == 0) {
+      take(dev::k_smooth<double, false, true>, dev::k_smooth<double, false, false>, 0);
+      take(dev::k_smooth<double, false, true, 1, true>, dev::k_smooth<double, false, false, 1, true>, LOCAL_SMEM);
+    } else if (k == 1 && h->cross) {
+      take(dev::k_smooth<float, true, true>, dev::k_smooth<float, true, false>, 0);
+    } else if (k == 1) {
+      take(dev::k_smooth<float, false, true>, dev::k_smooth<float, false, false>, 0);
+    } else if (h->cross) {
+      take(dev::k_smooth<float, true, true, R>, dev::k_smooth<float, true, false, R>, 0);
     } else {
-      auto fn = h->cross ? dev::k_smooth<float, true, true> : dev::k_smooth<float, false, true>;
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
-      for (auto g : {h->cross ? dev::k_smooth<float, true, false> : dev::k_smooth<float, false, false>})
-        cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (share > 1) {
-        constexpr int R = dev::BATCH_SHARE;
-        auto gp = h->cross ? dev::k_smooth<float, true, true, R> : dev::k_smooth<float, false, true, R>;
-        auto gn = h->cross ? dev::k_smooth<float, true, false, R> : dev::k_smooth<float, false, false, R>;
-        for (auto g : {gp, gn}) cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        int o = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, gp, 256, smem);
-        occ = std::min(occ, o);
-      }
+      take(dev::k_smooth<float, false, true, R>, dev::k_smooth<float, false, false, R>, 0);
     }
     if (occ < 1 || nsm < 1) continue;
     d.smooth_ok[k] = true;
