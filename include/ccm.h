@@ -402,7 +402,9 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap);
  * level's SMO-2 blocks and its 64 x 32 tiles with a regular cell (Sec. 4.1), and the residual
  * + restriction is one launch over the fine tiles that restriction visits (Alg. 2).  Each CTA
  * takes items c, c + G, c + 2 G, ... through a two-stage copy ring, G = the CTAs given to one
- * right-hand side: min(items, resident CTAs of the GPU / nrhs, launch cap).
+ * right-hand side: min(items, resident CTAs of the GPU / nrhs, launch cap).  FP32 sweeps of four
+ * or more right-hand sides advance them four at a time: the four's CTAs share their items, and an
+ * SMO-2 block is one item for all four.
  * ccm_set_launch_cap: at most max_ctas CTAs per right-hand side in both kernels on every
  *   level (0: no cap, the default), so that small grids also run every CTA through many ring
  *   items.  Results do not depend on it.  Synchronises the device and drops the captured
@@ -413,8 +415,8 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap);
  *   the level does not use that persistent kernel (small levels, the bottom level, the
  *   sequential smoother).  Host-only, no device work.  Errors: CCM_EINVAL. */
 typedef struct {
-  int sweep_items;     /* work items of one sweep launch (SMO-2 blocks + tiles) */
-  int sweep_blocks;    /* of which SMO-2 block items */
+  int sweep_items;     /* work items of one sweep per right-hand side (SMO-2 blocks + tiles) */
+  int sweep_blocks;    /* of which SMO-2 block items (a quarter, rounded up, where four share them) */
   int sweep_ctas;      /* CTAs per right-hand side */
   int restrict_items;  /* tiles of one residual + restriction launch */
   int restrict_ctas;   /* CTAs per right-hand side */

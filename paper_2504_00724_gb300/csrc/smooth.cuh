@@ -45,6 +45,7 @@ struct SmoothArgs {
   int nbi;             // block items (= a.nblk)
   int nitems;          // nbi + a.ntiles: items of one right-hand side
   int nb;              // right-hand sides of the launch (grid y: groups of R of them)
+  int ctas;            // CTAs per right-hand side
   uint32_t stage;      // bytes per stage (multiple of 128)
   int max_ext;         // most extended rows of a block (the per-row scratch after the stages)
 };
@@ -547,10 +548,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
     }
     if (threadIdx.x == 0) prefetch_l1(a.blk_off + b);
   }
-  const int G = gridDim.x;
+  // (the last group may be a small one: fewer items, and CTAs only of its right-hand sides)
   const int z0 = blockIdx.y * R, nr = R == 1 ? 1 : min(R, A.nb - z0);
   const int nitems = R == 1 ? A.nitems : A.nbi + nr * a.ntiles;
-  if (R > 1 && (int)blockIdx.x >= nitems) return;           // (the last group may be a small one)
+  const int G = R == 1 ? (int)gridDim.x : min((int)gridDim.x, nr * A.ctas);
+  if (R > 1 && (int)blockIdx.x >= min(G, nitems)) return;
   const int K = (nitems - (int)blockIdx.x + G - 1) / G;     // items of this CTA (>= 1)
   // its block items come first and take BLOCK_PARTS steps of the ring each: NB block steps in
   // all, K steps with the tiles'

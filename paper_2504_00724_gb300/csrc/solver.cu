@@ -406,10 +406,23 @@ template <typename T> const CUtensorMap& TmR(const DevLevel& L);
 template <> const CUtensorMap& TmR<double>(const DevLevel& L) { return L.tmr64; }
 template <> const CUtensorMap& TmR<float>(const DevLevel& L) { return L.tmr32; }
 
+// The shape of a level's persistent sweep for nb right-hand sides: `share` of them to a grid row
+// (the last row may have fewer), with `ctas` CTAs each
+struct SweepShape {
+  int k;          // of the level's launch shapes
+  int share, ctas;
+};
+SweepShape sweep_shape(const ccm_handle* H, const DevLevel& L, bool fp64, int nb) {
+  const int k = fp64 ? 0 : nb >= dev::BATCH_SHARE && L.smooth_ok[2] ? 2 : 1;
+  return {k, k == 2 ? dev::BATCH_SHARE : 1, persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], nb, H->launch_cap)};
+}
+
 // the persistent sweep (k_smooth): SMO-2 block items and TMA tile items in one launch
 template <typename T>
 void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
-  const int k = sizeof(T) == 8 ? 0 : H->nb >= dev::BATCH_SHARE && L.smooth_ok[2] ? 2 : 1;
+  // with a batch, fewer CTAs per right-hand side so that the whole launch stays resident
+  const SweepShape shape = sweep_shape(H, L, sizeof(T) == 8, H->nb);
+  const int k = shape.k, ctas = shape.ctas;
   dev::SmoothArgs<T> A{};
   dev::SweepArgs<T>& a = A.a;
   a.tiles = L.tiles64;
@@ -439,6 +452,7 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   A.nbi = L.nblk;
   A.nitems = L.nblk + L.ntiles64;
   A.nb = H->nb;
+  A.ctas = ctas;
   A.stage = L.smooth_stage[k];
   A.max_ext = std::max(1, L.max_ext);
   const bool l0f = &L == &H->L[0] && sizeof(T) == 4;
@@ -453,14 +467,12 @@ void sweep_persistent(ccm_handle* H, DevLevel& L, cudaStream_t s, DevLevel* C) {
   const CUtensorMap& tr = TmR<T>(L);
   a.bs = L.npad;
   a.bsc = C ? C->npad : 0;
-  // with a batch, fewer CTAs per right-hand side so that the whole launch stays resident
-  const int ctas = persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], H->nb, H->launch_cap);
   const size_t smem = L.smooth_smem[k];
   const CUtensorMap& tu = C ? TmUc<T>(L, *C) : tm;
   auto go = [&](auto kernel, dim3 grid) { KL(launch_k(kernel, grid, 256, smem, s, tm, tr, L.tmcls, tu, A)); };
   if constexpr (sizeof(T) == 4) {
     constexpr int R = dev::BATCH_SHARE;
-    if (k == 2) {           // groups of R right-hand sides, with the CTAs of R
+    if (shape.share == R) {       // groups of R right-hand sides, with the CTAs of R
       const dim3 grid(std::min(ctas * R, A.nbi + R * L.ntiles64), ceil_div(H->nb, R));
       if (C && H->cross) go(dev::k_smooth<T, true, true, R>, grid);
       else if (C) go(dev::k_smooth<T, false, true, R>, grid);
@@ -2211,9 +2223,10 @@ int ccm_level_launch(const ccm_handle* h, int level, int precision, int nrhs, cc
   const bool bj = h->par.smoother == 1 && h->par.ras_passes <= 1 && h->persistent;
   *out = ccm_launch_info{};
   if (!last && bj && L.smooth_ok[k]) {
-    out->sweep_items = L.nblk + L.ntiles64;
-    out->sweep_blocks = L.nblk;
-    out->sweep_ctas = persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], nrhs, h->launch_cap);
+    const SweepShape shape = sweep_shape(h, L, k == 0, nrhs);
+    out->sweep_blocks = ceil_div(L.nblk, shape.share);
+    out->sweep_items = out->sweep_blocks + L.ntiles64;
+    out->sweep_ctas = shape.ctas;
   }
   const HostLevel& hl = h->H.levels[level];
   for (int b = 0; b < L.nblk; ++b)
