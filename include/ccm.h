@@ -352,7 +352,10 @@ int ccm_solve_T_zero(ccm_handle* h, const double* rhs, double* lambda, int nrhs,
  *      composition).  Level arrays use the user layout of that level: [ny_m][nx_m] FP64
  *      device arrays with nx_m = nx >> m, values in physical units of level m.  In FP64 a cell's
  *      error is relative to its own terms.  (Inside the solves, ccm_vcycle and ccm_fmg the FP64
- *      stencil's rounding is relative to the largest value of a 68 x 36 tile, 2^-60 of it.) */
+ *      stencil's rounding is relative to the largest value of a 68 x 36 tile, 2^-60 of it.)  The
+ *      first call in a precision that is not the handle's allocates that precision's restriction
+ *      weights (8 B, FP32 4 B a cell; not during a stream capture, which then records an older
+ *      kernel). */
 
 /* out = L^(m) u on level m (no boundary term). */
 int ccm_level_apply(ccm_handle* h, int level, const double* u, double* out, void* stream);

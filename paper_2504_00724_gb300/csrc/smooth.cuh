@@ -642,18 +642,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3) k_smooth(const __
 namespace ccm {
 namespace dev {
 
-// ---- residual + restriction of a level (Alg. 2: the coarse right-hand side and a zero coarse
-// iterate) as one persistent launch over the fine 64 x 32 tiles that restriction visits.
-// A tile item's halo tile of u, its boxes of r and (FP32) of the restriction weights (68 x 32 over the
-// tile's rows) and its class bytes (80 x 36) arrive by TMA in one of two stages while the
-// previous item computes.  In FP64 each thread loads the weights of its coarse cells' children
-// into registers before the wait instead: without their box two CTAs per SM are resident, not
-// one.  The fitted rows of the tile's irregular cells (listed per tile:
-// row and position) are gathered from global memory before the wait, and so are the class
-// bytes of the coarse cells the thread restricts to; regular cells take the stencil from the
-// staged tile; then the 32 x 16 coarse cells get the volume-weighted 2 x 2 sums.
-// the weights 4 |C_k| / sum |C| of the volume-weighted sums (Sec. 4.1) over the children of every
-// coarse cell, once at set-up: two FP64 divisions a thread cost a tile of k_restrict_p 2.6 us
+// The weights 4 |C_k| / sum |C| of the volume-weighted sums (Sec. 4.1) over the children of every coarse
+// cell, once for each precision used (w64 or w32 may be null): two FP64 divisions a thread cost a tile of
+// k_restrict_p 2.6 us.
 __global__ void k_restrict_weights(int nxc, int nyc, int pitchf, const double* __restrict__ vol, double* __restrict__ w64,
                                    float* __restrict__ w32) {
   const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y;
@@ -665,11 +656,21 @@ __global__ void k_restrict_weights(int nxc, int nyc, int pitchf, const double* _
   for (int k = 0; k < 4; ++k) {
     const double w = sv > 0 ? 4 * v[k] / sv : 0.0;
     const long q = p + (k >> 1) * pitchf + (k & 1);
-    w64[q] = w;
-    w32[q] = (float)w;
+    if (w64) w64[q] = w;
+    if (w32) w32[q] = (float)w;
   }
 }
 
+// ---- residual + restriction of a level (Alg. 2: the coarse right-hand side and a zero coarse
+// iterate) as one persistent launch over the fine 64 x 32 tiles that restriction visits.
+// A tile item's halo tile of u, its boxes of r and (FP32) of the restriction weights (68 x 32 over the
+// tile's rows) and its class bytes (80 x 36) arrive by TMA in one of two stages while the
+// previous item computes.  In FP64 each thread loads the weights of its coarse cells' children
+// into registers before the wait instead: without their box two CTAs per SM are resident, not
+// one.  The fitted rows of the tile's irregular cells (listed per tile:
+// row and position) are gathered from global memory before the wait, and so are the class
+// bytes of the coarse cells the thread restricts to; regular cells take the stencil from the
+// staged tile; then the 32 x 16 coarse cells get the volume-weighted 2 x 2 sums.
 template <typename T>
 struct RestrictArgs {
   const int32_t* tiles;

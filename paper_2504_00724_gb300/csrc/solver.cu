@@ -56,10 +56,11 @@ struct DevLevel {
   size_t smooth_smem[3] = {0, 0, 0};
   int smooth_grid[3] = {0, 0, 0};
   int smooth_cap[3] = {0, 0, 0};   // resident CTAs of the persistent sweep over the whole GPU
-  double* rw64 = nullptr;       // restriction weights of the cells (levels with k_restrict_p)
-  float* rw32 = nullptr;
+  double* rw64 = nullptr;       // restriction weights of the cells (levels with k_restrict_p), of the
+  float* rw32 = nullptr;        // precisions that have been used (restriction_weights)
   CUtensorMap tmv64, tmv32;     // 68 x 32 boxes over them
-  bool restrict_ok[2] = {false, false};  // persistent restriction (k_restrict_p), [0] FP64, [1] FP32
+  // persistent restriction (k_restrict_p), [0] FP64, [1] FP32: its launch fits; its weights are there
+  bool restrict_fit[2] = {false, false}, restrict_ok[2] = {false, false};
   uint32_t restrict_stage[2] = {0, 0};
   int restrict_grid[2] = {0, 0};
   int restrict_cap[2] = {0, 0};
@@ -1142,6 +1143,42 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   cudaGetLastError();
 }
 
+// The restriction weights of one precision on the levels whose persistent restriction uses them: that
+// of the handle's cycles at set-up, the other with the first call of a level or cycle in it (8 or 4 B
+// a padded cell; not during a stream capture).  Levels without them take the older kernel.
+void restriction_weights(ccm_handle* h, bool fp64, cudaStream_t s = nullptr) {
+  const int k = fp64 ? 0 : 1;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  bool any = false;
+  for (size_t m = 0; m + 1 < h->L.size(); ++m) {
+    DevLevel& d = h->L[m];
+    if (!d.restrict_fit[k] || d.restrict_ok[k]) continue;
+    if (!any && (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)) {
+      cudaGetLastError();
+      return;
+    }
+    Arena& A = h->arena;
+    if (fp64) d.rw64 = A.try_alloc<double>(d.npad);
+    else d.rw32 = A.try_alloc<float>(d.npad);
+    if (!(fp64 ? (void*)d.rw64 : (void*)d.rw32)) continue;
+    const bool map = fp64 ? make_tmap(&d.tmv64, d.rw64, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY)
+                          : make_tmap(&d.tmv32, d.rw32, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::HX, dev::JY);
+    if (!map) {
+      A.free(fp64 ? (void*)d.rw64 : (void*)d.rw32);
+      d.restrict_fit[k] = false;
+      continue;
+    }
+    const DevLevel& c = h->L[m + 1];
+    KL(dev::k_restrict_weights<<<dim3(ceil_div(c.nx, 128), c.ny), 128>>>(c.nx, c.ny, d.pitch, d.vol64, fp64 ? d.rw64 : nullptr,
+                                                                         fp64 ? nullptr : d.rw32));
+    d.restrict_ok[k] = true;
+    any = true;
+  }
+  if (!any) return;
+  cudaStreamSynchronize(nullptr);
+  h->info.device_bytes = h->arena.bytes;
+}
+
 // set-up scratch; ccm_fail_scratch makes the next requests report that there is no memory
 std::atomic<int> g_fail_scratch{0};
 cudaError_t scratch_malloc(void** p, size_t bytes) {
@@ -1474,17 +1511,7 @@ int upload_hierarchy(ccm_handle* h) {
                     make_tmap(&d.tmuc32[b], c.u32[b], c.pitch, c.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::UCX, dev::UCY,
                               h->B);
       // the persistent restriction: two stages of u, r, class bytes and weights per tile
-      bool maps = d.ntiles64r > 0;
-      if (maps) {
-        d.rw64 = A.alloc<double>(d.npad);
-        d.rw32 = A.alloc<float>(d.npad);
-        if (A.err == cudaSuccess)
-          KL(dev::k_restrict_weights<<<dim3(ceil_div(hc.nx, 128), hc.ny), 128>>>(hc.nx, hc.ny, d.pitch, d.vol64, d.rw64, d.rw32));
-        maps = A.err == cudaSuccess &&
-               make_tmap(&d.tmv64, d.rw64, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 8, dev::HX, dev::JY) &&
-               make_tmap(&d.tmv32, d.rw32, d.pitch, d.rows, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, dev::HX, dev::JY);
-      }
-      for (int k = 0; k < 2 && maps; ++k) {
+      for (int k = 0; k < 2 && d.ntiles64r > 0; ++k) {
         const uint32_t stage = k == 0 ? dev::RestrictStage<double>::bytes : dev::RestrictStage<float>::bytes;
         const size_t smem = 2 * (size_t)stage;
         int occ = 0;
@@ -1500,7 +1527,7 @@ int upload_hierarchy(ccm_handle* h) {
           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem);
         }
         if (occ < 1 || nsm < 1) continue;
-        d.restrict_ok[k] = true;
+        d.restrict_fit[k] = true;
         d.restrict_stage[k] = stage;
         // FP64: one CTA per SM until there are two tiles for each, so that every CTA's first copy
         // has its SM's bandwidth to itself
@@ -1511,6 +1538,7 @@ int upload_hierarchy(ccm_handle* h) {
       cudaGetLastError();
     }
   }
+  restriction_weights(h, h->par.precision == CCM_FP64);
   // the cluster launch takes over from the first level with at most coarse_n cells a side
   // (block-Jacobi smoother only: its sweeps read nothing but the old iterate)
   if (h->par.coarse_n > 0 && h->par.smoother == 1 && h->par.ras_passes <= 1) {
@@ -2231,7 +2259,7 @@ int ccm_level_launch(const ccm_handle* h, int level, int precision, int nrhs, cc
   const HostLevel& hl = h->H.levels[level];
   for (int b = 0; b < L.nblk; ++b)
     out->block_inv_entries += (int64_t)(hl.blk[4 * b + 1] - hl.blk[4 * b]) * (hl.blk[4 * b + 3] - hl.blk[4 * b + 2]);
-  if (!last && bj && L.tma && L.ntiles64r && L.restrict_ok[k]) {
+  if (!last && bj && L.tma && L.ntiles64r && L.restrict_fit[k]) {
     out->restrict_items = L.ntiles64r;
     out->restrict_ctas = persistent_ctas(L.restrict_grid[k], L.restrict_cap[k], nrhs, h->launch_cap);
   }
@@ -2918,6 +2946,7 @@ int ccm_level_restrict(ccm_handle* h, int level, const double* u, const double* 
   if (check_level(h, level) || level == (int)h->L.size() - 1 || !u || !r || !rc) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   const LocalScope local(h);
+  restriction_weights(h, true, s);
   DevLevel& F = h->L[level];
   DevLevel& C = h->L[level + 1];
   load_level<double>(h, F, u, r, s);
@@ -2981,6 +3010,7 @@ int ccm_bottom_solve(ccm_handle* h, const double* r, double* u, void* stream) {
 int ccm_vcycle(ccm_handle* h, double* u, const double* r, int precision, void* stream) {
   if (!h || !u || !r) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  restriction_weights(h, precision == CCM_FP64, s);
   DevLevel& L = h->L[0];
   dim3 pg(ceil_div(L.nx, 128), L.ny);
   if (precision == CCM_FP64) {
@@ -2999,6 +3029,7 @@ int ccm_vcycle(ccm_handle* h, double* u, const double* r, int precision, void* s
 int ccm_fmg(ccm_handle* h, double* u, const double* r, int precision, void* stream) {
   if (!h || !u || !r) return CCM_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
+  restriction_weights(h, precision == CCM_FP64, s);
   DevLevel& L = h->L[0];
   dim3 pg(ceil_div(L.nx, 128), L.ny);
   if (precision == CCM_FP64) {
