@@ -405,7 +405,7 @@ int ccm_set_smo2_blocks(ccm_handle* h, int block, int overlap);
  * level's SMO-2 blocks and its 64 x 32 tiles with a regular cell (Sec. 4.1), and the residual
  * + restriction is one launch over the fine tiles that restriction visits (Alg. 2).  Each CTA
  * takes items c, c + G, c + 2 G, ... through a two-stage copy ring, G = the CTAs given to one
- * right-hand side: min(items, resident CTAs of the GPU / nrhs, launch cap).  FP32 sweeps of four
+ * right-hand side: min(items, resident CTAs of the GPU / nrhs, launch cap).  FP32 sweeps of 32
  * or more right-hand sides advance them four at a time: the four's CTAs share their items, and an
  * SMO-2 block is one item for all four.
  * ccm_set_launch_cap: at most max_ctas CTAs per right-hand side in both kernels on every

@@ -34,9 +34,13 @@ namespace dev {
 // that one CTA per SM is resident instead of two
 template <typename T>
 constexpr int BLOCK_PARTS = sizeof(T) == 8 ? 2 : 1;
-// right-hand sides of a batch that share block items (FP32; 256 threads update 64 core rows of 4)
-// disk 512^2, 64 right-hand sides: 22.6 ms a solve without, 20.1 with; below four the launch is not
-// bound by L2 and keeps its CTAs apart
+// Right-hand sides of a batch that share block items (FP32; 256 threads update 64 core rows of 4), in
+// batches of at least BATCH_SHARE_FROM.  A shared item takes its four residual gathers one after the
+// other, which is the launch's critical path until every CTA has many items.  Solves, sharing / apart, ms
+// (star 256^2, disk 512^2, star 1024^2): 4 right-hand sides 2.30 / 1.29, 3.43 / 2.33, 5.42 / 3.49; 24: 3.44 / 2.62,
+// 7.47 / 6.82, 13.1 / 12.6; 32: 3.56 / 4.23, 10.1 / 11.8, 21.1 / 24.3; 64: 7.20 / 7.67, 20.5 / 22.6.  Only the 128^2
+// grids still lose at 32 (star 1.77 / 1.76, disk 2.18 / 2.02), and only the larger ones gain at 16 (up to 9 %).
+constexpr int BATCH_SHARE_FROM = 32;
 constexpr int BATCH_SHARE = 4;
 
 template <typename T>

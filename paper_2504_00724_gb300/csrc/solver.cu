@@ -414,7 +414,7 @@ struct SweepShape {
   int share, ctas;
 };
 SweepShape sweep_shape(const ccm_handle* H, const DevLevel& L, bool fp64, int nb) {
-  const int k = fp64 ? 0 : nb >= dev::BATCH_SHARE && L.smooth_ok[2] ? 2 : 1;
+  const int k = fp64 ? 0 : nb >= dev::BATCH_SHARE_FROM && L.smooth_ok[2] ? 2 : 1;
   return {k, k == 2 ? dev::BATCH_SHARE : 1, persistent_ctas(L.smooth_grid[k], L.smooth_cap[k], nb, H->launch_cap)};
 }
 
@@ -1100,7 +1100,7 @@ void configure_sweep(ccm_handle* h, DevLevel& d, int nsm) {
   const int nitems = d.nblk + d.ntiles64;
   for (int k = 0; k < 3; ++k) d.smooth_ok[k] = false;
   constexpr int R = dev::BATCH_SHARE;
-  for (int k = 0; k < (h->B >= R ? 3 : 2) && d.tma && one_chunk && nitems > 0; ++k) {
+  for (int k = 0; k < (h->B >= dev::BATCH_SHARE_FROM ? 3 : 2) && d.tma && one_chunk && nitems > 0; ++k) {
     const size_t es = k == 0 ? sizeof(double) : sizeof(float);
     const size_t tile = k == 0 ? dev::TileStage<double>::bytes(true) : dev::TileStage<float>::bytes(true);
     if (k == 0 && d.max_core > 128) continue;
