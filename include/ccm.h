@@ -385,7 +385,7 @@ int ccm_vcycle(ccm_handle* h, double* u, const double* r, int precision, void* s
  * without repeating the host setup: omega (0, 1.5], nu1, nu2 (0 - 16, nu1 + nu2 >= 1),
  * inner_cycles (1 - 16), cycle (0 V, 1 FMG first).  Synchronises the device and drops the
  * captured iteration graphs (the next solve recaptures them).  The matrix that stands for the
- * small levels' part of the V-cycle is recomputed on the device (a few ms).  Used by the autotuner.  The
+ * small levels' part of the V-cycle is recomputed on the device when omega, nu1 or nu2 change (1 to 3 ms).  Used by the autotuner.  The
  * paper fixes omega = 0.5, nu1 = nu2 = 3 (Sec. 5); these are free parameters of Alg. 2.
  * Errors: CCM_EINVAL, CCM_ECUDA. */
 int ccm_set_cycle_params(ccm_handle* h, double omega, int nu1, int nu2, int inner_cycles, int cycle);

@@ -2276,11 +2276,14 @@ int ccm_set_cycle_params(ccm_handle* h, double omega, int nu1, int nu2, int inne
   for (ccm_handle* t : {h, h->adj}) {
     if (!t) continue;
     const double w22 = t->S64.omega_d != 0 ? t->par.omega / t->S64.omega_d : 0.0;   // the stencil's diagonal
+    // the matrix of the small levels is that of one V-cycle: the other parameters do not matter to it
+    const bool same = omega == t->par.omega && nu1 == t->par.nu1 && nu2 == t->par.nu2 && t->dense.m >= 0;
     t->par.omega = omega;
     t->par.nu1 = nu1;
     t->par.nu2 = nu2;
     t->par.inner_cycles = inner_cycles;
     t->par.cycle = cycle;
+    if (same) continue;
     if (w22 != 0) {
       t->S64.omega_d = omega / w22;
       t->S32.omega_d = (float)(omega / w22);

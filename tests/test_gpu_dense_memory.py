@@ -79,3 +79,18 @@ def test_setup_without_memory():
     finally:
         s.close()
         other.close()
+
+
+def test_parameters_that_the_matrix_does_not_depend_on_keep_it():
+    s, other, (u, r) = pair()
+    try:
+        want = s.vcycle(u, r, P.CCM_FP64)
+        n = P.lib().ccm_launch_count()
+        s.set_cycle_params(inner_cycles=2, cycle=1)
+        s.set_cycle_params(inner_cycles=1, cycle=0)
+        assert P.lib().ccm_launch_count() == n         # nothing ran on the device
+        assert torch.equal(s.vcycle(u, r, P.CCM_FP64), want)
+        assert s.solve(r)[1].rel_residual <= 1e-11
+    finally:
+        s.close()
+        other.close()
