@@ -308,8 +308,8 @@ int ccm_solve_host(ccm_handle* h, const double* f, const double* g, double* u, i
  * iteration of every member whose relative residual is still above its rtol (and below
  * its max_iter), each member's work on its own branch of the graph, then a one-thread-block
  * kernel that reads the members' FP64 residual norms and retires the converged ones.  The
- * arithmetic of a member is that of ccm_solve with one right-hand side; only the
- * convergence test moves from the host to the device.
+ * arithmetic and the decisions of a member are those of ccm_solve with one right-hand side,
+ * whose loop runs on the device too.
  * ccm_group_create captures every member's iteration (it synchronises `stream` and uses
  * each member's private capture stream; call it outside any stream capture, after
  * ccm_set_cycle_params).  The group keeps that cycle: a later ccm_set_cycle_params or
@@ -352,7 +352,7 @@ int ccm_solve_T_zero(ccm_handle* h, const double* rhs, double* lambda, int nrhs,
  *      composition).  Level arrays use the user layout of that level: [ny_m][nx_m] FP64
  *      device arrays with nx_m = nx >> m, values in physical units of level m.  In FP64 a cell's
  *      error is relative to its own terms.  (Inside the solves, ccm_vcycle and ccm_fmg the FP64
- *      stencil's rounding is relative to the largest value of a 68 x 36 tile, 2^-60 of it.)  The
+ *      stencil's rounding is relative to the largest value of a 68 x 36 tile, 2^-58 of it.)  The
  *      first call in a precision that is not the handle's allocates that precision's restriction
  *      weights (8 B, FP32 4 B a cell; not during a stream capture, which then records an older
  *      kernel). */

@@ -17,18 +17,20 @@
 //
 // These errors are relative to the tile's largest value, those of an FP64 sum to the cell's own
 // terms.  A pass whose results are the operator's values themselves (apply.cuh, a single sweep or
-// restriction) keeps the doubles beside the integers and looks at every cell (LOCAL): where the sum of
+// restriction) keeps the doubles beside the integers and looks at every cell (FINE): where the sum of
 // its |w u| is so small, against the tile's largest value, that their bound exceeds 3 2^-53 of that
 // sum (near a spike, in the tail of a narrow kernel, at some zeros of a smooth field: in one warp of 14
 // at most), the FP64 sum replaces the result (q_few).  Errors relative to a cell's sum of |w u| over the
 // tiles of random plane waves on 64^2 .. 4096^2 grids against 64-bit mantissas, rms / worst: FP64 sum
-// 4.5e-17 / 2.0e-16, this 0.1 - 0.6e-17 / 1.7e-16.  (q on 57 bits, Lap and Grad whole and no look at the
-// cell: 0.3 - 1.4e-17 / 1.0e-15, and no correct digit left in cells 2^-58 below the tile's largest.)
+// 4.5e-17 / 2.0e-16, this 0.1 - 0.6e-17 / 1.7e-16.
 //
-// Inside a solve no cell is looked at: everywhere in the tile the error is below the FP64 rounding
-// at its largest value, which the max-norm of the residual and the elliptic coupling of the cells see
+// Inside a solve no cell is looked at, and the form is plainer: q on 57 bits, 16 Lap and 8 Grad as whole
+// numbers, A = a / 12, C = c / 12, B = 8 b / 144 as 62-bit integers (its shifts fold into adds, some six
+// operations a cell fewer: star 1024^2 FP64 solve 4.06 ms, 4.14 with the form above; of the plane waves'
+// cells 0.3 - 1.4e-17 / 1.0e-15).  Everywhere in the tile its error is below the FP64 rounding at the
+// tile's largest value, which the max-norm of the residual and the elliptic coupling of the cells see
 // just as well, and corrections that fall by decades within a tile are common on coarse levels (with
-// the look at every cell a star 1024^2 FP64 solve takes 12.7 ms, without 4.0).
+// the look at every cell that solve takes 12.7 ms).
 //
 // Tiles that hold an infinity or a NaN, or whose largest value is outside 2^-800 .. 2^700, take the
 // FP64 sum, and so do operators with a coefficient outside 2^-100 .. 2^100.
@@ -47,9 +49,14 @@
 namespace ccm {
 namespace dev {
 
-struct QStencil {
-  long long A = 0, C = 0, B = 0;   // 16 a / 12, 16 c / 12, 64 b / 144 times 2^k
-  int cexp = 0;                    // the sum of the upper products times 2^(E - 1022 + cexp) is h^2 L u
+// coefficients times 2^k; the sum of the upper products times 2^(E - 1022 + cexp) is h^2 L u
+struct QCoef {
+  long long A = 0, C = 0, B = 0;
+  int cexp = 0;
+};
+
+struct QStencil : QCoef {          // 16 a / 12, 16 c / 12, 64 b / 144 (FINE)
+  QCoef plain;                     // a / 12, c / 12, 8 b / 144
   int ok = 0;                      // the coefficients are in range
   // least sum of |w u| over 2^s for which the integer form is as accurate as the FP64 sum, the
   // weights of the axis taps (centre, x +- 1, x +- 2, y +- 1, y +- 2), and the upper word of the
@@ -58,17 +65,15 @@ struct QStencil {
   unsigned near = 0;
 };
 
-inline QStencil q_stencil(double a, double b, double c) {
-  QStencil S;
-  const long double A = 16.0L * a / 12.0L, C = 16.0L * c / 12.0L, B = 64.0L * b / 144.0L;
+// v_i 2^(bits - e) as integers, |v_i| < 2^e; false where e is out of range
+inline bool q_coef(long double A, long double C, long double B, int bits, int qbits, QCoef& S, int& e) {
   long double m = std::fabs(A);
   if (std::fabs(C) > m) m = std::fabs(C);
   if (std::fabs(B) > m) m = std::fabs(B);
-  if (!(m > 0) || !std::isfinite((double)m)) return S;
-  int e = 0;
+  if (!(m > 0) || !std::isfinite((double)m)) return false;
   std::frexp((double)m, &e);                    // m < 2^e (a rounding up to 2^e only widens it)
-  if (e < -100 || e > 100) return S;
-  const int k = 63 - e;
+  if (e < -100 || e > 100) return false;
+  const int k = bits - e;
   const auto fix = [&](long double v) {
     const long double t = std::ldexp(v, k);
     return t >= 9223372036854775807.0L ? 9223372036854775807LL : t <= -9223372036854775807.0L ? -9223372036854775807LL
@@ -77,7 +82,17 @@ inline QStencil q_stencil(double a, double b, double c) {
   S.A = fix(A);
   S.C = fix(C);
   S.B = fix(B);
-  S.cexp = 64 - k - 60;
+  S.cexp = 64 - k - qbits;
+  return true;
+}
+
+inline QStencil q_stencil(double a, double b, double c) {
+  QStencil S;
+  int e = 0;
+  const long double la = a, lb = b, lc = c;
+  if (!q_coef(la / 12.0L, lc / 12.0L, lb / 18.0L, 62, 57, S.plain, e) ||
+      !q_coef(16.0L * la / 12.0L, 16.0L * lc / 12.0L, 64.0L * lb / 144.0L, 63, 60, S, e))
+    return S;
   S.ok = 1;
   // The bound on the error in units of 2^(s - 60): the values' rounding, half a unit in every tap
   // (64 / 12 in all along x and along y, 324 / 144 of the mixed term); the sixteenths' floors, times 16 / 12,
@@ -107,10 +122,11 @@ CCM_HD int q_scale(unsigned m, const QStencil& S) {
 }
 
 // q of the double with words (hi, lo) at tile scale E (its exponent field is at most E)
+template <bool FINE = true>
 CCM_HD long long q_fixed(unsigned hi, unsigned lo, int E) {
   const unsigned mh = (hi << 11) | (lo >> 21) | 0x80000000u, ml = lo << 11;
   const unsigned long long m = ((unsigned long long)mh << 32) | ml;   // 1.f times 2^63
-  const unsigned sh = (unsigned)(E - (int)((hi >> 20) & 0x7ffu)) + 3u;
+  const unsigned sh = (unsigned)(E - (int)((hi >> 20) & 0x7ffu)) + (FINE ? 3u : 6u);
   unsigned long long q;
 #ifdef __CUDA_ARCH__
   asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(m), "r"(sh));            // 0 from 64 on (zeros: 220 and up)
@@ -122,12 +138,20 @@ CCM_HD long long q_fixed(unsigned hi, unsigned lo, int E) {
   return ((long long)q ^ s) - s;
 }
 
+// Lap, and (where it is not FINE, 16 times) as a whole number; Grad likewise, and its rounded eighth
+template <bool FINE = true>
 CCM_HD long long q_lap(long long m2, long long m1, long long c, long long p1, long long p2) {
   const long long c2 = c + c;
-  return (m1 + p1 - c2) - ((m2 + p2 - c2) >> 4);
+  return FINE ? (m1 + p1 - c2) - ((m2 + p2 - c2) >> 4) : (m1 + p1 - c2) * 16 - (m2 + p2 - c2);
 }
-CCM_HD long long q_grad(long long m2, long long m1, long long p1, long long p2) { return (p1 - m1) + ((m2 - p2) >> 3); }
-CCM_HD long long q_grad8(long long m2, long long m1, long long p1, long long p2) { return q_grad(m2, m1, p1, p2); }
+template <bool FINE = true>
+CCM_HD long long q_grad(long long m2, long long m1, long long p1, long long p2) {
+  return FINE ? (p1 - m1) + ((m2 - p2) >> 3) : (m2 - p2) + (p1 - m1) * 8;
+}
+template <bool FINE = true>
+CCM_HD long long q_grad8(long long m2, long long m1, long long p1, long long p2) {
+  return FINE ? q_grad<true>(m2, m1, p1, p2) : (q_grad<false>(m2, m1, p1, p2) + 4) >> 3;
+}
 CCM_HD long long q_hi(long long x, long long y) {
 #ifdef __CUDA_ARCH__
   return __mul64hi(x, y);
@@ -142,7 +166,7 @@ CCM_HD long long q_lap_neg(long long m2, long long m1, long long c, long long p1
   const long long c2 = c + c;
   return (c2 - m1 - p1) - ((c2 - m2 - p2) >> 4);
 }
-CCM_HD long long q_axes(long long hx, long long neg_y, const QStencil& S) { return hx - q_hi(neg_y, S.C); }
+CCM_HD long long q_axes(long long hx, long long neg_y, const QCoef& S) { return hx - q_hi(neg_y, S.C); }
 
 // |q| 2^-60 from the upper word of q, rounded down (a lone unit of it is 2^-28)
 CCM_HD float q_part(long long q) {
@@ -210,13 +234,14 @@ struct QSlots {
     }
     return m;
   }
+  template <bool FINE>
   __device__ __forceinline__ void store(long long* q, int n, int E) const {
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int idx = threadIdx.x + 256 * k;
       if (idx < n)
         *reinterpret_cast<longlong2*>(q + 2 * idx) =
-            make_longlong2(q_fixed(hi[2 * k], lo[2 * k], E), q_fixed(hi[2 * k + 1], lo[2 * k + 1], E));
+            make_longlong2(q_fixed<FINE>(hi[2 * k], lo[2 * k], E), q_fixed<FINE>(hi[2 * k + 1], lo[2 * k + 1], E));
     }
   }
 };
@@ -225,10 +250,11 @@ struct QSlots {
 // x0 even, on a staged tile q [.][ROW] of integers whose cell (0, 0) is at (2, 2): two columns
 // and four rows a thread, each staged row read as aligned pairs that serve both columns; the
 // rows' Lap_x and Grad_x are formed as a row enters and kept until their cells are complete.
-// emit(k, s0, s1).  With LOCAL the result says whether every cell's own value alone is large enough
+// emit(k, s0, s1).  With FINE the result says whether every cell's own value alone is large enough
 // for the integer form (on the upper words, which are in registers: 2 operations a cell).
-template <bool CROSS, int ROW, bool LOCAL, class Emit>
-__device__ __forceinline__ bool q_rows(const long long* __restrict__ q, int x0, int y0, const QStencil& S, Emit emit) {
+template <bool CROSS, int ROW, bool FINE, class Emit>
+__device__ __forceinline__ bool q_rows(const long long* __restrict__ q, int x0, int y0, const QStencil& Q, Emit emit) {
+  const QCoef& S = FINE ? static_cast<const QCoef&>(Q) : Q.plain;
   long long c[2][8], d[2][8], X[2][4];
   unsigned least = 0xffffffffu;
 #pragma unroll
@@ -237,32 +263,34 @@ __device__ __forceinline__ bool q_rows(const long long* __restrict__ q, int x0, 
     const longlong2 b = row[1];
     c[0][r] = b.x;
     c[1][r] = b.y;
-    if (LOCAL && r >= 2 && r < 6) {
+    if (FINE && r >= 2 && r < 6) {
       const int v0 = (int)(b.x >> 32), v1 = (int)(b.y >> 32);
       least = min(least, min((unsigned)(v0 ^ (v0 >> 31)), (unsigned)(v1 ^ (v1 >> 31))));
     }
     if (CROSS || (r >= 2 && r < 6)) {
       const longlong2 a = row[0], e = row[2];
       if (CROSS) {
-        d[0][r] = q_grad8(a.x, a.y, b.y, e.x);
-        d[1][r] = q_grad8(a.y, b.x, e.x, e.y);
+        d[0][r] = q_grad8<FINE>(a.x, a.y, b.y, e.x);
+        d[1][r] = q_grad8<FINE>(a.y, b.x, e.x, e.y);
       }
       if (r >= 2 && r < 6) {
-        X[0][r - 2] = q_hi(q_lap(a.x, a.y, b.x, b.y, e.x), S.A);
-        X[1][r - 2] = q_hi(q_lap(a.y, b.x, b.y, e.x, e.y), S.A);
+        X[0][r - 2] = q_hi(q_lap<FINE>(a.x, a.y, b.x, b.y, e.x), S.A);
+        X[1][r - 2] = q_hi(q_lap<FINE>(a.y, b.x, b.y, e.x, e.y), S.A);
       }
     }
     if (r >= 4) {
       long long s[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        s[j] = q_axes(X[j][r - 4], q_lap_neg(c[j][r - 4], c[j][r - 3], c[j][r - 2], c[j][r - 1], c[j][r]), S);
-        if (CROSS) s[j] += q_hi(q_grad(d[j][r - 4], d[j][r - 3], d[j][r - 1], d[j][r]), S.B);
+        const long long m2 = c[j][r - 4], m1 = c[j][r - 3], m = c[j][r - 2], p1 = c[j][r - 1], p2 = c[j][r];
+        if (FINE) s[j] = q_axes(X[j][r - 4], q_lap_neg(m2, m1, m, p1, p2), S);
+        else s[j] = X[j][r - 4] + q_hi(q_lap<false>(m2, m1, m, p1, p2), S.C);
+        if (CROSS) s[j] += q_hi(q_grad<FINE>(d[j][r - 4], d[j][r - 3], d[j][r - 1], d[j][r]), S.B);
       }
       emit(r - 4, s[0], s[1]);
     }
   }
-  return !LOCAL || least >= S.near;
+  return !FINE || least >= Q.near;
 }
 
 // Of these cells those whose sum of |w u| is too small for the integer form (bit 2 k + j: cell

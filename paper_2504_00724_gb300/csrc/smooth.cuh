@@ -318,9 +318,9 @@ __device__ __forceinline__ void tile_stencil64(double* tile, long long* q, unsig
       }
     return;
   }
-  v.store(q, NP, E);
+  v.template store<LOCAL>(q, NP, E);
   __syncthreads();
-  const int e = E - 1022 + Q.cexp;
+  const int e = E - 1022 + (LOCAL ? Q.cexp : Q.plain.cexp);
   if (on) {
     const bool ok = q_rows<CROSS, HX, LOCAL>(q, x0, y0, Q, [&](int k, long long s0, long long s1) { emit(k, q_double(s0, e), q_double(s1, e)); });
     if (LOCAL && !ok && m != 0) few();

@@ -27,7 +27,7 @@ int main(int, char** v) {
   std::mt19937_64 g(11);
   std::normal_distribution<double> N;
   std::uniform_real_distribution<double> U(0, 1);
-  double worst = 0, worst64 = 0;
+  double worst = 0, worst64 = 0, plain = 0;
   long ints = 0, all = 0;
   for (int tile = 0; tile < (kind == 4 ? 200 : 4); ++tile) {
     const int n = 64 << (tile % 7);
@@ -43,7 +43,10 @@ int main(int, char** v) {
     }
     if (kind == 1) u[17][31 + tile] = 1e18;
     if (kind == 5) u[9][5] = 1;
-    for (auto& r : u) for (double x : r) m = std::max(m, q_word(hi(x), lo(x)));
+    double top = 0, sum = 0;
+    for (auto& r : u) for (double x : r) { m = std::max(m, q_word(hi(x), lo(x))); top = std::max(top, std::fabs(x)); }
+    for (int d = 0; d < 5; ++d) for (int e = 0; e < 5; ++e)
+      sum += std::fabs(b * gra[d] * gra[e] / 144 + (d == 2 ? a * lap[e] / 12 : 0) + (e == 2 ? c * lap[d] / 12 : 0));
     const int E = q_scale(m, S);
     if (E < 0) return 2;
     for (int j = 0; j < 36; ++j) for (int i = 0; i < 68; ++i) q[j][i] = q_fixed(hi(u[j][i]), lo(u[j][i]), E);
@@ -60,6 +63,14 @@ int main(int, char** v) {
       }
       ++all;
       if (terms > 0) worst64 = std::max(worst64, (double)(fabsl(f - x) / terms));
+      // the plain form of the solves' passes: relative to the tile's largest value
+      const auto P = [&](int dj, int di) { return q_fixed<false>(hi(u[j + dj][i + di]), lo(u[j + dj][i + di]), E); };
+      long long ps = q_hi(q_lap<false>(P(0, -2), P(0, -1), P(0, 0), P(0, 1), P(0, 2)), S.plain.A) +
+                     q_hi(q_lap<false>(P(-2, 0), P(-1, 0), P(0, 0), P(1, 0), P(2, 0)), S.plain.C);
+      long long pd[5];
+      for (int k = 0; k < 5; ++k) pd[k] = q_grad8<false>(P(k - 2, -2), P(k - 2, -1), P(k - 2, 1), P(k - 2, 2));
+      if (b != 0) ps += q_hi(q_grad<false>(pd[0], pd[1], pd[3], pd[4]), S.plain.B);
+      plain = std::max(plain, (double)(fabsl(q_double(ps, E - 1022 + S.plain.cexp) - x) / (top * sum)));
       if (few && terms > 0) continue;          // (a cell whose taps are all 0 keeps its integer result, 0)
       ++ints;
       const long long own = q[j][i] >> 32;
@@ -74,7 +85,7 @@ int main(int, char** v) {
       worst = std::max(worst, (double)(fabsl(r - x) / terms));
     }
   }
-  printf("%.17g %.17g %.17g\n", worst, worst64, (double)ints / all);
+  printf("%.17g %.17g %.17g %.17g\n", worst, worst64, (double)ints / all, plain);
 }
 '''
 
@@ -94,9 +105,11 @@ def harness(tmp_path_factory):
 @pytest.mark.parametrize("kind", range(7))
 def test_every_cell_is_as_accurate_as_its_fp64_sum(harness, abc, kind):
     out = subprocess.run([harness, *map(repr, map(float, abc)), str(kind)], capture_output=True, text=True, check=True).stdout
-    worst, worst64, share = map(float, out.split())
+    worst, worst64, share, plain = map(float, out.split())
     # the bound of the integer form, and the rounding of its result
     assert worst <= (3 + 1) * 2.0 ** -53
     assert worst <= max(1.5 * worst64, 2.5e-16)     # the FP64 sum's worst cell on the same field: 1 to 2.5e-16
+    # values to 2^-58, the eighth, three floors, and the rounding of the result
+    assert plain <= 1.1 * 2.0 ** -53
     if kind in (4, 6):
         assert share >= 0.97                        # and it is the form that is used
