@@ -3,22 +3,27 @@
 
 #include <cstddef>
 
-#include "fixed.cuh"
+#ifdef __CUDACC__
+#define CCM_HDC __host__ __device__ constexpr
+#else
+#define CCM_HDC constexpr
+#endif
 
 namespace ccm {
 namespace dev {
 
-// Extended rows of the first part: half of them, rounded up to an even number (the second part's copy
-// starts on 16 bytes) and so never fewer than the second part's.
-CCM_HD int block_split(int ne) { return ne < 2 ? ne : ((ne + 1) / 2 + 1) & ~1; }
+// extended rows of the first part: about half, even (the second part's copy starts on 16 bytes)
+CCM_HDC int block_split(int ne) { return (ne / 2 + 1) & ~1; }
 
 // bytes of the bulk copy of `rows` rows of nc columns
-CCM_HD unsigned block_copy_bytes(int rows, int nc, int es) { return (unsigned)(((long)rows * nc * es + 15) & ~15L); }
+CCM_HDC unsigned block_copy_bytes(int rows, int nc, size_t es) { return (unsigned)(((long)rows * nc * es + 15) & ~15L); }
 
 // bytes that a stage needs for any block of at most max_ext extended and max_core core rows, whole
-// or (parts) any part of it: the first part is the longer one, and longest at max_ext
+// or (parts) any part of it: the second part is the longer one where ne = 4 k + 1, and the longer
+// part does not get shorter as ne grows
 inline size_t block_stage_bytes(int max_ext, int max_core, int es, bool parts) {
-  return block_copy_bytes(parts ? block_split(max_ext) : max_ext, max_core, es);
+  const int first = block_split(max_ext), second = max_ext - first;
+  return block_copy_bytes(parts ? (first > second ? first : second) : max_ext, max_core, es);
 }
 
 }  // namespace dev

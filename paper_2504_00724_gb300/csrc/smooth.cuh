@@ -116,7 +116,7 @@ __device__ __forceinline__ void smooth_issue(const SmoothArgs<T>& A, const CUten
     const int e1 = BLOCK_PARTS<T> == 2 && !half ? block_split(ne) : ne;
     const uint32_t abytes = block_copy_bytes(e1 - e0, nc, sizeof(T));
     mbar_expect_tx(bar, abytes);
-    if (abytes) bulk_load(st, a.inv + a.blk_off[b] + (long)e0 * nc, abytes, bar);   // (a block of 1 or 2 rows: an empty second part)
+    if (abytes) bulk_load(st, a.inv + a.blk_off[b] + (long)e0 * nc, abytes, bar);   // (a block of 1 or 2 rows: an empty part)
   } else {
     using S = TileStage<T>;
     const int t = item - A.nbi;
