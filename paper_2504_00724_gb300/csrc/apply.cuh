@@ -82,9 +82,9 @@ __device__ __noinline__ void apply_few(const ApplyArgs& A, const double* tile, c
 
 // out = L u + N g (TRANS: L^T v on the cells that no fitted row's stencil reaches, and N^T v).
 // star 4096^2, 4.9 M of 16.8 M cells active, 39 MB read and 134 MB written (26 us at the copy rate):
-// 71 us; without the look at the cells' sums 66 us (4 us of the difference its tests, which follow the
-// results, the rest the cells that fail them); with the classes loaded first and cell by cell, so that
-// a tile took two round trips and 10 loads a thread in place of 5, 85 us.
+// 68 to 71 us, by the values; without the look at the cells' sums 66 us (the quick test takes 1 us of
+// the difference, the cells that fail it the rest); with the classes loaded first and cell by cell, so
+// that a tile took two round trips and 10 loads a thread in place of 5, 85 us before that.
 template <bool CROSS, bool TRANS>
 __global__ void __launch_bounds__(256, 3) k_apply(const __grid_constant__ ApplyArgs A) {
   __shared__ __align__(16) double tile[HY * HX];

@@ -8,7 +8,7 @@
 // tolerance (or their iteration limit, or a non-finite residual, or a timed-out wait) by
 // clearing their IF condition, and clears the WHILE condition when no member is left.
 // k_group_init runs once before the loop on the initial residuals.  The decisions are the
-// ones the single-problem solve takes on the host, per member.
+// ones of the single-problem solve's loop (k_loop_decide), per member.
 #pragma once
 
 #include "kernels.cuh"
