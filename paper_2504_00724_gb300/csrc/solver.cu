@@ -2283,6 +2283,8 @@ int ccm_set_cycle_params(ccm_handle* h, double omega, int nu1, int nu2, int inne
     t->par.nu2 = nu2;
     t->par.inner_cycles = inner_cycles;
     t->par.cycle = cycle;
+    drop_kept(t);
+    t->info.device_bytes = t->arena.bytes;
     if (same) continue;
     if (w22 != 0) {
       t->S64.omega_d = omega / w22;
